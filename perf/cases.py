@@ -328,7 +328,7 @@ def work(case):
 
 def tolerance(case):
     # about four times the distances to exact() measured on a GB300: fp32 layers 4e-8 to 9e-8, 16-bit layers 1.7e-3
-    # (their bf16 outputs), attention 2.2e-3 in bf16 and 3e-4 in f16, K/V projections and norms 2e-4 to 3e-4
+    # (their bf16 outputs), attention 2.3e-3 in bf16 and 4e-4 in f16, K/V projections and norms 2e-4 to 3e-4
     kind, f32 = case["kind"], case["dtype"] == "f32"
     if kind == "pack":
         return "exact"
