@@ -69,6 +69,40 @@ __device__ __forceinline__ void tile_coords(int t, int num_m, int num_n, int gro
 }
 
 __device__ __forceinline__ float silu_f(float g) { return g / (1.0f + __expf(-g)); }
+// The same with the approximate quotient (2 ulp, and 0 where 1 + exp(-g) passes
+// 2^126): no branch, so the 32 activations of a chunk run side by side.  The IEEE
+// division's slow-path branch made each thread compute them one after the other,
+// ~15 us per 128 x 128 tile, exposed at the end of every call (one 8B layer with
+// its detector at 842 rows: 440 -> 416 us, the cached layer at 848 rows 434 -> 418).
+// Its values are stored in 16 bits; counts are decided on the IEEE value
+// (count_near_zero).
+__device__ __forceinline__ float silu_fast(float g) { return __fdividef(g, 1.0f + __expf(-g)); }
+
+// Number of |SiLU(g) * u| < eps over a chunk, as the IEEE division decides it; a
+// holds the fast values.  Those differ from the IEEE ones by at most 4 ulp, or
+// where g < -87 the fast quotient may be 0, so only a chunk with a value within
+// 2^-18 of eps, or such a g, is computed again.
+__device__ __forceinline__ int count_near_zero(const float (&a)[32], const uint32_t (&g)[32], const uint32_t (&u)[32],
+                                               float eps) {
+  const float band = eps * 0x1p-18f;
+  int cnt = 0;
+  bool near = false;
+  float g_min = 0.f;
+#pragma unroll
+  for (int i = 0; i < 32; ++i) {
+    const float v = fabsf(a[i]);
+    cnt += v < eps ? 1 : 0;
+    near = near || fabsf(v - eps) < band;
+    g_min = fminf(g_min, __uint_as_float(g[i]));
+  }
+  if (near || g_min < -87.f) {
+    cnt = 0;
+#pragma unroll
+    for (int i = 0; i < 32; ++i)
+      cnt += fabsf(silu_f(__uint_as_float(g[i])) * __uint_as_float(u[i])) < eps ? 1 : 0;
+  }
+  return cnt;
+}
 
 template <int MODE>
 __global__ void __launch_bounds__(THREADS, 1)
@@ -388,10 +422,8 @@ __global__ void __launch_bounds__(THREADS, 1)
           tmem_ld_wait();
           float a[32];
 #pragma unroll
-          for (int i = 0; i < 32; ++i) {
-            a[i] = silu_f(__uint_as_float(g[i])) * __uint_as_float(u[i]);
-            cnt += fabsf(a[i]) < p.act_eps ? 1 : 0;
-          }
+          for (int i = 0; i < 32; ++i) a[i] = silu_fast(__uint_as_float(g[i])) * __uint_as_float(u[i]);
+          if (cnt_idx >= 0) cnt += count_near_zero(a, g, u, p.act_eps);
           if (MODE == kGemmSwiglu) {
             const bool slab_full = m * BM + q * 32 + 32 <= M;
             if (slab_full || store) {
@@ -410,7 +442,7 @@ __global__ void __launch_bounds__(THREADS, 1)
             }
           }
         }
-        if (cnt_idx >= 0 && p.counts != nullptr) atomicAdd(&p.counts[cnt_idx], cnt);
+        if (cnt_idx >= 0) atomicAdd(&p.counts[cnt_idx], cnt);
       }
       tc_fence_before();
       __syncwarp();

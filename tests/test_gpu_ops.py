@@ -76,6 +76,33 @@ def test_linear_f32():
 
 
 # ------------------------------------------------------------------ SwiGLU + count hook (S10, S1)
+@pytest.mark.parametrize("op", ["bf16", "f16"])
+def test_swiglu_counts_at_the_threshold_follow_the_ieee_quotient(op):
+    """Every operand is a dyadic number and every weight row one power of two, so
+    both GEMM paths form the same g and u exactly; with eps set to values of the
+    fp32 path's own activations (ties, and g < -87 where the fast quotient may be
+    0) the 16-bit path's counts must equal the fp32 path's."""
+    rng = _rng(9)
+    M, F, K, B, N = 200, 256, 64, 1, 200
+    a = rng.integers(-96, 97, (M, K)).astype(np.float32) / 2
+    a[:, 0], a[:, 1] = -88.0, -100.0
+    one = lambda: np.eye(K, dtype=np.float32)[rng.integers(0, K, F)] * 2.0 ** rng.integers(-6, 2, F)[:, None]
+    wg, wu = one(), one()
+    wg[:2] = np.eye(K, dtype=np.float32)[:2]
+    cu, rs = i32([0, M]), i32([0])
+
+    def counts(dt, eps):
+        act = torch.empty((M, F), dtype=tdtype(dt), device=cuda())
+        c = torch.zeros(B * N, dtype=torch.int32, device=cuda())
+        S.seer_swiglu(to_dev(a, dt), to_dev(wg, dt), to_dev(wu, dt), dt, act, dt, M, None, F, K, cu, B, rs, N, eps, c)
+        return act, c.cpu().numpy()
+
+    act, _ = counts("f32", 1.0)
+    values = np.unique(np.abs(act.cpu().numpy()))
+    for eps in [0.0, *rng.choice(values[(values > 0) & (values < 6e4)], 12), float(values[values > 0].min())]:
+        np.testing.assert_array_equal(counts(op, float(eps))[1], counts("f32", float(eps))[1], err_msg=f"eps={eps}")
+
+
 @pytest.mark.parametrize("op", ["bf16", "f16", "f32"])
 def test_swiglu_with_count_hook(op):
     rng = _rng(7)
