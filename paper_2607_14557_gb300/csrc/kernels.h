@@ -37,7 +37,9 @@ struct GemmParams {
   uint32_t idesc;         // tcgen05 instruction descriptor (operand type f16 or bf16)
   int out_type;           // ElemType of C (kBF16 / kF16; kF32 on the CUDA-core path)
   int res_type;           // ElemType of R
-  int group_m;            // raster: m-tiles per group (see tc_gemm.cu)
+  int bn;                 // accumulator columns per tile (multiple of 32)
+  int stages;             // operand ring depth
+  int group_m;            // raster: row tiles per group (see tc_gemm.cu)
   float rope_theta;       // Rope: frequency base (> 0)
   int rope_cols;          // Rope: leading output columns that are rotated (the q|k columns)
 };
@@ -62,14 +64,23 @@ struct AttnParams {
 };
 
 // tcgen05 / TMA kernels (16-bit operands).  Tensor maps are encoded on the host.
-int tc_gemm_smem_bytes();
-// L2 raster of the persistent GEMM (GemmParams::group_m) for a B operand of
-// b_bytes and an A row-tile of a_tile_bytes.
-int tc_gemm_group_m(long b_bytes, long a_tile_bytes);
+// How one GEMM call is tiled: a tile is cg * 128 rows by bn accumulator columns,
+// computed by cg SMs together.
+struct GemmPlan {
+  int cg;        // SMs per tile: 1, or 2 (paired tensor-core tiles)
+  int bn;        // accumulator columns per tile (Swiglu / Count: bn / 2 of F)
+  int stages;    // operand ring depth
+  int group_m;   // raster: row tiles per group
+};
+// m_tiles: 128-row tiles; n_cols: accumulator columns (N; Swiglu / Count: 2 F);
+// K: depth; num_sms: SMs of the device.
+GemmPlan tc_gemm_plan(int mode, long m_tiles, long n_cols, int K, int num_sms);
 // mC: the 16-bit output C (Store, Residual, Rope) or act (Swiglu) with 32 x 32
-// boxes and no swizzle, for the epilogue's TMA stores (unused by Count).
-cudaError_t launch_tc_gemm(int mode, const CUtensorMap& mA, const CUtensorMap& mB0, const CUtensorMap& mB1,
-                           const CUtensorMap& mC, const GemmParams& p, int num_sms, cudaStream_t st);
+// boxes and no swizzle, for the epilogue's TMA stores (unused by Count).  mA
+// has boxes of 128 rows, mB0 and mB1 boxes of bn / 2 rows.
+cudaError_t launch_tc_gemm(int mode, const GemmPlan& plan, const CUtensorMap& mA, const CUtensorMap& mB0,
+                           const CUtensorMap& mB1, const CUtensorMap& mC, const GemmParams& p, int num_sms,
+                           cudaStream_t st);
 int tc_attn_smem_bytes();
 // grid: persistent CTAs (at most one per SM); they take the units of the
 // schedule from p.work_next until *p.work_count are done

@@ -270,14 +270,14 @@ seer_status do_linear(const void* a, const void* w, seer_dtype op_dt, const void
     if (!aligned16(a) || !aligned16(w) || !aligned16(c) || (r && !aligned16(r)))
       return fail(SEER_ERR_UNSUPPORTED, "16-bit linear needs 16-byte aligned pointers");
     if (M_cap == 0) return SEER_OK;
-    p.idesc = make_idesc(128, 256, 0, op_dt == SEER_F16);
-    p.group_m = tc_gemm_group_m(2l * N * K, 2l * 128 * K);
+    const GemmPlan plan = tc_gemm_plan(mode, (M_cap + 127l) / 128, N, K, di->num_sms);
+    p.idesc = make_idesc(128 * plan.cg, plan.bn, 0, op_dt == SEER_F16);
     CUtensorMap mA, mB, mC;
     SEER_TRY(make_map16(&mA, a, op_dt, M_cap, K, K, 128));
-    SEER_TRY(make_map16(&mB, w, op_dt, N, K, K, 128));
+    SEER_TRY(make_map16(&mB, w, op_dt, N, K, K, plan.bn / 2));
     SEER_TRY(make_map16(&mC, c, c_dt, M_cap, N, N, 32, 32, false));
     Phase ph(phase, st);
-    SEER_CUDA(launch_tc_gemm(mode, mA, mB, mB, mC, p, di->num_sms, st), "tc_gemm launch");
+    SEER_CUDA(launch_tc_gemm(mode, plan, mA, mB, mB, mC, p, di->num_sms, st), "tc_gemm launch");
   } else {
     if (c_dt != SEER_F32 || (r && r_dt != SEER_F32)) return fail(SEER_ERR_UNSUPPORTED, "fp32 linear needs fp32 output");
     if (M_cap == 0) return SEER_OK;
@@ -334,16 +334,17 @@ seer_status do_swiglu(const void* a, const void* wg, const void* wu, seer_dtype 
     SEER_CUDA(cudaMemsetAsync(counts, 0, sizeof(int32_t) * static_cast<size_t>(B) * N, st), "memset counts");
   if (M_cap == 0) return SEER_OK;
   if (is16(op_dt)) {
-    p.idesc = make_idesc(128, 256, 0, op_dt == SEER_F16);
-    p.group_m = tc_gemm_group_m(2l * 2 * F * K, 2l * 128 * K);
+    const long m_tiles = mode == kGemmCount ? static_cast<long>(B) * ((N + 127l) / 128) : (M_cap + 127l) / 128;
+    const GemmPlan plan = tc_gemm_plan(mode, m_tiles, 2l * F, K, di->num_sms);
+    p.idesc = make_idesc(128 * plan.cg, plan.bn, 0, op_dt == SEER_F16);
     CUtensorMap mA, mG, mU, mC;
     SEER_TRY(make_map16(&mA, a, op_dt, M_cap, K, K, 128));
-    SEER_TRY(make_map16(&mG, wg, op_dt, F, K, K, 128));
-    SEER_TRY(make_map16(&mU, wu, op_dt, F, K, K, 128));
+    SEER_TRY(make_map16(&mG, wg, op_dt, F, K, K, plan.bn / 2));
+    SEER_TRY(make_map16(&mU, wu, op_dt, F, K, K, plan.bn / 2));
     if (mode == kGemmSwiglu) SEER_TRY(make_map16(&mC, act, act_dt, M_cap, F, F, 32, 32, false));
     else mC = mA;                                  // Count stores nothing
     Phase ph(phase, st);
-    SEER_CUDA(launch_tc_gemm(mode, mA, mG, mU, mC, p, di->num_sms, st), "tc_gemm launch");
+    SEER_CUDA(launch_tc_gemm(mode, plan, mA, mG, mU, mC, p, di->num_sms, st), "tc_gemm launch");
   } else {
     Phase ph(phase, st);
     SEER_CUDA(launch_simt_gemm(mode, static_cast<const float*>(a), static_cast<const float*>(wg),

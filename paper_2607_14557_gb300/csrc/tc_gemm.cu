@@ -3,12 +3,22 @@
 // descriptor) and fp32 accumulation in tensor memory (TMEM); C and the
 // residual R are f16 or bf16 independently.
 //
-// One CTA per SM, 192 threads, warp-specialised:
-//   warp 0      TMA producer: 128x64 A tile + two 128x64 B tiles per stage
-//               (128-byte swizzle), 4-stage ring of 48 KB stages;
-//   warp 1      TMEM allocator + MMA issuer: 4 x tcgen05.mma (M=128, N=256,
-//               K=16) per stage into one of two 256-column fp32
-//               accumulators (double buffered, 512 columns);
+// A tile is 256 rows x bn columns computed by a pair of SMs (cta_group::2: each
+// CTA of a 2-CTA cluster stages its own 128 rows of A and half of B's rows, one
+// thread of the first CTA issues the MMAs for both, and each CTA's tensor memory
+// receives its own rows), or 128 x bn by one SM when there is a single row tile.
+// The pair reads a third less operand data per product than one-SM tiles of 128
+// x 256 (64 instead of 96 bytes per clock and SM at the tensor rate), which
+// leaves room for six stages instead of four; bn is chosen per call so that the
+// last wave of tiles is nearly full (tc_gemm_plan, with the measured times).
+//
+// One CTA per SM, 192 threads, warp-specialised, persistent over the tiles:
+//   warp 0      TMA producer: A and B tiles 64 deep (128-byte swizzle) into a
+//               192 KB ring; in a pair every byte is counted on the first
+//               CTA's barrier and a stage is released by a commit to both;
+//   warp 1      TMEM allocator + MMA issuer: 4 x tcgen05.mma (K = 16) per stage
+//               into one of two 256-column fp32 accumulators (double
+//               buffered, 512 columns);
 //               producer and issuer are whole warps in lockstep, one elected
 //               lane issuing;
 //   warps 2-5   epilogue: tcgen05.ld of the accumulator (each warp owns one
@@ -31,33 +41,38 @@
 // Every stored 16-bit value passes a range guard: an infinite or NaN result
 // (an f16 intermediate that overflowed +-65504) records kErrRange in the
 // device error word, which seer_check_device reports.
+#include <math.h>
+
 #include "common.cuh"
 #include "kernels.h"
 
 namespace seer {
 namespace {
 
-constexpr int BM = 128;
-constexpr int BN = 256;
+constexpr int BM = 128;                              // rows per CTA of a tile
 constexpr int BK = 64;
-constexpr int STAGES = 4;
 constexpr int A_TILE_BYTES = BM * BK * 2;            // 16 KB
-constexpr int B_HALF_BYTES = 128 * BK * 2;           // 16 KB
-constexpr int STAGE_BYTES = A_TILE_BYTES + 2 * B_HALF_BYTES;  // 48 KB
+constexpr int MAX_STAGES = 12;
 constexpr int THREADS = 192;
-constexpr int ACC_COLS = 256;
+constexpr int ACC_COLS = 256;                        // one of the two accumulators
 constexpr int TMEM_COLS = 512;
 constexpr int BAR_BYTES = 256;
 constexpr int ROPE_HEAD = 128;                       // head width of the Rope epilogue
 constexpr int ROPE_BYTES = ROPE_HEAD / 2 * 8;        // (hi, lo) inverse frequency per pair
 constexpr int EPI_CHUNK = 32 * 32 * 2;              // a warp's 32 rows x 32 columns, 16-bit
 constexpr int EPI_BYTES = 4 * 2 * EPI_CHUNK;         // 4 epilogue warps x 2 staging buffers
-constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + BAR_BYTES + ROPE_BYTES + EPI_BYTES + 1024;
+constexpr int FIXED_BYTES = BAR_BYTES + ROPE_BYTES + EPI_BYTES + 1024;
+constexpr int RING_BYTES = 196608;                   // operand ring: six stages of a 256-column pair tile
+static_assert(8 * (2 * MAX_STAGES + 4) + 8 <= BAR_BYTES, "barrier block");
+static_assert(RING_BYTES + FIXED_BYTES <= 232448, "shared memory per CTA");
 
-// Raster: groups of `group_m` m-tiles; inside a group m varies fastest and
+// Operand bytes one CTA stages per 64-deep k-block.
+__host__ __device__ constexpr int stage_bytes(int cg, int bn) { return A_TILE_BYTES + bn / cg * BK * 2; }
+
+// Raster: groups of `group_m` row tiles; inside a group m varies fastest and
 // the group sweeps every n-tile.  group_m = 1 keeps the whole B operand hot in
-// L2 while A streams once; a large group_m keeps a slab of A hot while B
-// streams once per group (chosen on the host from the operand sizes).
+// L2 while A streams once; a larger group_m keeps a slab of A hot while B
+// streams once per group (chosen in tc_gemm_plan).
 __device__ __forceinline__ void tile_coords(int t, int num_m, int num_n, int group_m, int& m, int& n) {
   const int per_group = group_m * num_n;
   const int g = t / per_group;
@@ -104,31 +119,36 @@ __device__ __forceinline__ int count_near_zero(const float (&a)[32], const uint3
   return cnt;
 }
 
-template <int MODE>
+template <int MODE, int CG>
 __global__ void __launch_bounds__(THREADS, 1)
     tc_gemm_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CUtensorMap mB0,
                    const __grid_constant__ CUtensorMap mB1, const __grid_constant__ CUtensorMap mC, const GemmParams p) {
   pdl_wait();
+  const int BN = p.bn;
+  const int stages = p.stages;
+  const int sbytes = stage_bytes(CG, BN);
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  uint64_t* full = reinterpret_cast<uint64_t*>(smem + STAGES * STAGE_BYTES);
-  uint64_t* empty = full + STAGES;
-  uint64_t* acc_full = empty + STAGES;
+  uint8_t* fixed = smem + stages * sbytes;
+  uint64_t* full = reinterpret_cast<uint64_t*>(fixed);
+  uint64_t* empty = full + MAX_STAGES;
+  uint64_t* acc_full = empty + MAX_STAGES;
   uint64_t* acc_empty = acc_full + 2;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + 2);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-  float2* rope_tab = reinterpret_cast<float2*>(smem + STAGES * STAGE_BYTES + BAR_BYTES);
-  uint8_t* epi_stage = smem + STAGES * STAGE_BYTES + BAR_BYTES + ROPE_BYTES;   // [4 warps][2][EPI_CHUNK]
+  float2* rope_tab = reinterpret_cast<float2*>(fixed + BAR_BYTES);
+  uint8_t* epi_stage = fixed + BAR_BYTES + ROPE_BYTES;   // [4 warps][2][EPI_CHUNK]
 
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
+  const uint32_t rank = CG == 2 ? cluster_ctarank() : 0u;   // CTA of the pair; rank 0 issues the MMAs
 
   // ---- problem size (device row counts are clamped, never trusted blindly)
   int M = p.M_cap;
-  int num_m, tiles_per_seq = 1;
+  int num_mt, tiles_per_seq = 1;                            // 128-row tiles, one per CTA of a tile
   if (MODE == kGemmCount) {
     tiles_per_seq = (p.Nw + BM - 1) / BM;
-    num_m = p.B * tiles_per_seq;
+    num_mt = p.B * tiles_per_seq;
   } else {
     if (p.M_dev != nullptr) {
       const int md = *p.M_dev;
@@ -139,29 +159,33 @@ __global__ void __launch_bounds__(THREADS, 1)
         M = md;
       }
     }
-    num_m = (M + BM - 1) / BM;
+    num_mt = (M + BM - 1) / BM;
   }
-  const bool halfN = (MODE == kGemmSwiglu || MODE == kGemmCount);
-  const int num_n = halfN ? p.N / 128 : p.N / BN;
+  constexpr bool halfN = (MODE == kGemmSwiglu || MODE == kGemmCount);
+  const int tile_n = halfN ? BN / 2 : BN;                   // columns of p.N covered by a tile
+  const int num_m = (num_mt + CG - 1) / CG;
+  const int num_n = (p.N + tile_n - 1) / tile_n;
   const int num_tiles = num_m * num_n;
   const int KB = p.K / BK;
   const int group_m = p.group_m > 0 ? p.group_m : 1;
+  const int t_first = blockIdx.x / CG, t_step = gridDim.x / CG;
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < STAGES; ++s) {
+    for (int s = 0; s < stages; ++s) {
       mbar_init(&full[s], 1);
       mbar_init(&empty[s], 1);
     }
     for (int a = 0; a < 2; ++a) {
       mbar_init(&acc_full[a], 1);
-      mbar_init(&acc_empty[a], 4);
+      mbar_init(&acc_empty[a], 4 * CG);                     // every epilogue warp of the tile's CTAs
     }
     *abort_flag = 0;
     fence_barrier_init();
   }
-  if (warp == 1) tmem_alloc(tmem_slot, TMEM_COLS);
+  if (warp == 1) tmem_alloc<CG>(tmem_slot, TMEM_COLS);
   tc_fence_before();
   __syncthreads();
+  if (CG == 2) cluster_sync();                              // the peer's barriers are initialised
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
 
@@ -171,52 +195,76 @@ __global__ void __launch_bounds__(THREADS, 1)
     // lanes, with a warp-uniform outcome); the elected lane issues the copies
     // and MMAs.  A lone lane in a divergent branch loses issue slots to the
     // FMA-heavy epilogue warp on its SM sub-partition.
+    // In a pair each CTA loads its own 128 rows of A and its half of B's rows
+    // and counts the bytes on rank 0's barrier, which expects both CTAs' bytes;
+    // each waits on its own `empty`, signalled in both by the MMAs' commit (by
+    // then rank 0's barrier has completed the stage's phase, so a peer's bytes
+    // can only reach the phase they belong to).
     const bool leader = elect_one();
     if (leader) {
       tma_prefetch_desc(&mA);
       tma_prefetch_desc(&mB0);
       tma_prefetch_desc(&mB1);
     }
+    const uint32_t full0 = CG == 2 ? cluster_addr(full, 0) : 0u;
+    const int half_b = BN / 2 * BK * 2;                     // bytes of one half of B's rows
     int s = 0;
     uint32_t ph = 0;
     long issued = 0;
-    for (int t = blockIdx.x; t < num_tiles && !__any_sync(0xffffffffu, *abort_flag != 0); t += gridDim.x) {
+    for (int t = t_first; t < num_tiles && !__any_sync(0xffffffffu, *abort_flag != 0); t += t_step) {
       int m, n;
       tile_coords(t, num_m, num_n, group_m, m, n);
+      const int mt = m * CG + static_cast<int>(rank);
       int a_row;
       if (MODE == kGemmCount) {
-        const int b = m / tiles_per_seq;
-        const int j = m - b * tiles_per_seq;
+        const int mv = min(mt, num_mt - 1);                 // a pair's second tile may not exist: any rows
+        const int b = mv / tiles_per_seq;
+        const int j = mv - b * tiles_per_seq;
         const int rs = p.resp_start[b];
         if (leader && (rs < 0 || rs + p.Nw > p.M_cap)) record_error(p.err, kErrLayout);
         a_row = rs + j * BM;
       } else {
-        a_row = m * BM;
+        a_row = mt * BM;
       }
-      const int b_row0 = halfN ? n * 128 : n * BN;
-      const int b_row1 = halfN ? n * 128 : n * BN + 128;
+      const int b_row0 = n * tile_n;
+      const int b_row1 = halfN ? n * tile_n : n * tile_n + BN / 2;
       bool ok = true;
       for (int kb = 0; kb < KB; ++kb) {
         if (!warp_wait(&empty[s], ph ^ 1u, abort_flag, p.err)) { ok = false; break; }
         if (leader) {
-          uint8_t* sa = smem + s * STAGE_BYTES;
-          mbar_arrive_expect_tx(&full[s], STAGE_BYTES);
-          tma_load_2d(sa, &mA, &full[s], kb * BK, a_row);
-          tma_load_2d(sa + A_TILE_BYTES, &mB0, &full[s], kb * BK, b_row0);
-          tma_load_2d(sa + A_TILE_BYTES + B_HALF_BYTES, &mB1, &full[s], kb * BK, b_row1);
+          uint8_t* sa = smem + s * sbytes;
+          if (CG == 1) {
+            mbar_arrive_expect_tx(&full[s], sbytes);
+            tma_load_2d(sa, &mA, &full[s], kb * BK, a_row);
+            tma_load_2d(sa + A_TILE_BYTES, &mB0, &full[s], kb * BK, b_row0);
+            tma_load_2d(sa + A_TILE_BYTES + half_b, &mB1, &full[s], kb * BK, b_row1);
+          } else {
+            if (rank == 0) mbar_arrive_expect_tx(&full[s], 2 * sbytes);
+            const uint32_t bar = full0 + static_cast<uint32_t>(s * sizeof(uint64_t));
+            tma_load_2d_pair(sa, &mA, bar, kb * BK, a_row);
+            if (rank == 0) tma_load_2d_pair(sa + A_TILE_BYTES, &mB0, bar, kb * BK, b_row0);
+            else tma_load_2d_pair(sa + A_TILE_BYTES, &mB1, bar, kb * BK, b_row1);
+          }
         }
         __syncwarp();
         ++issued;
-        if (++s == STAGES) { s = 0; ph ^= 1u; }
+        if (++s == stages) { s = 0; ph ^= 1u; }
       }
       if (!ok) break;
     }
-    if (*abort_flag && leader) {
-      // let copies still in flight land before the CTA's shared memory is released
-      const long first = issued > STAGES ? issued - STAGES : 0;
-      for (long i = first; i < issued; ++i)
-        mbar_wait_drain(&full[i % STAGES], static_cast<uint32_t>((i / STAGES) & 1), 200000000ull);
+    if (CG == 2) {
+      // wait until the MMAs have released every stage (their commits arrive here too)
+      for (int i = 0; i < stages && warp_wait(&empty[s], ph ^ 1u, abort_flag, p.err); ++i)
+        if (++s == stages) { s = 0; ph ^= 1u; }
     }
+    if (*abort_flag && leader && rank == 0) {
+      // let copies still in flight land before the shared memory is released
+      // (a pair's second CTA leaves only after this one, see the final barrier)
+      const long first = issued > stages ? issued - stages : 0;
+      for (long i = first; i < issued; ++i)
+        mbar_wait_drain(&full[i % stages], static_cast<uint32_t>((i / stages) & 1), 200000000ull);
+    }
+    if (CG == 2 && rank != 0 && leader) pdl_trigger();      // rank 0 triggers after its last MMAs
   } else if (warp == 1) {
     // ------------------------------------------------ MMA issuer
     const bool leader = elect_one();
@@ -225,7 +273,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     uint32_t ph = 0;
     int acc = 0;
     uint32_t acc_ph = 0;
-    for (int t = blockIdx.x; t < num_tiles; t += gridDim.x) {
+    for (int t = t_first; t < num_tiles && rank == 0; t += t_step) {
       if (!warp_wait(&acc_empty[acc], acc_ph ^ 1u, abort_flag, p.err)) break;
       tc_fence_after();
       const uint32_t d_tmem = tmem_base + static_cast<uint32_t>(acc * ACC_COLS);
@@ -234,25 +282,30 @@ __global__ void __launch_bounds__(THREADS, 1)
         if (!warp_wait(&full[s], ph, abort_flag, p.err)) { ok = false; break; }
         tc_fence_after();
         if (leader) {
-          const uint32_t sa = smem_u32(smem + s * STAGE_BYTES);
+          const uint32_t sa = smem_u32(smem + s * sbytes);
           const uint64_t adesc = make_sdesc_sw128(sa, 16, 1024);
           const uint64_t bdesc = make_sdesc_sw128(sa + A_TILE_BYTES, 16, 1024);
 #pragma unroll
           for (int k = 0; k < BK / 16; ++k) {
             // +32 bytes along K inside the 128-byte swizzle atom = +2 in the address field
-            tc_mma_f16(d_tmem, adesc + 2 * k, bdesc + 2 * k, idesc, (kb | k) != 0 ? 1u : 0u);
+            if (CG == 1) tc_mma_f16(d_tmem, adesc + 2 * k, bdesc + 2 * k, idesc, (kb | k) != 0 ? 1u : 0u);
+            else tc_mma_f16_pair(d_tmem, adesc + 2 * k, bdesc + 2 * k, idesc, (kb | k) != 0 ? 1u : 0u);
           }
-          tc_commit(&empty[s]);
+          if (CG == 1) tc_commit(&empty[s]);
+          else tc_commit_pair(&empty[s]);
         }
         __syncwarp();
-        if (++s == STAGES) { s = 0; ph ^= 1u; }
+        if (++s == stages) { s = 0; ph ^= 1u; }
       }
       if (!ok) break;
-      if (leader) tc_commit(&acc_full[acc]);
+      if (leader) {
+        if (CG == 1) tc_commit(&acc_full[acc]);
+        else tc_commit_pair(&acc_full[acc]);
+      }
       __syncwarp();
       if (++acc == 2) { acc = 0; acc_ph ^= 1u; }
     }
-    if (leader) pdl_trigger();                   // last MMAs issued: the next kernel may launch
+    if (leader && rank == 0) pdl_trigger();      // last MMAs issued: the next kernel may launch
   } else {
     // -------------------------------------------------- epilogue warps 2..5
     const int q = warp & 3;                    // TMEM lane quarter owned by this warp
@@ -288,19 +341,24 @@ __global__ void __launch_bounds__(THREADS, 1)
     int acc = 0;
     uint32_t acc_ph = 0;
     uint32_t nonfinite = 0;                      // range guard over this thread's stores
-    for (int t = blockIdx.x; t < num_tiles; t += gridDim.x) {
+    const uint32_t acc_empty0 = CG == 2 ? cluster_addr(acc_empty, 0) : 0u;
+    for (int t = t_first; t < num_tiles; t += t_step) {
       int m, n;
       tile_coords(t, num_m, num_n, group_m, m, n);
+      const int mt = m * CG + static_cast<int>(rank);          // this CTA's 128-row tile
+      // columns of this tile inside the matrix (the last tile may be narrower)
+      const int cols = min(tile_n, p.N - n * tile_n);
       // warp-uniform outcome: the TMEM loads below are warp-collective, and
       // after an abort the lanes of a warp could otherwise decide differently
       if (!__all_sync(0xffffffffu, mbar_wait(&acc_full[acc], acc_ph, abort_flag, p.err))) break;
       tc_fence_after();
       const uint32_t tacc = tmem_base + lane_off + static_cast<uint32_t>(acc * ACC_COLS);
       if (MODE == kGemmRope) {
-        // the tile holds two heads; pair (c, c + 64) of a head rotates by pos * f_c
-        const int row = m * BM + row_in_tile;
+        // the tile holds whole heads; pair (c, c + 64) of a head rotates by pos * f_c
+        const int row = mt * BM + row_in_tile;
         const bool valid = row < M;
-        const bool rotate = n * BN < p.rope_cols;       // tile-uniform (rope_cols % BN == 0)
+        const bool rotate = n * BN < p.rope_cols;       // tile-uniform (rope_cols % 256 == 0, BN 128 or 256)
+        const int heads = cols / ROPE_HEAD;
         const bool of16 = p.out_type == kF16;
         uint16_t* crow = reinterpret_cast<uint16_t*>(p.C) + static_cast<size_t>(valid ? row : 0) * p.ldc + n * BN;
         const float pos = (valid && rotate) ? static_cast<float>(row_position(p.cu, p.B, row)) : 0.f;
@@ -313,7 +371,7 @@ __global__ void __launch_bounds__(THREADS, 1)
             else { cs[e] = 1.f; sn[e] = 0.f; }
           }
 #pragma unroll 1
-          for (int hh = 0; hh < BN / ROPE_HEAD; ++hh) {
+          for (int hh = 0; hh < heads; ++hh) {
             const int c0 = hh * ROPE_HEAD + c * 32, c1 = c0 + ROPE_HEAD / 2;
             uint32_t r0[32], r1[32];
             tmem_ld32(tacc + c0, r0);
@@ -343,16 +401,16 @@ __global__ void __launch_bounds__(THREADS, 1)
           }
         }
       } else if (MODE == kGemmStore || MODE == kGemmResidual) {
-        const int row = m * BM + row_in_tile;
+        const int row = mt * BM + row_in_tile;
         const bool valid = row < M;
-        const bool slab_full = m * BM + q * 32 + 32 <= M;      // this warp's 32 rows all valid: TMA store
+        const bool slab_full = mt * BM + q * 32 + 32 <= M;     // this warp's 32 rows all valid: TMA store
         const bool of16 = p.out_type == kF16, rf16 = p.res_type == kF16;
         uint16_t* crow = reinterpret_cast<uint16_t*>(p.C) + static_cast<size_t>(valid ? row : 0) * p.ldc + n * BN;
         const uint16_t* rrow =
             MODE == kGemmResidual ? reinterpret_cast<const uint16_t*>(p.R) + static_cast<size_t>(valid ? row : 0) * p.ldr + n * BN
                                   : nullptr;
 #pragma unroll 1
-        for (int c = 0; c < BN / 32; ++c) {
+        for (int c = 0; c < cols / 32; ++c) {
           uint32_t r[32];
           tmem_ld32(tacc + c * 32, r);
           tmem_ld_wait();
@@ -378,7 +436,7 @@ __global__ void __launch_bounds__(THREADS, 1)
               nonfinite |= nonfinite_term(w[i], of16);
             }
             if (slab_full) {
-              store_chunk(w, n * BN + c * 32, m * BM + q * 32);
+              store_chunk(w, n * BN + c * 32, mt * BM + q * 32);
             } else {
               // a lane owns one row: 64 contiguous bytes as two full 32-byte sectors
               st_global_v8(crow + c * 32, w[0], w[1], w[2], w[3], w[4], w[5], w[6], w[7]);
@@ -387,16 +445,16 @@ __global__ void __launch_bounds__(THREADS, 1)
           }
         }
       } else {
-        // gate columns 0..127, up columns 128..255 of the accumulator
+        // gate columns 0 .. BN/2 - 1, up columns BN/2 .. BN - 1 of the accumulator
         int row, cnt_idx = -1;
         bool store = false;
         if (MODE == kGemmCount) {
-          const int b = m / tiles_per_seq;
-          const int tl = (m - b * tiles_per_seq) * BM + row_in_tile;
+          const int b = mt / tiles_per_seq;
+          const int tl = (mt - b * tiles_per_seq) * BM + row_in_tile;
           row = -1;
-          if (tl < p.Nw) cnt_idx = b * p.Nw + tl;
+          if (mt < num_mt && tl < p.Nw) cnt_idx = b * p.Nw + tl;
         } else {
-          row = m * BM + row_in_tile;
+          row = mt * BM + row_in_tile;
           store = row < M;
           if (store && p.counts != nullptr) {
             // segment of this row (binary search in cu), then its window offset
@@ -412,20 +470,20 @@ __global__ void __launch_bounds__(THREADS, 1)
         int cnt = 0;
         const bool of16 = p.out_type == kF16;
         uint16_t* arow =
-            MODE == kGemmSwiglu ? reinterpret_cast<uint16_t*>(p.C) + static_cast<size_t>(store ? row : 0) * p.ldc + n * 128
+            MODE == kGemmSwiglu ? reinterpret_cast<uint16_t*>(p.C) + static_cast<size_t>(store ? row : 0) * p.ldc + n * tile_n
                                 : nullptr;
 #pragma unroll 1
-        for (int c = 0; c < 4; ++c) {
+        for (int c = 0; c < cols / 32; ++c) {
           uint32_t g[32], u[32];
           tmem_ld32(tacc + c * 32, g);
-          tmem_ld32(tacc + 128 + c * 32, u);
+          tmem_ld32(tacc + BN / 2 + c * 32, u);
           tmem_ld_wait();
           float a[32];
 #pragma unroll
           for (int i = 0; i < 32; ++i) a[i] = silu_fast(__uint_as_float(g[i])) * __uint_as_float(u[i]);
           if (cnt_idx >= 0) cnt += count_near_zero(a, g, u, p.act_eps);
           if (MODE == kGemmSwiglu) {
-            const bool slab_full = m * BM + q * 32 + 32 <= M;
+            const bool slab_full = mt * BM + q * 32 + 32 <= M;
             if (slab_full || store) {
               uint32_t w[16];
 #pragma unroll
@@ -434,7 +492,7 @@ __global__ void __launch_bounds__(THREADS, 1)
                 nonfinite |= nonfinite_term(w[i], of16);
               }
               if (slab_full) {
-                store_chunk(w, n * 128 + c * 32, m * BM + q * 32);
+                store_chunk(w, n * tile_n + c * 32, mt * BM + q * 32);
               } else {
                 st_global_v8(arow + c * 32, w[0], w[1], w[2], w[3], w[4], w[5], w[6], w[7]);
                 st_global_v8(arow + c * 32 + 16, w[8], w[9], w[10], w[11], w[12], w[13], w[14], w[15]);
@@ -446,7 +504,10 @@ __global__ void __launch_bounds__(THREADS, 1)
       }
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(&acc_empty[acc]);
+      if (lane == 0) {
+        if (CG == 1) mbar_arrive(&acc_empty[acc]);
+        else mbar_arrive_cluster(acc_empty0 + static_cast<uint32_t>(acc * sizeof(uint64_t)));
+      }
       if (++acc == 2) { acc = 0; acc_ph ^= 1u; }
     }
     report_range(nonfinite, p.err);              // a stored value overflowed the 16-bit type (or was NaN)
@@ -456,25 +517,33 @@ __global__ void __launch_bounds__(THREADS, 1)
 
   tc_fence_before();
   __syncthreads();
+  // a pair leaves together: neither CTA's shared memory goes while the other's
+  // MMAs, copies or arrivals may still reach it
+  if (CG == 2) cluster_sync();
   if (warp == 1) {
     tc_fence_after();
-    tmem_dealloc(tmem_base, TMEM_COLS);
+    tmem_dealloc<CG>(tmem_base, TMEM_COLS);
   }
 }
 
-template <int MODE>
-cudaError_t launch_mode(const CUtensorMap& mA, const CUtensorMap& mB0, const CUtensorMap& mB1, const CUtensorMap& mC,
-                        const GemmParams& p, int num_sms, cudaStream_t st) {
+template <int MODE, int CG>
+cudaError_t launch_mode(const GemmPlan& plan, const CUtensorMap& mA, const CUtensorMap& mB0, const CUtensorMap& mB1,
+                        const CUtensorMap& mC, GemmParams p, int num_sms, cudaStream_t st) {
   static bool attr_set[64] = {};
-  cudaError_t e = set_smem_limit_once(tc_gemm_kernel<MODE>, SMEM_BYTES, attr_set);
+  cudaError_t e = set_smem_limit_once(tc_gemm_kernel<MODE, CG>, RING_BYTES + FIXED_BYTES, attr_set);
   if (e != cudaSuccess) return e;
-  long num_m;
-  if (MODE == kGemmCount) num_m = static_cast<long>(p.B) * ((p.Nw + BM - 1) / BM);
-  else num_m = (p.M_cap + BM - 1) / BM;
-  const long num_n = (MODE == kGemmSwiglu || MODE == kGemmCount) ? p.N / 128 : p.N / BN;
-  long tiles = num_m * num_n;
+  long num_mt;
+  if (MODE == kGemmCount) num_mt = static_cast<long>(p.B) * ((p.Nw + BM - 1) / BM);
+  else num_mt = (p.M_cap + BM - 1) / BM;
+  const int tile_n = (MODE == kGemmSwiglu || MODE == kGemmCount) ? plan.bn / 2 : plan.bn;
+  const long tiles = ((num_mt + CG - 1) / CG) * ((p.N + tile_n - 1) / tile_n);
   if (tiles <= 0) return cudaSuccess;
-  const int grid = static_cast<int>(tiles < num_sms ? tiles : num_sms);
+  p.bn = plan.bn;
+  p.stages = plan.stages;
+  p.group_m = plan.group_m;
+  const int units = num_sms / CG;
+  const int grid = static_cast<int>(tiles < units ? tiles : units);
+  const int smem = plan.stages * stage_bytes(CG, plan.bn) + FIXED_BYTES;
   // Overlapping the launch with the previous kernel pays off for short GEMMs,
   // where the launch gap is a visible share of the run.  Long GEMMs launched
   // that way measured 5-8% slower on GB300 (cause not isolated; their blocks
@@ -483,38 +552,75 @@ cudaError_t launch_mode(const CUtensorMap& mA, const CUtensorMap& mB0, const CUt
   constexpr long kOverlapMaxSteps = 320;     // k-blocks per CTA (about five 64-deep tiles)
   const long steps = (tiles * (p.K / BK) + grid - 1) / grid;
   const bool overlap = launch_overlap_enabled() && steps <= kOverlapMaxSteps;
-  return launch_kernel_overlap(overlap, tc_gemm_kernel<MODE>, dim3(grid), dim3(THREADS), SMEM_BYTES, st, mA, mB0, mB1,
-                               mC, p);
+  return launch_kernel_overlap(overlap, CG, tc_gemm_kernel<MODE, CG>, dim3(grid * CG), dim3(THREADS), smem, st, mA, mB0,
+                               mB1, mC, p);
+}
+
+template <int MODE>
+cudaError_t launch_cg(const GemmPlan& plan, const CUtensorMap& mA, const CUtensorMap& mB0, const CUtensorMap& mB1,
+                      const CUtensorMap& mC, const GemmParams& p, int num_sms, cudaStream_t st) {
+  return plan.cg == 2 ? launch_mode<MODE, 2>(plan, mA, mB0, mB1, mC, p, num_sms, st)
+                      : launch_mode<MODE, 1>(plan, mA, mB0, mB1, mC, p, num_sms, st);
 }
 
 }  // namespace
 
-int tc_gemm_smem_bytes() { return SMEM_BYTES; }
-
-// L2 raster of the tcgen05 GEMM: keep the whole weight operand resident when
-// it is at most 40 MB (group_m = 1, n varies fastest), otherwise keep about
-// 48 MB of 128-row slabs of A resident while the weights stream past them.
-// Both budgets come from sweeps on GB300 at the 8B layer shapes (35194 rows,
-// burst clocks, a cool-down before every point): the O projection (33.5 MB
-// of weights) is fastest with its weights resident; with 48 MB of slabs the
-// down projection (3 MB slabs, group 16) runs 1618 -> 1676 TFLOP/s and the
-// 4096-deep GEMMs (1 MB slabs, group 48) stay within 1% of 24 MB.
-int tc_gemm_group_m(long b_bytes, long a_tile_bytes) {
-  constexpr long kResident = 40l << 20;
-  constexpr long kBudget = 48l << 20;
-  if (b_bytes <= kResident) return 1;
-  const long g = kBudget / (a_tile_bytes > 0 ? a_tile_bytes : 1);
-  return static_cast<int>(g < 1 ? 1 : (g > 4096 ? 4096 : g));
+// Tile choice: the tile with the smallest modelled time, waves of tiles x
+// k-blocks x time of a k-block + the fixed part of a call (launch, first
+// operands, last epilogue).  The constants (us) are fits to GB300 timings of the
+// 8B layer's shapes at 127, 300, 842 and 2976 rows: per 64-deep k-block with all
+// SMs busy a pair takes 0.281 at 256 columns (the tensor rate), 0.264 at 224, 0.22
+// at 192, 0.19 at 160 and never below 0.18; one SM, which stages a third more
+// operand bytes per product, 0.366 / 0.35 / 0.29 / 0.22 at 256 / 224 / 192 / 128
+// columns (the SMs together read ~15 TB/s from L2) and never below 0.2.  So pairs
+// are the rule; one-SM tiles remain where a pair's second SM would idle (an odd,
+// small number of row tiles), and narrower tiles where they fill the last wave.
+// Examples (us, one-SM 256-column tiles -> chosen): 842 rows QKV 73.5 -> 57.7
+// (224 columns, 2.9 waves of pairs instead of 2.2 of SMs), O 30.8 -> 26.9 and
+// down 77.7 -> 60.7 (224: 76 tiles on 76 pairs); 127 rows QKV 30.7 -> 22.8 (96
+// columns), O 30.6 -> 17.3, down 75.7 -> 43; 2976 rows O 74.6 -> 63.0, down 238
+// -> 182; 35194 rows QKV 1990 -> 1927, down 2323 -> 2154.
+GemmPlan tc_gemm_plan(int mode, long m_tiles, long n_cols, int K, int num_sms) {
+  const bool half_n = mode == kGemmSwiglu || mode == kGemmCount;
+  // whole 32-column chunks of the output, and whole heads for Rope
+  const int step = mode == kGemmRope ? 128 : (half_n ? 64 : 32);
+  GemmPlan g{2, 256, 0, 1};
+  double best = 0.0;
+  for (int cg = 2; cg >= 1; --cg) {
+    for (int bn = 256; bn >= step; bn -= step) {
+      const long tiles = ((m_tiles + cg - 1) / cg) * ((n_cols + bn - 1) / bn);
+      const long units = num_sms / cg;
+      const double block = cg == 2 ? fmax(0.18, 0.03 + 0.001 * bn) : fmax(0.2, 0.08 + 0.00112 * bn);
+      const double fixed = cg == 2 ? 6.0 + 0.015 * bn : 4.2 + 0.0125 * bn;
+      const double cost = fixed + static_cast<double>((tiles + units - 1) / units) * (K / BK) * block;
+      if (g.stages == 0 || cost < 0.98 * best) {      // wide pair tiles unless another choice is clearly faster
+        best = cost;
+        g.cg = cg;
+        g.bn = bn;
+        g.stages = RING_BYTES / stage_bytes(cg, bn);
+      }
+    }
+  }
+  if (g.stages > MAX_STAGES) g.stages = MAX_STAGES;
+  // L2 raster: the 76 pair tiles in flight form a block of about 16 x 5, so each
+  // operand slab is shared by many SMs at once: 16 columns of tiles swept per row
+  // tile where the matrix has no more, else groups of 16 row tiles.  Swept on GB300
+  // (35194 rows, us): QKV 2137 / 1980 / 1934 / 1950 / 2134 at groups 1 / 8 / 16 / 24 /
+  // 48, gate/up 4487 / 3991 / 3822 / 3821 / 4180, O (16 columns of tiles) 661 / 675 /
+  // 674 / 682 / 743, down 2005 / 2039 / 2038 / 2073 / 2219.
+  g.group_m = (n_cols + g.bn - 1) / g.bn <= 16 ? 1 : 16;
+  return g;
 }
 
-cudaError_t launch_tc_gemm(int mode, const CUtensorMap& mA, const CUtensorMap& mB0, const CUtensorMap& mB1,
-                           const CUtensorMap& mC, const GemmParams& p, int num_sms, cudaStream_t st) {
+cudaError_t launch_tc_gemm(int mode, const GemmPlan& plan, const CUtensorMap& mA, const CUtensorMap& mB0,
+                           const CUtensorMap& mB1, const CUtensorMap& mC, const GemmParams& p, int num_sms,
+                           cudaStream_t st) {
   switch (mode) {
-    case kGemmStore: return launch_mode<kGemmStore>(mA, mB0, mB1, mC, p, num_sms, st);
-    case kGemmResidual: return launch_mode<kGemmResidual>(mA, mB0, mB1, mC, p, num_sms, st);
-    case kGemmSwiglu: return launch_mode<kGemmSwiglu>(mA, mB0, mB1, mC, p, num_sms, st);
-    case kGemmCount: return launch_mode<kGemmCount>(mA, mB0, mB1, mC, p, num_sms, st);
-    case kGemmRope: return launch_mode<kGemmRope>(mA, mB0, mB1, mC, p, num_sms, st);
+    case kGemmStore: return launch_cg<kGemmStore>(plan, mA, mB0, mB1, mC, p, num_sms, st);
+    case kGemmResidual: return launch_cg<kGemmResidual>(plan, mA, mB0, mB1, mC, p, num_sms, st);
+    case kGemmSwiglu: return launch_cg<kGemmSwiglu>(plan, mA, mB0, mB1, mC, p, num_sms, st);
+    case kGemmCount: return launch_cg<kGemmCount>(plan, mA, mB0, mB1, mC, p, num_sms, st);
+    case kGemmRope: return launch_cg<kGemmRope>(plan, mA, mB0, mB1, mC, p, num_sms, st);
     default: return cudaErrorInvalidValue;
   }
 }

@@ -75,6 +75,40 @@ def test_linear_f32():
     check_close(host(c), a.astype(np.float64) @ w.astype(np.float64).T + r, "f32", "linear f32")
 
 
+@pytest.mark.parametrize("M,N,K", [
+    (1, 256, 64), (127, 4096, 128), (128, 256, 4096),              # one row tile: one SM per tile, narrow tiles
+    (129, 256, 192), (255, 2304, 128), (257, 512, 64),             # pairs; a last pair with one row tile
+    (700, 4096, 256), (1100, 12288, 64), (842, 4096, 4096),        # last column tile narrower than the others
+    (2600, 4096, 128), (4500, 2304, 64)])                          # several waves, both raster orders
+@pytest.mark.parametrize("res", [False, True])
+def test_linear_tile_choices(M, N, K, res):
+    """Every tile shape the GEMM's plan picks (one SM or a pair, 32 .. 256 columns):
+    small integers, so every product and sum is exact in fp32 (|sum| <= 4 K < 2^24)
+    and the result is the fp64 one rounded once to bf16."""
+    rng = _rng(M + N + K)
+    a, w = rng.integers(-2, 3, (M, K)).astype(np.float32), rng.integers(-2, 3, (N, K)).astype(np.float32)
+    r = rng.integers(-8, 9, (M, N)).astype(np.float32)
+    ad, wd, rd = to_dev(a, "f16"), to_dev(w, "f16"), to_dev(r, "f16")
+    c = torch.full((M + 1, N), float("nan"), dtype=torch.bfloat16, device=cuda())
+    S.seer_linear(ad, wd, "f16", rd if res else None, "f16", c, "bf16", M, None, N, K)
+    ref = ad.double() @ wd.double().T + (rd.double() if res else 0.0)
+    assert torch.equal(c[:M], ref.to(torch.bfloat16))
+    assert torch.isnan(c[M]).all()                                  # nothing past the last row
+
+
+@pytest.mark.parametrize("M,F,K", [(1, 128, 64), (127, 1280, 64), (200, 384, 128), (300, 12288, 64), (900, 1408, 64)])
+def test_swiglu_tile_choices(M, F, K):
+    """Gate/up tiles of every width, the last one narrower than the others."""
+    rng = _rng(M + F + K)
+    a = _store(rng.standard_normal((M, K)), "f16")
+    wg, wu = (_store(0.2 * rng.standard_normal((F, K)), "f16") for _ in range(2))
+    act = torch.full((M + 1, F), float("nan"), dtype=torch.float16, device=cuda())
+    S.seer_swiglu(to_dev(a, "f16"), to_dev(wg, "f16"), to_dev(wu, "f16"), "f16", act, "f16", M, None, F, K)
+    g, u = (a.astype(np.float64) @ w.astype(np.float64).T for w in (wg, wu))
+    check_close(host(act[:M]), g / (1.0 + np.exp(-g)) * u, "bf16", "swiglu")
+    assert torch.isnan(act[M]).all()
+
+
 # ------------------------------------------------------------------ SwiGLU + count hook (S10, S1)
 @pytest.mark.parametrize("op", ["bf16", "f16"])
 def test_swiglu_counts_at_the_threshold_follow_the_ieee_quotient(op):
