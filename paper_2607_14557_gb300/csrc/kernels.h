@@ -98,8 +98,8 @@ cudaError_t launch_attn_schedule(const int* cu, const int* cu_kv, const int* kv_
 
 // CUDA-core kernels (fp32 storage; small shapes).
 cudaError_t launch_simt_gemm(int mode, const float* A, const float* B0, const float* B1, const GemmParams& p,
-                             cudaStream_t st);
-cudaError_t launch_simt_attn(const float* qkv, const AttnParams& p, cudaStream_t st);
+                             int num_sms, cudaStream_t st);
+cudaError_t launch_simt_attn(const float* qkv, const AttnParams& p, int num_sms, cudaStream_t st);
 
 // Element-wise / scan kernels (both storage types).
 cudaError_t launch_rmsnorm(const void* x, int in_type, const void* g, void* y, int out_type, int M_cap,

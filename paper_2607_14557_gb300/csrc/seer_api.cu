@@ -283,7 +283,7 @@ seer_status do_linear(const void* a, const void* w, seer_dtype op_dt, const void
     if (M_cap == 0) return SEER_OK;
     Phase ph(phase, st);
     SEER_CUDA(launch_simt_gemm(rot ? kGemmStore : mode, static_cast<const float*>(a), static_cast<const float*>(w),
-                               nullptr, p, st),
+                               nullptr, p, di->num_sms, st),
               "simt_gemm launch");
     if (rot)
       SEER_CUDA(launch_rope(c, kF32, rope.cu, rope.B, M_cap, rope.n_heads, rope.head_dim, rope.theta, di->err,
@@ -348,7 +348,7 @@ seer_status do_swiglu(const void* a, const void* wg, const void* wu, seer_dtype 
   } else {
     Phase ph(phase, st);
     SEER_CUDA(launch_simt_gemm(mode, static_cast<const float*>(a), static_cast<const float*>(wg),
-                               static_cast<const float*>(wu), p, st),
+                               static_cast<const float*>(wu), p, di->num_sms, st),
               "simt_gemm launch");
   }
   return SEER_OK;
@@ -437,7 +437,7 @@ seer_status do_attention(const void* qkv, void* o, seer_dtype dt, const int32_t*
     if (dh > 128 || dh % 4 != 0) return fail(SEER_ERR_UNSUPPORTED, "fp32 attention needs head_dim <= 128, %% 4 == 0");
     if (T_cap == 0) return SEER_OK;
     Phase ph(PH_ATTN, st);
-    SEER_CUDA(launch_simt_attn(static_cast<const float*>(qkv), p, st), "simt_attn launch");
+    SEER_CUDA(launch_simt_attn(static_cast<const float*>(qkv), p, di->num_sms, st), "simt_attn launch");
   }
   return SEER_OK;
 }

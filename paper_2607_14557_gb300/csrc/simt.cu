@@ -10,27 +10,64 @@
 namespace seer {
 namespace {
 
-constexpr int TB = 64;   // output tile (rows and columns)
-constexpr int TK = 32;
-constexpr int LPT = TB * TK / 256;   // elements of each operand tile a thread loads per k-step
-
 __device__ __forceinline__ float silu_f(float g) { return g / (1.0f + __expf(-g)); }
 
-// C tile 64x64, 256 threads, 4x4 outputs per thread.  For Swiglu/Count the
-// block computes matching gate and up tiles of the same F columns.
-template <int MODE>
-__global__ void __launch_bounds__(256) simt_gemm_kernel(const float* __restrict__ A, const float* __restrict__ B0,
-                                                        const float* __restrict__ B1, const GemmParams p) {
+// Asynchronous copy of VEC floats (16 or 4 bytes) to shared memory; the rest of a
+// copy past `valid` is filled with zeros (nothing is read when !valid).
+template <int VEC>
+__device__ __forceinline__ void cp_async(float* dst, const float* src, bool valid) {
+  if (VEC == 4)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(valid ? 16 : 0)
+                 : "memory");
+  else
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(valid ? 4 : 0)
+                 : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+// Floats per staged row of TK: an odd number of 16-byte words, so 16-byte reads
+// of 8 rows meet no bank twice.
+__host__ __device__ constexpr int staged_ld(int tk) { return tk + 4; }
+
+// acc.x += a0 * b0, acc.y += a1 * b1 (packed fp32 multiply-add, sm_100+).
+__device__ __forceinline__ void ffma2(float2& acc, float a0, float a1, float b0, float b1) {
+  asm("{\n\t.reg .b64 ra, rb, rc;\n\t"
+      "mov.b64 ra, {%2, %3};\n\t"
+      "mov.b64 rb, {%4, %5};\n\t"
+      "mov.b64 rc, {%0, %1};\n\t"
+      "fma.rn.f32x2 rc, ra, rb, rc;\n\t"
+      "mov.b64 {%0, %1}, rc;\n\t}"
+      : "+f"(acc.x), "+f"(acc.y) : "f"(a0), "f"(a1), "f"(b0), "f"(b1));
+}
+
+// C tile BM x BN per block, TM x TN outputs per thread (rows ty + i * TY, columns
+// tx + j * TX).  Both operands stay row-major in shared memory (k contiguous) and
+// a thread reads four k of a row with one 16-byte load, so four k cost TM + TN
+// loads for 4 TM TN multiply-adds; STAGES k-steps are in flight by cp.async.  The
+// multiply-adds are packed pairs: an output is the sum of its even-k and its odd-k
+// chain; the detector's (Count) is one chain over ascending k.
+// For Swiglu / Count the block holds BN / 2 gate columns and the matching up
+// columns, and a thread's first TN / 2 columns are gates.
+// Bound by instruction issue beside the FMA pipes (44 TFLOP/s of 80 at the largest
+// shape; scalar multiply-adds 41) and, for few rows, by the latency of the k-steps.
+template <int MODE, int BM, int BN, int TM, int TN, int TK, int STAGES, int MIN_BLOCKS, int VEC>
+__global__ void __launch_bounds__((BM / TM) * (BN / TN), MIN_BLOCKS)
+    simt_gemm_kernel(const float* __restrict__ A, const float* __restrict__ B0, const float* __restrict__ B1,
+                     const GemmParams p) {
   pdl_enter();
-  __shared__ float As[TK][TB + 1];
-  __shared__ float Bs0[TK][TB + 1];
-  __shared__ float Bs1[TK][TB + 1];
+  constexpr int TX = BN / TN, TY = BM / TM, NTHR = TX * TY, LDT = staged_ld(TK);
+  constexpr bool PAIR = MODE != kGemmCount;
   constexpr bool TWO = (MODE == kGemmSwiglu || MODE == kGemmCount);
+  constexpr int COLS = TWO ? BN / 2 : BN;            // columns of p.N per block
+  extern __shared__ float4 simt_smem[];
+  float* sm = reinterpret_cast<float*>(simt_smem);   // [STAGES][BM + BN][LDT]
 
   int M = p.M_cap;
   int tiles_per_seq = 1;
   if (MODE == kGemmCount) {
-    tiles_per_seq = (p.Nw + TB - 1) / TB;
+    tiles_per_seq = (p.Nw + BM - 1) / BM;
   } else if (p.M_dev != nullptr) {
     const int md = *p.M_dev;
     if (md < 0 || md > p.M_cap) {
@@ -51,221 +88,406 @@ __global__ void __launch_bounds__(256) simt_gemm_kernel(const float* __restrict_
       if (threadIdx.x == 0) record_error(p.err, kErrLayout);
       return;
     }
-    row_base = rs + j * TB;
-    rows_here = min(TB, p.Nw - j * TB);
+    row_base = rs + j * BM;
+    rows_here = min(BM, p.Nw - j * BM);
   } else {
-    row_base = mt * TB;
+    row_base = mt * BM;
     if (row_base >= M) return;
-    rows_here = min(TB, M - row_base);
+    rows_here = min(BM, M - row_base);
   }
-  const int col_base = nt * TB;
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  float acc0[4][4] = {}, acc1[4][4] = {};
+  const int col_base = nt * COLS;
+  const int tx = threadIdx.x % TX, ty = threadIdx.x / TX;
 
-  // the next k-step's operands are loaded into registers while the current
-  // one is multiplied out of shared memory
-  float ra[LPT], rb0[LPT], rb1[LPT];
-  auto load = [&](int k0) {
-#pragma unroll
-    for (int e = 0; e < LPT; ++e) {
-      const int i = threadIdx.x + 256 * e;
-      const int r = i / TK, kk = k0 + i % TK;
-      ra[e] = (r < rows_here && kk < p.K) ? A[static_cast<size_t>(row_base + r) * p.K + kk] : 0.f;
-      const int c = col_base + r;
-      rb0[e] = (c < p.N && kk < p.K) ? B0[static_cast<size_t>(c) * p.K + kk] : 0.f;
-      if (TWO) rb1[e] = (c < p.N && kk < p.K) ? B1[static_cast<size_t>(c) * p.K + kk] : 0.f;
-    }
-  };
-  load(0);
-  for (int k0 = 0; k0 < p.K; k0 += TK) {
-#pragma unroll
-    for (int e = 0; e < LPT; ++e) {
-      const int i = threadIdx.x + 256 * e;
-      const int r = i / TK, k = i % TK;
-      As[k][r] = ra[e];
-      Bs0[k][r] = rb0[e];
-      if (TWO) Bs1[k][r] = rb1[e];
-    }
-    __syncthreads();
-    if (k0 + TK < p.K) load(k0 + TK);
-#pragma unroll
-    for (int k = 0; k < TK; ++k) {
-      float a[4], b0[4], b1[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        a[i] = As[k][ty * 4 + i];
-        b0[i] = Bs0[k][tx * 4 + i];
-        if (TWO) b1[i] = Bs1[k][tx * 4 + i];
+  // stage k0 .. k0 + TK - 1 of both operands (zeros past the rows, columns and K)
+  auto load = [&](int stage, int k0) {
+    float* dst = sm + stage * (BM + BN) * LDT;
+    constexpr int PER_ROW = TK / VEC;
+#pragma unroll 4
+    for (int i = threadIdx.x; i < (BM + BN) * PER_ROW; i += NTHR) {
+      const int r = i / PER_ROW, kk = (i % PER_ROW) * VEC;
+      const bool kin = k0 + kk < p.K;                // K % VEC == 0
+      const float* src = A;
+      bool valid = false;
+      if (r < BM) {
+        valid = kin && r < rows_here;
+        if (valid) src = A + static_cast<size_t>(row_base + r) * p.K + k0 + kk;
+      } else {
+        const int c = r - BM;
+        const int col = col_base + (TWO && c >= COLS ? c - COLS : c);
+        valid = kin && col < p.N;
+        const float* w = TWO && c >= COLS ? B1 : B0;
+        if (valid) src = w + static_cast<size_t>(col) * p.K + k0 + kk;
       }
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int jj = 0; jj < 4; ++jj) {
-          acc0[i][jj] = fmaf(a[i], b0[jj], acc0[i][jj]);
-          if (TWO) acc1[i][jj] = fmaf(a[i], b1[jj], acc1[i][jj]);
-        }
+      cp_async<VEC>(dst + r * LDT + kk, src, valid);
     }
-    __syncthreads();
+    cp_async_commit();
+  };
+
+  float2 acc[TM][TN] = {};
+  const int steps = (p.K + TK - 1) / TK;
+#pragma unroll
+  for (int s = 0; s < STAGES - 1; ++s) {
+    if (s < steps) load(s, s * TK);
+    else cp_async_commit();
+  }
+  for (int s = 0; s < steps; ++s) {
+    cp_async_wait<STAGES - 2>();
+    __syncthreads();                                 // step s landed; the stage filled next is read out
+    if (s + STAGES - 1 < steps) load((s + STAGES - 1) % STAGES, (s + STAGES - 1) * TK);
+    else cp_async_commit();
+    const float* As = sm + (s % STAGES) * (BM + BN) * LDT;
+    const float* Bs = As + BM * LDT;
+#pragma unroll
+    for (int k = 0; k < TK; k += 4) {
+      float4 b[TN];
+#pragma unroll
+      for (int j = 0; j < TN; ++j) b[j] = *reinterpret_cast<const float4*>(Bs + (tx + j * TX) * LDT + k);
+#pragma unroll
+      for (int i = 0; i < TM; ++i) {
+        const float4 a = *reinterpret_cast<const float4*>(As + (ty + i * TY) * LDT + k);
+#pragma unroll
+        for (int j = 0; j < TN; ++j) {
+          if (PAIR) {
+            ffma2(acc[i][j], a.x, a.y, b[j].x, b[j].y);
+            ffma2(acc[i][j], a.z, a.w, b[j].z, b[j].w);
+          } else {
+            acc[i][j].x = fmaf(a.x, b[j].x, acc[i][j].x);
+            acc[i][j].x = fmaf(a.y, b[j].y, acc[i][j].x);
+            acc[i][j].x = fmaf(a.z, b[j].z, acc[i][j].x);
+            acc[i][j].x = fmaf(a.w, b[j].w, acc[i][j].x);
+          }
+        }
+      }
+    }
   }
 
   float* C = reinterpret_cast<float*>(p.C);
   const float* R = reinterpret_cast<const float*>(p.R);
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int lr = ty * 4 + i;
-    if (lr >= rows_here) continue;
+  for (int i = 0; i < TM; ++i) {
+    const int lr = ty + i * TY;
+    const bool in = lr < rows_here;
     const int row = row_base + lr;
     int cnt = 0;
+    if (in) {
 #pragma unroll
-    for (int jj = 0; jj < 4; ++jj) {
-      const int col = col_base + tx * 4 + jj;
-      if (col >= p.N) continue;
-      if (MODE == kGemmStore) {
-        C[static_cast<size_t>(row) * p.ldc + col] = acc0[i][jj];
-      } else if (MODE == kGemmResidual) {
-        C[static_cast<size_t>(row) * p.ldc + col] = acc0[i][jj] + R[static_cast<size_t>(row) * p.ldr + col];
-      } else {
-        const float a = silu_f(acc0[i][jj]) * acc1[i][jj];
-        cnt += fabsf(a) < p.act_eps ? 1 : 0;
-        if (MODE == kGemmSwiglu) C[static_cast<size_t>(row) * p.ldc + col] = a;
+      for (int j = 0; j < (TWO ? TN / 2 : TN); ++j) {
+        const int col = col_base + tx + j * TX;
+        if (col >= p.N) continue;
+        const float v0 = PAIR ? acc[i][j].x + acc[i][j].y : acc[i][j].x;
+        if (MODE == kGemmStore) {
+          C[static_cast<size_t>(row) * p.ldc + col] = v0;
+        } else if (MODE == kGemmResidual) {
+          C[static_cast<size_t>(row) * p.ldc + col] = v0 + R[static_cast<size_t>(row) * p.ldr + col];
+        } else {
+          const float2 u = acc[i][TWO ? j + TN / 2 : j];
+          const float v = silu_f(v0) * (PAIR ? u.x + u.y : u.x);
+          cnt += fabsf(v) < p.act_eps ? 1 : 0;
+          if (MODE == kGemmSwiglu) C[static_cast<size_t>(row) * p.ldc + col] = v;
+        }
       }
     }
-    if (TWO && p.counts != nullptr && cnt > 0) {
-      int idx = -1;
-      if (MODE == kGemmCount) {
-        idx = seq * p.Nw + (mt - seq * tiles_per_seq) * TB + lr;
-      } else {
-        int lo = 0, hi = p.B;
-        while (hi - lo > 1) {
-          const int mid = (lo + hi) >> 1;
-          if (p.cu[mid] <= row) lo = mid; else hi = mid;
+    if (TWO && p.counts != nullptr) {
+      // a row's TX threads are consecutive lanes: one atomic per row and block
+#pragma unroll
+      for (int off = TX / 2; off > 0; off >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, off);
+      if (in && tx == 0 && cnt > 0) {
+        int idx = -1;
+        if (MODE == kGemmCount) {
+          idx = seq * p.Nw + (mt - seq * tiles_per_seq) * BM + lr;
+        } else {
+          int lo = 0, hi = p.B;
+          while (hi - lo > 1) {
+            const int mid = (lo + hi) >> 1;
+            if (p.cu[mid] <= row) lo = mid; else hi = mid;
+          }
+          const int tl = row - p.resp_start[lo];
+          if (tl >= 0 && tl < p.Nw && row < p.cu[lo + 1]) idx = lo * p.Nw + tl;
         }
-        const int tl = row - p.resp_start[lo];
-        if (tl >= 0 && tl < p.Nw && row < p.cu[lo + 1]) idx = lo * p.Nw + tl;
+        if (idx >= 0) atomicAdd(&p.counts[idx], cnt);
       }
-      if (idx >= 0) atomicAdd(&p.counts[idx], cnt);
     }
   }
 }
 
-// One warp per (query row, head): lanes split the head dimension, keys are
-// visited in order with an online softmax (fp32).
-__global__ void __launch_bounds__(256) simt_attn_kernel(const float* __restrict__ qkv, const AttnParams p) {
+// Attention of BQ query rows of one segment and head per block (16 x TY threads),
+// keys in tiles of 64 with an online softmax (fp32, expf).
+// Scores: a thread holds BQ / TY rows (ty + TY i) x 4 keys (tx + 16 j), Q and K
+// row-major in shared memory and read four dims at a time; a row's 16 threads are
+// consecutive lanes, so its max and sum are shuffles; the probabilities go
+// through shared memory and a thread accumulates its rows x the output columns
+// 4 tx .. 4 tx + 3 (and + 64).  The next K tile is copied by cp.async while the
+// current tile's softmax and PV run, the next V tile while the next scores do.
+// Bound by instruction issue beside the FMA pipes and shared-memory reads.  A warp
+// per (row, head) that reads every key itself took 1209 us for the 8-segment
+// batch of 58 .. 794 rows, 8 heads of 64; this kernel 146.
+constexpr int AKV = 64;                      // keys per tile
+constexpr int APS = AKV + 16;                // floats per row of probabilities (two rows meet no bank twice)
+
+__host__ __device__ constexpr int attn_ld(int dh) { return 4 * ((dh / 4) | 1); }   // an odd number of 16-byte words
+
+template <int BQ, int TY, int VEC>
+__global__ void __launch_bounds__(16 * TY) simt_attn_kernel(const float* __restrict__ qkv, const AttnParams p) {
   pdl_enter();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const long task = static_cast<long>(blockIdx.x) * 8 + warp;
+  constexpr int TM = BQ / TY;
   const int H = p.n_heads, dh = p.head_dim, D = H * dh;
   const int total = p.cu[p.B];
   if (total < 0 || total > p.T_cap) {
-    if (task == 0 && lane == 0) record_error(p.err, kErrRows);
+    if (blockIdx.x == 0 && threadIdx.x == 0) record_error(p.err, kErrRows);
     return;
   }
-  if (task >= static_cast<long>(total) * H) return;
-  const int row = static_cast<int>(task / H), h = static_cast<int>(task % H);
+  // slot -> (segment, query tile): the slots of segment b start at cu[b] / BQ + b,
+  // at least as far apart as its tiles
+  const int slot = blockIdx.x / H, h = blockIdx.x % H;
   int lo = 0, hi = p.B;
   while (hi - lo > 1) {
     const int mid = (lo + hi) >> 1;
-    if (p.cu[mid] <= row) lo = mid; else hi = mid;
+    if (p.cu[mid] / BQ + mid <= slot) lo = mid; else hi = mid;
   }
-  const int seq0 = p.cu[lo];
+  const int seq0 = p.cu[lo], L = p.cu[lo + 1] - seq0;
+  const int q0 = (slot - (seq0 / BQ + lo)) * BQ;
+  if (q0 < 0 || q0 >= L) return;
   const int kv0 = p.cu_kv ? p.cu_kv[lo] : seq0;
-  const int Lkv = p.cu_kv ? p.cu_kv[lo + 1] - kv0 : p.cu[lo + 1] - seq0;
+  const int Lkv = p.cu_kv ? p.cu_kv[lo + 1] - kv0 : L;
   const int kvL = p.kv_len ? p.kv_len[lo] : Lkv;
   if (kvL <= 0 || kvL > Lkv) {
-    if (lane == 0) record_error(p.err, kErrLayout);
+    if (threadIdx.x == 0) record_error(p.err, kErrLayout);
     return;
   }
-  const float* kvsrc = p.kv ? static_cast<const float*>(p.kv) : qkv;
-  const int per = (dh + 31) / 32;   // <= 4
-  float q[4], o[4];
-  const float* qrow = qkv + static_cast<size_t>(row) * 3 * D + h * dh;
-  for (int i = 0; i < 4; ++i) {
-    const int c = lane + 32 * i;
-    q[i] = (i < per && c < dh) ? qrow[c] : 0.f;
-    o[i] = 0.f;
+  const int rows = min(BQ, L - q0);
+  const int ld = attn_ld(dh);
+  extern __shared__ float4 simt_smem[];
+  float* Qs = reinterpret_cast<float*>(simt_smem);   // [BQ][ld]
+  float* Ks = Qs + BQ * ld;                           // [AKV][ld]
+  float* Vs = Ks + AKV * ld;                          // [AKV][ld]
+  float* Ps = Vs + AKV * ld;                          // [BQ][APS]
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  const int per_row = dh / VEC;
+
+  for (int i = threadIdx.x; i < BQ * per_row; i += 16 * TY) {
+    const int r = i / per_row, c = (i - r * per_row) * VEC;
+    const bool valid = r < rows;
+    cp_async<VEC>(Qs + r * ld + c, qkv + static_cast<size_t>(seq0 + q0 + (valid ? r : 0)) * 3 * D + h * dh + c, valid);
   }
+  const float* kvsrc = p.kv ? static_cast<const float*>(p.kv) : qkv;
+  auto load_keys = [&](float* dst, int column, int k0) {   // one K or V tile, zeros past the valid keys
+    for (int i = threadIdx.x; i < AKV * per_row; i += 16 * TY) {
+      const int r = i / per_row, c = (i - r * per_row) * VEC;
+      const bool valid = k0 + r < kvL;
+      cp_async<VEC>(dst + r * ld + c, kvsrc + static_cast<size_t>(kv0 + (valid ? k0 + r : 0)) * p.ld_kv + column + h * dh + c,
+                    valid);
+    }
+    cp_async_commit();
+  };
+  load_keys(Ks, p.xk0, 0);                            // Q is part of this group
+  load_keys(Vs, p.xv0, 0);
+
   const float scale = 1.0f / sqrtf(static_cast<float>(dh));
-  float m = -INFINITY, l = 0.f;
-  // keys in chunks of KC: the chunk's loads are all in flight together and its
-  // KC warp reductions are independent, then one online-softmax update
-  constexpr int KC = 8;
-  for (int k0 = 0; k0 < kvL; k0 += KC) {
-    float kv_k[KC][4], kv_v[KC][4], sc[KC];
+  float m[TM], l[TM], o[TM][8];
 #pragma unroll
-    for (int j = 0; j < KC; ++j) {
-      const bool valid = k0 + j < kvL;
-      const float* kvrow = kvsrc + static_cast<size_t>(kv0 + (valid ? k0 + j : 0)) * p.ld_kv;
+  for (int i = 0; i < TM; ++i) {
+    m[i] = -INFINITY;
+    l[i] = 0.f;
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int c = lane + 32 * i;
-        const bool in = valid && i < per && c < dh;
-        kv_k[j][i] = in ? kvrow[p.xk0 + h * dh + c] : 0.f;
-        kv_v[j][i] = in ? kvrow[p.xv0 + h * dh + c] : 0.f;
+    for (int c = 0; c < 8; ++c) o[i][c] = 0.f;
+  }
+  const int c0 = 4 * tx, c1 = 64 + 4 * tx;            // output columns of this thread
+  const bool has0 = c0 < dh, has1 = c1 < dh;
+  const int tiles = (kvL + AKV - 1) / AKV;
+  for (int t = 0; t < tiles; ++t) {
+    cp_async_wait<1>();                               // K of tile t (its V is the group after)
+    __syncthreads();
+    float sc[TM][4] = {};
+    for (int k = 0; k < dh; k += 4) {
+      float4 kk[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) kk[j] = *reinterpret_cast<const float4*>(Ks + (tx + 16 * j) * ld + k);
+#pragma unroll
+      for (int i = 0; i < TM; ++i) {
+        const float4 q = *reinterpret_cast<const float4*>(Qs + (ty + TY * i) * ld + k);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          sc[i][j] = fmaf(q.x, kk[j].x, sc[i][j]);
+          sc[i][j] = fmaf(q.y, kk[j].y, sc[i][j]);
+          sc[i][j] = fmaf(q.z, kk[j].z, sc[i][j]);
+          sc[i][j] = fmaf(q.w, kk[j].w, sc[i][j]);
+        }
       }
     }
+    __syncthreads();                                  // every warp is done with K
+    if (t + 1 < tiles) load_keys(Ks, p.xk0, (t + 1) * AKV);
+    else cp_async_commit();
+    const int valid = kvL - t * AKV;                  // keys of this tile, >= 1
 #pragma unroll
-    for (int j = 0; j < KC; ++j) {
-      float part = 0.f;
+    for (int i = 0; i < TM; ++i) {
+      float mx = m[i];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) part = fmaf(q[i], kv_k[j][i], part);
-      sc[j] = part;
+      for (int j = 0; j < 4; ++j) {
+        sc[i][j] = tx + 16 * j < valid ? sc[i][j] * scale : -INFINITY;
+        mx = fmaxf(mx, sc[i][j]);
+      }
+#pragma unroll
+      for (int off = 8; off > 0; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
+      const float alpha = expf(m[i] - mx);
+      m[i] = mx;
+      float sum = 0.f;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const float e = expf(sc[i][j] - mx);
+        sum += e;
+        Ps[(ty + TY * i) * APS + tx + 16 * j] = e;
+      }
+      l[i] = l[i] * alpha + sum;                      // this thread's share; summed over the row at the end
+#pragma unroll
+      for (int c = 0; c < 8; ++c) o[i][c] *= alpha;
     }
+    cp_async_wait<1>();                               // V of tile t
+    __syncthreads();
+    const int keys = min(AKV, (valid + 3) & ~3);      // past the valid keys P is 0 and V is zero-filled
+    for (int k = 0; k < keys; k += 4) {
+      float4 pr[TM];
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1)
+      for (int i = 0; i < TM; ++i) pr[i] = *reinterpret_cast<const float4*>(Ps + (ty + TY * i) * APS + k);
 #pragma unroll
-      for (int j = 0; j < KC; ++j) sc[j] += __shfl_xor_sync(0xffffffffu, sc[j], off);
-    float m_new = m;
+      for (int e = 0; e < 4; ++e) {
+        const float* vrow = Vs + (k + e) * ld;
+        if (has0) {
+          const float4 v = *reinterpret_cast<const float4*>(vrow + c0);
 #pragma unroll
-    for (int j = 0; j < KC; ++j) {
-      sc[j] = k0 + j < kvL ? sc[j] * scale : -INFINITY;
-      m_new = fmaxf(m_new, sc[j]);
+          for (int i = 0; i < TM; ++i) {
+            const float w = e == 0 ? pr[i].x : (e == 1 ? pr[i].y : (e == 2 ? pr[i].z : pr[i].w));
+            o[i][0] = fmaf(w, v.x, o[i][0]);
+            o[i][1] = fmaf(w, v.y, o[i][1]);
+            o[i][2] = fmaf(w, v.z, o[i][2]);
+            o[i][3] = fmaf(w, v.w, o[i][3]);
+          }
+        }
+        if (has1) {
+          const float4 v = *reinterpret_cast<const float4*>(vrow + c1);
+#pragma unroll
+          for (int i = 0; i < TM; ++i) {
+            const float w = e == 0 ? pr[i].x : (e == 1 ? pr[i].y : (e == 2 ? pr[i].z : pr[i].w));
+            o[i][4] = fmaf(w, v.x, o[i][4]);
+            o[i][5] = fmaf(w, v.y, o[i][5]);
+            o[i][6] = fmaf(w, v.z, o[i][6]);
+            o[i][7] = fmaf(w, v.w, o[i][7]);
+          }
+        }
+      }
     }
-    const float alpha = expf(m - m_new);
-    l *= alpha;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) o[i] *= alpha;
-#pragma unroll
-    for (int j = 0; j < KC; ++j) {
-      const float pr = expf(sc[j] - m_new);
-      l += pr;
-#pragma unroll
-      for (int i = 0; i < 4; ++i) o[i] = fmaf(pr, kv_v[j][i], o[i]);
-    }
-    m = m_new;
+    __syncthreads();                                  // every warp is done with V
+    if (t + 1 < tiles) load_keys(Vs, p.xv0, (t + 1) * AKV);
+    else cp_async_commit();
   }
-  float* out = reinterpret_cast<float*>(p.out) + static_cast<size_t>(row) * p.ldo + h * dh;
-  for (int i = 0; i < per; ++i) {
-    const int c = lane + 32 * i;
-    if (c < dh) out[c] = o[i] / l;
+#pragma unroll
+  for (int i = 0; i < TM; ++i) {
+    float sum = l[i];
+#pragma unroll
+    for (int off = 8; off > 0; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
+    const int r = ty + TY * i;
+    if (r >= rows) continue;
+    float* out = reinterpret_cast<float*>(p.out) + static_cast<size_t>(seq0 + q0 + r) * p.ldo + h * dh;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      if (has0) out[c0 + c] = o[i][c] / sum;
+      if (has1) out[c1 + c] = o[i][4 + c] / sum;
+    }
   }
 }
 
 }  // namespace
 
-cudaError_t launch_simt_gemm(int mode, const float* A, const float* B0, const float* B1, const GemmParams& p,
-                             cudaStream_t st) {
-  int mtiles;
-  if (mode == kGemmCount) mtiles = p.B * ((p.Nw + TB - 1) / TB);
-  else mtiles = (p.M_cap + TB - 1) / TB;
-  const int ntiles = (p.N + TB - 1) / TB;
+namespace {
+
+template <int MODE, int BM, int BN, int TM, int TN, int TK, int STAGES, int MIN_BLOCKS, int VEC>
+cudaError_t launch_vec(dim3 grid, const float* A, const float* B0, const float* B1, const GemmParams& p, cudaStream_t st) {
+  constexpr int smem = static_cast<int>(sizeof(float)) * STAGES * (BM + BN) * staged_ld(TK);
+  if (smem > 48 * 1024) {
+    static bool attr_set[64] = {};
+    cudaError_t e = set_smem_limit_once(simt_gemm_kernel<MODE, BM, BN, TM, TN, TK, STAGES, MIN_BLOCKS, VEC>, smem, attr_set);
+    if (e != cudaSuccess) return e;
+  }
+  return launch_kernel(simt_gemm_kernel<MODE, BM, BN, TM, TN, TK, STAGES, MIN_BLOCKS, VEC>, grid, dim3((BM / TM) * (BN / TN)), smem, st,
+                       A, B0, B1, p);
+}
+
+template <int MODE, int BM, int BN, int TM, int TN, int TK, int STAGES, int MIN_BLOCKS>
+cudaError_t launch_tile(const float* A, const float* B0, const float* B1, const GemmParams& p, bool vec,
+                        cudaStream_t st) {
+  constexpr int COLS = (MODE == kGemmSwiglu || MODE == kGemmCount) ? BN / 2 : BN;
+  const long mtiles = MODE == kGemmCount ? static_cast<long>(p.B) * ((p.Nw + BM - 1) / BM) : (p.M_cap + BM - 1l) / BM;
+  const long ntiles = (p.N + COLS - 1l) / COLS;
   if (mtiles <= 0 || ntiles <= 0) return cudaSuccess;
   if (mtiles > 65535) return cudaErrorInvalidValue;
-  dim3 grid(ntiles, mtiles);
+  const dim3 grid(static_cast<unsigned>(ntiles), static_cast<unsigned>(mtiles));
+  return vec ? launch_vec<MODE, BM, BN, TM, TN, TK, STAGES, MIN_BLOCKS, 4>(grid, A, B0, B1, p, st)
+             : launch_vec<MODE, BM, BN, TM, TN, TK, STAGES, MIN_BLOCKS, 1>(grid, A, B0, B1, p, st);
+}
+
+// The largest tile that leaves every SM several blocks (us at 64 x 64 / 32 x 64 /
+// 32 x 32 / 16 x 32 tiles; the transposing 64 x 64 kernel before): 2624 x 1536 x 512
+// 108 / 112 / 134 / 189 (147); 2624 x 512 x 1536 150 / 142 / 143 / 199 (191); 600 x
+// 1536 x 512 49 / 29 / 35 / 50; 600 x 512 x 1536 75 / 50 / 39 / 57; 208 x 768 x 256
+// 13 / 11 / 9.1 / 8.7 (16); 208 x 256 x 768 41 / 27 / 17 / 14 (44); 8192 x 4096 x 1024
+// 44 TFLOP/s at 64 x 64.
+template <int MODE>
+cudaError_t launch_mode(const float* A, const float* B0, const float* B1, const GemmParams& p, int num_sms,
+                        cudaStream_t st) {
+  const auto aligned = [](const float* q) { return (reinterpret_cast<uintptr_t>(q) & 15u) == 0; };
+  const bool vec = p.K % 4 == 0 && aligned(A) && aligned(B0) && (B1 == nullptr || aligned(B1));
+  constexpr bool TWO = MODE == kGemmSwiglu || MODE == kGemmCount;
+  const auto m_tiles = [&](int bm) {
+    return MODE == kGemmCount ? static_cast<long>(p.B) * ((p.Nw + bm - 1) / bm) : (p.M_cap + bm - 1l) / bm;
+  };
+  const auto tiles = [&](int bm, int bn) { return m_tiles(bm) * ((p.N + (TWO ? bn / 2 : bn) - 1l) / (TWO ? bn / 2 : bn)); };
+  if (tiles(64, 64) >= 4l * num_sms || m_tiles(32) > 65535)
+    return launch_tile<MODE, 64, 64, 8, 4, 32, 3, 3>(A, B0, B1, p, vec, st);
+  if (tiles(32, 64) >= 2l * num_sms) return launch_tile<MODE, 32, 64, 4, 4, 32, 4, 4>(A, B0, B1, p, vec, st);
+  if (tiles(32, 32) >= num_sms || m_tiles(16) > 65535)
+    return launch_tile<MODE, 32, 32, 4, 2, 32, 5, 1>(A, B0, B1, p, vec, st);
+  return launch_tile<MODE, 16, 32, 2, 2, 32, 6, 1>(A, B0, B1, p, vec, st);
+}
+
+template <int BQ, int TY, int VEC>
+cudaError_t launch_attn(const float* qkv, const AttnParams& p, cudaStream_t st) {
+  const long blocks = ((static_cast<long>(p.T_cap) + BQ - 1) / BQ + p.B) * p.n_heads;
+  if (blocks > 0x7fffffffL) return cudaErrorInvalidValue;
+  constexpr auto bytes = [](int dh) { return static_cast<int>(sizeof(float)) * ((BQ + 2 * AKV) * attn_ld(dh) + BQ * APS); };
+  static bool attr_set[64] = {};
+  cudaError_t e = set_smem_limit_once(simt_attn_kernel<BQ, TY, VEC>, bytes(128), attr_set);
+  if (e != cudaSuccess) return e;
+  return launch_kernel(simt_attn_kernel<BQ, TY, VEC>, dim3(static_cast<unsigned>(blocks)), dim3(16 * TY), bytes(p.head_dim), st,
+                       qkv, p);
+}
+
+}  // namespace
+
+cudaError_t launch_simt_gemm(int mode, const float* A, const float* B0, const float* B1, const GemmParams& p,
+                             int num_sms, cudaStream_t st) {
   switch (mode) {
-    case kGemmStore: return launch_kernel(simt_gemm_kernel<kGemmStore>, grid, dim3(256), 0, st, A, B0, B1, p);
-    case kGemmResidual: return launch_kernel(simt_gemm_kernel<kGemmResidual>, grid, dim3(256), 0, st, A, B0, B1, p);
-    case kGemmSwiglu: return launch_kernel(simt_gemm_kernel<kGemmSwiglu>, grid, dim3(256), 0, st, A, B0, B1, p);
-    case kGemmCount: return launch_kernel(simt_gemm_kernel<kGemmCount>, grid, dim3(256), 0, st, A, B0, B1, p);
+    case kGemmStore: return launch_mode<kGemmStore>(A, B0, B1, p, num_sms, st);
+    case kGemmResidual: return launch_mode<kGemmResidual>(A, B0, B1, p, num_sms, st);
+    case kGemmSwiglu: return launch_mode<kGemmSwiglu>(A, B0, B1, p, num_sms, st);
+    case kGemmCount: return launch_mode<kGemmCount>(A, B0, B1, p, num_sms, st);
     default: return cudaErrorInvalidValue;
   }
 }
 
-cudaError_t launch_simt_attn(const float* qkv, const AttnParams& p, cudaStream_t st) {
-  const long tasks = static_cast<long>(p.T_cap) * p.n_heads;
-  if (tasks <= 0) return cudaSuccess;
-  const long blocks = (tasks + 7) / 8;
-  if (blocks > 0x7fffffffL) return cudaErrorInvalidValue;
-  return launch_kernel(simt_attn_kernel, dim3(static_cast<unsigned>(blocks)), dim3(256), 0, st, qkv, p);
+cudaError_t launch_simt_attn(const float* qkv, const AttnParams& p, int num_sms, cudaStream_t st) {
+  if (p.T_cap <= 0) return cudaSuccess;
+  const auto aligned = [](const void* q) { return (reinterpret_cast<uintptr_t>(q) & 15u) == 0; };
+  // rows of the separate K/V source start 16-byte aligned when its width and columns do
+  const bool vec = aligned(qkv) && (p.kv == nullptr || (aligned(p.kv) && p.ld_kv % 4 == 0)) && p.xk0 % 4 == 0 && p.xv0 % 4 == 0;
+  // 32-row tiles once their blocks fill the SMs twice (unless most segments are far
+  // shorter), then 16-row tiles, with twice the threads where even those leave SMs
+  // idle.  Measured at 32 rows / 16 rows / 16 rows with 256 threads, us: segments of
+  // 114 .. 794 rows, 8 heads of 64 146 / 166 / 214; one of 700 rows 92 / 83 / 97; one of
+  // 121 rows, 4 heads 16 / 14 / 10; 64-row tiles 154 / 123 / 20.
+  const auto blocks = [&](long bq) { return (p.T_cap / bq + p.B) * p.n_heads; };
+  if (blocks(32) >= 2l * num_sms && p.T_cap / p.B >= 16)
+    return vec ? launch_attn<32, 8, 4>(qkv, p, st) : launch_attn<32, 8, 1>(qkv, p, st);
+  if (blocks(16) >= num_sms) return vec ? launch_attn<16, 8, 4>(qkv, p, st) : launch_attn<16, 8, 1>(qkv, p, st);
+  return vec ? launch_attn<16, 16, 4>(qkv, p, st) : launch_attn<16, 16, 1>(qkv, p, st);
 }
 
 }  // namespace seer

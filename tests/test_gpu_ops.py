@@ -109,6 +109,66 @@ def test_swiglu_tile_choices(M, F, K):
     assert torch.isnan(act[M]).all()
 
 
+@pytest.mark.parametrize("M,N,K", [(1, 4, 4), (31, 33, 17), (33, 96, 768), (65, 260, 35), (130, 3000, 20),
+                                   (300, 1000, 100), (1300, 1030, 36), (2000, 2050, 6)])
+@pytest.mark.parametrize("offset", [0, 1])
+def test_linear_f32_tile_choices(M, N, K, offset):
+    """Every fp32 tile size at ragged edges, 16-byte copies and (odd K or operands
+    one float past a 16-byte boundary) 4-byte copies; small integers: exact."""
+    rng = _rng(M + N + K)
+    a, w, r = (torch.from_numpy(rng.integers(-4, 5, (m, n)).astype(np.float32)).to(cuda())
+               for m, n in ((M, K), (N, K), (M, N)))
+    off = lambda t: torch.cat([t.new_zeros(offset), t.flatten()])[offset:].view(t.shape)
+    c = torch.full((M + 1, N), float("nan"), dtype=torch.float32, device=cuda())
+    S.seer_linear(off(a), off(w), "f32", r, "f32", c, "f32", M, None, N, K)
+    assert torch.equal(c[:M], (a.double() @ w.double().T + r.double()).float())
+    assert torch.isnan(c[M]).all()
+
+
+@pytest.mark.parametrize("M,F,K", [(9, 36, 20), (70, 130, 33), (200, 1540, 12), (900, 2052, 20)])
+def test_swiglu_f32_tile_choices(M, F, K):
+    """fp32 gate/up tiles of every size with the count hook; activations against
+    fp64, counts against the kernel's own activations."""
+    rng = _rng(M + F + K)
+    a, wg, wu = (rng.standard_normal(s).astype(np.float32) * c for s, c in (((M, K), 1.0), ((F, K), 0.3), ((F, K), 0.3)))
+    act = torch.full((M + 1, F), float("nan"), dtype=torch.float32, device=cuda())
+    counts = torch.zeros(M, dtype=torch.int32, device=cuda())
+    S.seer_swiglu(to_dev(a, "f32"), to_dev(wg, "f32"), to_dev(wu, "f32"), "f32", act, "f32", M, None, F, K, i32([0, M]), 1,
+                  i32([0]), M, 0.05, counts)
+    g, u = (a.astype(np.float64) @ w.astype(np.float64).T for w in (wg, wu))
+    check_close(host(act[:M]), g / (1.0 + np.exp(-g)) * u, "f32", "swiglu f32")
+    assert torch.isnan(act[M]).all()
+    eps = torch.tensor(0.05, dtype=torch.float32, device=cuda())
+    assert torch.equal(counts, (act[:M].abs() < eps).sum(1, dtype=torch.int32))
+
+
+@pytest.mark.parametrize("H,dh,lens,kv", [
+    (2, 64, [1, 15, 16, 17], [1, 15, 9, 17]),                       # 16-row tiles, 256 threads
+    (3, 4, [5, 64, 65], [5, 64, 1]), (2, 28, [70, 3, 129], [70, 2, 128]), (1, 100, [200], [130]), (2, 128, [131], [131]),
+    (16, 64, [150, 31], [97, 31]), (12, 128, [200], [129]),         # 16-row tiles
+    (32, 32, [400, 63, 257], [399, 63, 64]),                        # 32-row tiles
+    (40, 128, [300, 129, 64], [300, 65, 64]), (40, 12, [500, 33], [461, 33])])
+@pytest.mark.parametrize("offset", [0, 1])
+def test_attention_f32_tile_choices(H, dh, lens, kv, offset):
+    """fp32 attention at the edges of its query and key tiles and head widths, rows
+    16-byte aligned and not; keys past kv_len hold NaN and must not be read."""
+    D, T = H * dh, sum(lens)
+    rng = _rng(H + dh + T)
+    x = rng.standard_normal((T, 3 * D)).astype(np.float32)
+    cu = np.concatenate([[0], np.cumsum(lens)])
+    dirty = x.copy()
+    for a, b, k in zip(cu[:-1], cu[1:], kv):
+        dirty[a + k:b, D:] = np.nan
+    buf = torch.from_numpy(np.concatenate([np.zeros(offset, np.float32), dirty.ravel()])).to(cuda())
+    o = torch.full((T + 1, D), float("nan"), dtype=torch.float32, device=cuda())
+    S.seer_attention(buf[offset:], o, "f32", i32(cu), i32(kv), len(lens), T, H, dh)
+    ref = np.concatenate([oracle.attention(*(x[a:a + n, c * D:(c + 1) * D].astype(np.float64)
+                                             for c, n in ((0, b - a), (1, k), (2, k))), H)
+                          for a, b, k in zip(cu[:-1], cu[1:], kv)])
+    check_close(host(o[:T]), ref, "f32", "attention f32")
+    assert torch.isnan(o[T]).all()
+
+
 # ------------------------------------------------------------------ SwiGLU + count hook (S10, S1)
 @pytest.mark.parametrize("op", ["bf16", "f16"])
 def test_swiglu_counts_at_the_threshold_follow_the_ieee_quotient(op):
