@@ -400,9 +400,8 @@ __device__ __forceinline__ int elect_lane0() { return (threadIdx.x & 31) == 0; }
 // programmatic dependent of the previous kernel in the stream (when launch
 // overlap is on): the next kernel may be launched, and its blocks placed,
 // before the current one has finished.  Every kernel of the library calls
-// pdl_wait() before anything else: it returns once the kernels it depends on
-// have completed and their writes are visible, so no kernel touches global
-// memory while its predecessor runs.  pdl_trigger() lets the next kernel
+// pdl_wait() before it touches global memory: it returns once the kernels it
+// depends on have completed and their writes are visible.  pdl_trigger() lets the next kernel
 // launch; a kernel calls it only after its own wait, which keeps the chain
 // ordered, and where it calls it sets how long the successor's blocks sit
 // waiting: short kernels trigger at entry, the persistent GEMM once its last

@@ -26,9 +26,10 @@
 //               32 x 32 output chunks staged in shared memory and written by
 //               TMA stores marked L2 evict-first (a tile whose rows run past
 //               the device row count stores its valid rows lane by lane).
-// The epilogue of tile t overlaps the main loop of tile t+1.  Every CTA waits
-// for the previous kernel of the stream at entry (griddepcontrol.wait) and
-// lets the next kernel launch once its last MMAs are issued.
+// The epilogue of tile t overlaps the main loop of tile t+1.  Every CTA sets up
+// its barriers and tensor memory, then waits for the previous kernel of the
+// stream (griddepcontrol.wait), and lets the next kernel launch once its last
+// MMAs are issued.
 //
 // Epilogues (Sec. 3.1 Eq. 2 projections; Sec. 3.2 sparsity hook):
 //   Store     C = A B^T                                    (QKV projection)
@@ -123,7 +124,6 @@ template <int MODE, int CG>
 __global__ void __launch_bounds__(THREADS, 1)
     tc_gemm_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CUtensorMap mB0,
                    const __grid_constant__ CUtensorMap mB1, const __grid_constant__ CUtensorMap mC, const GemmParams p) {
-  pdl_wait();
   const int BN = p.bn;
   const int stages = p.stages;
   const int sbytes = stage_bytes(CG, BN);
@@ -142,6 +142,32 @@ __global__ void __launch_bounds__(THREADS, 1)
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
   const uint32_t rank = CG == 2 ? cluster_ctarank() : 0u;   // CTA of the pair; rank 0 issues the MMAs
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < stages; ++s) {
+      mbar_init(&full[s], 1);
+      mbar_init(&empty[s], 1);
+    }
+    for (int a = 0; a < 2; ++a) {
+      mbar_init(&acc_full[a], 1);
+      mbar_init(&acc_empty[a], 4 * CG);                     // every epilogue warp of the tile's CTAs
+    }
+    *abort_flag = 0;
+    fence_barrier_init();
+    tma_prefetch_desc(&mA);
+    tma_prefetch_desc(&mB0);
+    tma_prefetch_desc(&mB1);
+  }
+  if (warp == 1) tmem_alloc<CG>(tmem_slot, TMEM_COLS);
+  tc_fence_before();
+  __syncthreads();
+  if (CG == 2) cluster_sync();                              // the peer's barriers are initialised
+  tc_fence_after();
+  const uint32_t tmem_base = *tmem_slot;
+
+  // barriers, tensor memory and descriptors are set up while the previous kernel
+  // drains; nothing before this reads or writes global memory
+  pdl_wait();
 
   // ---- problem size (device row counts are clamped, never trusted blindly)
   int M = p.M_cap;
@@ -170,25 +196,6 @@ __global__ void __launch_bounds__(THREADS, 1)
   const int group_m = p.group_m > 0 ? p.group_m : 1;
   const int t_first = blockIdx.x / CG, t_step = gridDim.x / CG;
 
-  if (threadIdx.x == 0) {
-    for (int s = 0; s < stages; ++s) {
-      mbar_init(&full[s], 1);
-      mbar_init(&empty[s], 1);
-    }
-    for (int a = 0; a < 2; ++a) {
-      mbar_init(&acc_full[a], 1);
-      mbar_init(&acc_empty[a], 4 * CG);                     // every epilogue warp of the tile's CTAs
-    }
-    *abort_flag = 0;
-    fence_barrier_init();
-  }
-  if (warp == 1) tmem_alloc<CG>(tmem_slot, TMEM_COLS);
-  tc_fence_before();
-  __syncthreads();
-  if (CG == 2) cluster_sync();                              // the peer's barriers are initialised
-  tc_fence_after();
-  const uint32_t tmem_base = *tmem_slot;
-
   if (warp == 0) {
     // ------------------------------------------------ TMA producer
     // Producer and issuer run as whole warps in lockstep (every wait by all
@@ -201,11 +208,6 @@ __global__ void __launch_bounds__(THREADS, 1)
     // then rank 0's barrier has completed the stage's phase, so a peer's bytes
     // can only reach the phase they belong to).
     const bool leader = elect_one();
-    if (leader) {
-      tma_prefetch_desc(&mA);
-      tma_prefetch_desc(&mB0);
-      tma_prefetch_desc(&mB1);
-    }
     const uint32_t full0 = CG == 2 ? cluster_addr(full, 0) : 0u;
     const int half_b = BN / 2 * BK * 2;                     // bytes of one half of B's rows
     int s = 0;
@@ -348,6 +350,20 @@ __global__ void __launch_bounds__(THREADS, 1)
       const int mt = m * CG + static_cast<int>(rank);          // this CTA's 128-row tile
       // columns of this tile inside the matrix (the last tile may be narrower)
       const int cols = min(tile_n, p.N - n * tile_n);
+      const bool slab_full = mt * BM + q * 32 + 32 <= M;       // this warp's 32 rows all valid: TMA store
+      const bool of16 = p.out_type == kF16, rf16 = p.res_type == kF16;
+      const int row = mt * BM + row_in_tile;
+      const bool valid = row < M;
+      // the tile's residual row is loaded while the MMAs run: fetched chunk by chunk
+      // after them, its latency was most of the epilogue (O projection of 842 rows
+      // 26.9 -> 25.0 us)
+      uint4 res[MODE == kGemmResidual ? ACC_COLS / 8 : 1];
+      if (MODE == kGemmResidual) {
+        const uint4* rp = reinterpret_cast<const uint4*>(reinterpret_cast<const uint16_t*>(p.R) +
+                                                         static_cast<size_t>(valid ? row : 0) * p.ldr + n * BN);
+#pragma unroll
+        for (int i = 0; i < ACC_COLS / 8; ++i) res[i] = valid && i * 8 < cols ? rp[i] : make_uint4(0, 0, 0, 0);
+      }
       // warp-uniform outcome: the TMEM loads below are warp-collective, and
       // after an abort the lanes of a warp could otherwise decide differently
       if (!__all_sync(0xffffffffu, mbar_wait(&acc_full[acc], acc_ph, abort_flag, p.err))) break;
@@ -355,11 +371,8 @@ __global__ void __launch_bounds__(THREADS, 1)
       const uint32_t tacc = tmem_base + lane_off + static_cast<uint32_t>(acc * ACC_COLS);
       if (MODE == kGemmRope) {
         // the tile holds whole heads; pair (c, c + 64) of a head rotates by pos * f_c
-        const int row = mt * BM + row_in_tile;
-        const bool valid = row < M;
         const bool rotate = n * BN < p.rope_cols;       // tile-uniform (rope_cols % 256 == 0, BN 128 or 256)
         const int heads = cols / ROPE_HEAD;
-        const bool of16 = p.out_type == kF16;
         uint16_t* crow = reinterpret_cast<uint16_t*>(p.C) + static_cast<size_t>(valid ? row : 0) * p.ldc + n * BN;
         const float pos = (valid && rotate) ? static_cast<float>(row_position(p.cu, p.B, row)) : 0.f;
 #pragma unroll 1
@@ -401,61 +414,57 @@ __global__ void __launch_bounds__(THREADS, 1)
           }
         }
       } else if (MODE == kGemmStore || MODE == kGemmResidual) {
-        const int row = mt * BM + row_in_tile;
-        const bool valid = row < M;
-        const bool slab_full = mt * BM + q * 32 + 32 <= M;     // this warp's 32 rows all valid: TMA store
-        const bool of16 = p.out_type == kF16, rf16 = p.res_type == kF16;
-        uint16_t* crow = reinterpret_cast<uint16_t*>(p.C) + static_cast<size_t>(valid ? row : 0) * p.ldc + n * BN;
-        const uint16_t* rrow =
-            MODE == kGemmResidual ? reinterpret_cast<const uint16_t*>(p.R) + static_cast<size_t>(valid ? row : 0) * p.ldr + n * BN
-                                  : nullptr;
-#pragma unroll 1
-        for (int c = 0; c < cols / 32; ++c) {
-          uint32_t r[32];
-          tmem_ld32(tacc + c * 32, r);
+        // two chunks of 32 columns per step, their accumulator loads in flight together
+#pragma unroll
+        for (int c = 0; c < ACC_COLS / 32; c += 2) {
+          if (c * 32 >= cols) break;
+          uint32_t acc32[2][32];
+          tmem_ld32(tacc + c * 32, acc32[0]);
+          tmem_ld32(tacc + c * 32 + 32, acc32[1]);        // past bn: stale columns, not stored
           tmem_ld_wait();
-          if (slab_full || valid) {
-            float v[32];
 #pragma unroll
-            for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
-            if (MODE == kGemmResidual) {
-              const uint4* rp = reinterpret_cast<const uint4*>(rrow + c * 32);
+          for (int h = 0; h < 2; ++h) {
+            if ((c + h) * 32 < cols && (slab_full || valid)) {
+              float v[32];
 #pragma unroll
-              for (int i = 0; i < 4; ++i) {
-                const uint4 rv = rp[i];
-                v[8 * i + 0] += lo16(rv.x, rf16); v[8 * i + 1] += hi16(rv.x, rf16);
-                v[8 * i + 2] += lo16(rv.y, rf16); v[8 * i + 3] += hi16(rv.y, rf16);
-                v[8 * i + 4] += lo16(rv.z, rf16); v[8 * i + 5] += hi16(rv.z, rf16);
-                v[8 * i + 6] += lo16(rv.w, rf16); v[8 * i + 7] += hi16(rv.w, rf16);
+              for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(acc32[h][i]);
+              if (MODE == kGemmResidual) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                  const uint4 rv = res[(c + h) * 4 + i];
+                  v[8 * i + 0] += lo16(rv.x, rf16); v[8 * i + 1] += hi16(rv.x, rf16);
+                  v[8 * i + 2] += lo16(rv.y, rf16); v[8 * i + 3] += hi16(rv.y, rf16);
+                  v[8 * i + 4] += lo16(rv.z, rf16); v[8 * i + 5] += hi16(rv.z, rf16);
+                  v[8 * i + 6] += lo16(rv.w, rf16); v[8 * i + 7] += hi16(rv.w, rf16);
+                }
               }
-            }
-            uint32_t w[16];
+              uint32_t w[16];
 #pragma unroll
-            for (int i = 0; i < 16; ++i) {
-              w[i] = pack2(v[2 * i], v[2 * i + 1], of16);
-              nonfinite |= nonfinite_term(w[i], of16);
-            }
-            if (slab_full) {
-              store_chunk(w, n * BN + c * 32, mt * BM + q * 32);
-            } else {
-              // a lane owns one row: 64 contiguous bytes as two full 32-byte sectors
-              st_global_v8(crow + c * 32, w[0], w[1], w[2], w[3], w[4], w[5], w[6], w[7]);
-              st_global_v8(crow + c * 32 + 16, w[8], w[9], w[10], w[11], w[12], w[13], w[14], w[15]);
+              for (int i = 0; i < 16; ++i) {
+                w[i] = pack2(v[2 * i], v[2 * i + 1], of16);
+                nonfinite |= nonfinite_term(w[i], of16);
+              }
+              if (slab_full) {
+                store_chunk(w, n * BN + (c + h) * 32, mt * BM + q * 32);
+              } else {
+                // a lane owns one row: 64 contiguous bytes as two full 32-byte sectors
+                uint16_t* crow = reinterpret_cast<uint16_t*>(p.C) + static_cast<size_t>(row) * p.ldc + n * BN + (c + h) * 32;
+                st_global_v8(crow, w[0], w[1], w[2], w[3], w[4], w[5], w[6], w[7]);
+                st_global_v8(crow + 16, w[8], w[9], w[10], w[11], w[12], w[13], w[14], w[15]);
+              }
             }
           }
         }
       } else {
         // gate columns 0 .. BN/2 - 1, up columns BN/2 .. BN - 1 of the accumulator
-        int row, cnt_idx = -1;
+        int cnt_idx = -1;
         bool store = false;
         if (MODE == kGemmCount) {
           const int b = mt / tiles_per_seq;
           const int tl = (mt - b * tiles_per_seq) * BM + row_in_tile;
-          row = -1;
           if (mt < num_mt && tl < p.Nw) cnt_idx = b * p.Nw + tl;
         } else {
-          row = mt * BM + row_in_tile;
-          store = row < M;
+          store = valid;
           if (store && p.counts != nullptr) {
             // segment of this row (binary search in cu), then its window offset
             int lo = 0, hi = p.B;
@@ -468,7 +477,6 @@ __global__ void __launch_bounds__(THREADS, 1)
           }
         }
         int cnt = 0;
-        const bool of16 = p.out_type == kF16;
         uint16_t* arow =
             MODE == kGemmSwiglu ? reinterpret_cast<uint16_t*>(p.C) + static_cast<size_t>(store ? row : 0) * p.ldc + n * tile_n
                                 : nullptr;
@@ -483,7 +491,6 @@ __global__ void __launch_bounds__(THREADS, 1)
           for (int i = 0; i < 32; ++i) a[i] = silu_fast(__uint_as_float(g[i])) * __uint_as_float(u[i]);
           if (cnt_idx >= 0) cnt += count_near_zero(a, g, u, p.act_eps);
           if (MODE == kGemmSwiglu) {
-            const bool slab_full = mt * BM + q * 32 + 32 <= M;
             if (slab_full || store) {
               uint32_t w[16];
 #pragma unroll
@@ -544,16 +551,11 @@ cudaError_t launch_mode(const GemmPlan& plan, const CUtensorMap& mA, const CUten
   const int units = num_sms / CG;
   const int grid = static_cast<int>(tiles < units ? tiles : units);
   const int smem = plan.stages * stage_bytes(CG, plan.bn) + FIXED_BYTES;
-  // Overlapping the launch with the previous kernel pays off for short GEMMs,
-  // where the launch gap is a visible share of the run.  Long GEMMs launched
-  // that way measured 5-8% slower on GB300 (cause not isolated; their blocks
-  // are then placed in the order the previous kernel's blocks retire), so
-  // they launch normally.
-  constexpr long kOverlapMaxSteps = 320;     // k-blocks per CTA (about five 64-deep tiles)
-  const long steps = (tiles * (p.K / BK) + grid - 1) / grid;
-  const bool overlap = launch_overlap_enabled() && steps <= kOverlapMaxSteps;
-  return launch_kernel_overlap(overlap, CG, tc_gemm_kernel<MODE, CG>, dim3(grid * CG), dim3(THREADS), smem, st, mA, mB0,
-                               mB1, mC, p);
+  // long calls gain little from the overlap but lose nothing (one layer of 35k rows:
+  // 11.9 ms either way); one of 842 rows 391 us without any, 383 with calls of up to
+  // five tiles per SM overlapped, 379 with all
+  return launch_kernel_overlap(launch_overlap_enabled(), CG, tc_gemm_kernel<MODE, CG>, dim3(grid * CG), dim3(THREADS),
+                               smem, st, mA, mB0, mB1, mC, p);
 }
 
 template <int MODE>
