@@ -53,10 +53,10 @@ __device__ __forceinline__ uint32_t store8(void* base, size_t i8, const float (&
 
 // y = x * rsqrt(mean(x^2) + eps) * g, one warp per row; input type IN, output
 // (and gain) type OUT; fp32 arithmetic.
-template <int IN, int OUT>
+template <int IN, int OUT, bool MAP>
 __global__ void __launch_bounds__(256) rmsnorm_kernel(const void* __restrict__ x, const void* __restrict__ g,
                                                       void* __restrict__ y, int M_cap, const int* M_dev, int d,
-                                                      float eps, int* err) {
+                                                      float eps, const RowMap map, int* err) {
   pdl_enter();
   int M = M_cap;
   if (M_dev != nullptr) {
@@ -74,10 +74,12 @@ __global__ void __launch_bounds__(256) rmsnorm_kernel(const void* __restrict__ x
   uint32_t nonfinite = 0;
   for (int row = blockIdx.x * 8 + warp; row < M; row += nwarps) {
     const size_t base8 = static_cast<size_t>(row) * d8;
+    const int src = MAP ? mapped_row(map, row, M_cap, err) : row;
+    const size_t src8 = static_cast<size_t>(src < 0 ? 0 : src) * d8;
     float ss = 0.f;
     for (int v = lane; v < d8; v += 32) {
       float e[8];
-      load8<IN>(x, base8 + v, e);
+      load8<IN>(x, src8 + v, e);
 #pragma unroll
       for (int i = 0; i < 8; ++i) ss = fmaf(e[i], e[i], ss);
     }
@@ -86,10 +88,10 @@ __global__ void __launch_bounds__(256) rmsnorm_kernel(const void* __restrict__ x
     const float inv = rsqrtf(ss / static_cast<float>(d) + eps);
     for (int v = lane; v < d8; v += 32) {
       float e[8], gg[8];
-      load8<IN>(x, base8 + v, e);
+      load8<IN>(x, src8 + v, e);
       load8<OUT>(g, v, gg);
 #pragma unroll
-      for (int i = 0; i < 8; ++i) e[i] = e[i] * inv * gg[i];
+      for (int i = 0; i < 8; ++i) e[i] = src < 0 ? 0.f : e[i] * inv * gg[i];
       nonfinite |= store8<OUT>(y, base8 + v, e);
     }
   }
@@ -105,10 +107,10 @@ __global__ void __launch_bounds__(256) rmsnorm_kernel(const void* __restrict__ x
 // the same for every row, is staged once per block in shared memory (8 KB at
 // d = 4096); read from global memory per row, its loads were hoisted beside
 // the row's 64 registers and spilled.
-template <int IN, int OUT, int VPL>
+template <int IN, int OUT, int VPL, bool MAP>
 __global__ void __launch_bounds__(256, 2) rmsnorm_rows_kernel(const void* __restrict__ x, const void* __restrict__ g,
                                                            void* __restrict__ y, int M_cap, const int* M_dev, int d,
-                                                           float eps, int* err) {
+                                                           float eps, const RowMap map, int* err) {
   pdl_enter();
   int M = M_cap;
   if (M_dev != nullptr) {
@@ -131,11 +133,13 @@ __global__ void __launch_bounds__(256, 2) rmsnorm_rows_kernel(const void* __rest
   uint32_t nonfinite = 0;
   for (int row = blockIdx.x * 8 + warp; row < M; row += nwarps) {
     const size_t base8 = static_cast<size_t>(row) * d8;
+    const int src = MAP ? mapped_row(map, row, M_cap, err) : row;
+    const size_t src8 = static_cast<size_t>(src) * d8;
     uint4 raw[VPL];
 #pragma unroll
     for (int i = 0; i < VPL; ++i) {
       const int v = lane + 32 * i;
-      raw[i] = v < d8 ? __ldg(xv + base8 + v) : make_uint4(0, 0, 0, 0);
+      raw[i] = v < d8 && src >= 0 ? __ldg(xv + src8 + v) : make_uint4(0, 0, 0, 0);
     }
     // the sum of squares unpacks through an opaque copy of each word, so the
     // scaling below unpacks again instead of keeping 8 floats per vector live
@@ -541,29 +545,37 @@ __global__ void __launch_bounds__(256, 4) pack_route_kernel(const uint8_t* __res
 }  // namespace
 
 cudaError_t launch_rmsnorm(const void* x, int in_type, const void* g, void* y, int out_type, int M_cap,
-                           const int* M_dev, int d, float eps, int* err, cudaStream_t st) {
+                           const int* M_dev, int d, float eps, const RowMap& map, int* err, cudaStream_t st) {
   if (M_cap <= 0) return cudaSuccess;
   int blocks = (M_cap + 7) / 8;
   if (blocks > 65535 * 4) blocks = 65535 * 4;
   // 16-bit rows up to 4096 wide: register-resident variant sized to the row
   const int vpl = (d / 8 + 31) / 32;
-#define SEER_NORM_ROWS(I, O, V)                                                                                   \
-  if (in_type == I && out_type == O && vpl <= V)                                                                 \
-    return launch_kernel(rmsnorm_rows_kernel<I, O, V>, dim3(blocks), dim3(256), 0, st, x, g, y, M_cap, M_dev, d, \
-                         eps, err);
-#define SEER_NORM_16(I, O) SEER_NORM_ROWS(I, O, 4) SEER_NORM_ROWS(I, O, 8) SEER_NORM_ROWS(I, O, 16)
-  SEER_NORM_16(kBF16, kF16)
-  SEER_NORM_16(kF16, kF16)
-  SEER_NORM_16(kBF16, kBF16)
+#define SEER_NORM_ROWS(I, O, V, MAPPED)                                                                              \
+  if (in_type == I && out_type == O && vpl <= V && mapped == MAPPED)                                                 \
+    return launch_kernel(rmsnorm_rows_kernel<I, O, V, MAPPED>, dim3(blocks), dim3(256), 0, st, x, g, y, M_cap, M_dev, \
+                         d, eps, map, err);
+#define SEER_NORM_16(I, O, MAPPED) \
+  SEER_NORM_ROWS(I, O, 4, MAPPED) SEER_NORM_ROWS(I, O, 8, MAPPED) SEER_NORM_ROWS(I, O, 16, MAPPED)
+#define SEER_NORM(I, O, MAPPED)                                                                                  \
+  if (in_type == I && out_type == O && mapped == MAPPED)                                                         \
+    return launch_kernel(rmsnorm_kernel<I, O, MAPPED>, dim3(blocks), dim3(256), 0, st, x, g, y, M_cap, M_dev, d, \
+                         eps, map, err);
+  const bool mapped = map.cu != nullptr;          // f16 outputs only (the K/V prefill's norm)
+  SEER_NORM_16(kBF16, kF16, false)
+  SEER_NORM_16(kF16, kF16, false)
+  SEER_NORM_16(kBF16, kBF16, false)
+  SEER_NORM_16(kBF16, kF16, true)
+  SEER_NORM_16(kF16, kF16, true)
+  SEER_NORM(kBF16, kF16, false)
+  SEER_NORM(kF16, kF16, false)
+  SEER_NORM(kBF16, kBF16, false)
+  SEER_NORM(kF32, kF32, false)
+  SEER_NORM(kBF16, kF16, true)
+  SEER_NORM(kF16, kF16, true)
+#undef SEER_NORM
 #undef SEER_NORM_16
 #undef SEER_NORM_ROWS
-#define SEER_NORM(I, O) \
-  if (in_type == I && out_type == O) return launch_kernel(rmsnorm_kernel<I, O>, dim3(blocks), dim3(256), 0, st, x, g, y, M_cap, M_dev, d, eps, err);
-  SEER_NORM(kBF16, kF16)
-  SEER_NORM(kF16, kF16)
-  SEER_NORM(kBF16, kBF16)
-  SEER_NORM(kF32, kF32)
-#undef SEER_NORM
   return cudaErrorInvalidValue;
 }
 

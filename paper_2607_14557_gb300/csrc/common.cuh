@@ -499,4 +499,24 @@ __device__ __forceinline__ int row_position(const int* cu, int B, int row) {
   return row - cu[lo];
 }
 
+// Row of the mapped matrix for `row` (see RowMap), or -1 when the row belongs to no
+// segment or its segment would leave either matrix (src_rows: rows of this one),
+// which is recorded.
+template <typename Map>
+__device__ __forceinline__ int mapped_row(const Map& map, int row, int src_rows, int* err) {
+  int lo = 0, hi = map.B;
+  while (hi - lo > 1) {
+    const int mid = (lo + hi) >> 1;
+    if (map.cu[mid] <= row) lo = mid; else hi = mid;
+  }
+  const int first = map.cu[lo], end = map.cu[lo + 1];
+  if (row < first || row >= end) return -1;
+  const int start = map.start[lo] + (map.add ? map.add[lo] : 0);
+  if (first < 0 || start < 0 || end > src_rows || start + (end - first) > map.rows) {
+    record_error(err, kErrLayout);
+    return -1;
+  }
+  return start + (row - first);
+}
+
 }  // namespace seer

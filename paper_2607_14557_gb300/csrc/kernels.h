@@ -16,6 +16,17 @@ enum GemmMode : int {
   kGemmSwiglu = 2,    // act = SiLU(A Bg^T) * (A Bu^T), optional near-zero counts
   kGemmCount = 3,     // counts only (detector): A rows gathered per sequence window
   kGemmRope = 4,      // C = A B^T, then columns < rope_cols rotated per head (rotary embedding)
+  kGemmKv = 5,        // C = A B^T, columns >= split stored at mapped rows of a second matrix (K/V cache)
+};
+
+// Rows of segments that live at other places in another matrix: row r of segment
+// b (cu[b] <= r < cu[b+1]) is row start[b] (+ add[b]) + r - cu[b] there.
+struct RowMap {
+  const int* cu;          // [B+1], or null: no mapping
+  const int* start;       // [B]
+  const int* add;         // [B], or null
+  int B;
+  int rows;               // rows of the other matrix
 };
 
 struct GemmParams {
@@ -42,6 +53,10 @@ struct GemmParams {
   int group_m;            // raster: row tiles per group (see tc_gemm.cu)
   float rope_theta;       // Rope: frequency base (> 0)
   int rope_cols;          // Rope: leading output columns that are rotated (the q|k columns)
+  void* C2;               // Kv: matrix of the mapped columns [map.rows, ldc2]
+  int ldc2;
+  int split;              // Kv: first mapped column (multiple of 32)
+  RowMap map;             // Kv: where its rows go
 };
 
 struct AttnParams {
@@ -77,10 +92,11 @@ struct GemmPlan {
 GemmPlan tc_gemm_plan(int mode, long m_tiles, long n_cols, int K, int num_sms);
 // mC: the 16-bit output C (Store, Residual, Rope) or act (Swiglu) with 32 x 32
 // boxes and no swizzle, for the epilogue's TMA stores (unused by Count).  mA
-// has boxes of 128 rows, mB0 and mB1 boxes of bn / 2 rows.
+// has boxes of 128 rows, mB0 and mB1 boxes of bn / 2 rows; mC2 is C2 in boxes
+// like mC's (Kv only).
 cudaError_t launch_tc_gemm(int mode, const GemmPlan& plan, const CUtensorMap& mA, const CUtensorMap& mB0,
-                           const CUtensorMap& mB1, const CUtensorMap& mC, const GemmParams& p, int num_sms,
-                           cudaStream_t st);
+                           const CUtensorMap& mB1, const CUtensorMap& mC, const CUtensorMap& mC2, const GemmParams& p,
+                           int num_sms, cudaStream_t st);
 int tc_attn_smem_bytes();
 // grid: persistent CTAs (at most one per SM); they take the units of the
 // schedule from p.work_next until *p.work_count are done
@@ -102,8 +118,10 @@ cudaError_t launch_simt_gemm(int mode, const float* A, const float* B0, const fl
 cudaError_t launch_simt_attn(const float* qkv, const AttnParams& p, int num_sms, cudaStream_t st);
 
 // Element-wise / scan kernels (both storage types).
+// map.cu set: row r of y is the norm of the row of x that the map names (rows
+// of segments outside x become zero and are recorded).
 cudaError_t launch_rmsnorm(const void* x, int in_type, const void* g, void* y, int out_type, int M_cap,
-                           const int* M_dev, int d, float eps, int* err, cudaStream_t st);
+                           const int* M_dev, int d, float eps, const RowMap& map, int* err, cudaStream_t st);
 cudaError_t launch_rope(void* qkv, int type, const int* cu, int B, int T_cap, int n_heads, int head_dim, float theta,
                         int* err, int num_sms, cudaStream_t st);
 // Per-segment row copies (see aux_kernels.cu): rows of segment b go from src

@@ -232,9 +232,18 @@ struct RopeArgs {
   int head_dim = 0;
 };
 
+// Columns >= split of do_linear's product stored at mapped rows of a K/V cache
+// instead (16-bit operands).
+struct KvDest {
+  void* kv = nullptr;      // [map.rows, ld]
+  int ld = 0;
+  int split = 0;
+  RowMap map{};
+};
+
 seer_status do_linear(const void* a, const void* w, seer_dtype op_dt, const void* r, seer_dtype r_dt, void* c,
                       seer_dtype c_dt, int M_cap, const int32_t* M_dev, int N, int K, cudaStream_t st, int phase,
-                      const RopeArgs& rope = RopeArgs()) {
+                      const RopeArgs& rope = RopeArgs(), const KvDest& dest = KvDest()) {
   if (M_cap < 0 || N <= 0 || K <= 0) return fail(SEER_ERR_INVALID_ARG, "linear: bad sizes M=%d N=%d K=%d", M_cap, N, K);
   if (!a || !w || !c) return fail(SEER_ERR_INVALID_ARG, "linear: null pointer");
   if (!valid_dt(op_dt) || !valid_dt(c_dt) || (r && !valid_dt(r_dt))) return fail(SEER_ERR_INVALID_ARG, "linear: unknown dtype");
@@ -255,7 +264,13 @@ seer_status do_linear(const void* a, const void* w, seer_dtype op_dt, const void
   const bool rot = rope.theta > 0.f;
   if (rot && (r || !rope.cu || rope.B <= 0 || N != 3 * rope.n_heads * rope.head_dim))
     return fail(SEER_ERR_INVALID_ARG, "linear: the rotary epilogue needs a q|k|v output, cu_seqlens and no residual");
-  const int mode = r ? kGemmResidual : (rot ? kGemmRope : kGemmStore);
+  const int mode = r ? kGemmResidual : (rot ? kGemmRope : (dest.kv ? kGemmKv : kGemmStore));
+  if (dest.kv) {
+    p.C2 = dest.kv;
+    p.ldc2 = dest.ld;
+    p.split = dest.split;
+    p.map = dest.map;
+  }
   if (rot) {
     p.rope_theta = rope.theta;
     p.rope_cols = 2 * rope.n_heads * rope.head_dim;
@@ -276,8 +291,10 @@ seer_status do_linear(const void* a, const void* w, seer_dtype op_dt, const void
     SEER_TRY(make_map16(&mA, a, op_dt, M_cap, K, K, 128));
     SEER_TRY(make_map16(&mB, w, op_dt, N, K, K, plan.bn / 2));
     SEER_TRY(make_map16(&mC, c, c_dt, M_cap, N, N, 32, 32, false));
+    CUtensorMap mC2 = mC;
+    if (dest.kv) SEER_TRY(make_map16(&mC2, dest.kv, c_dt, dest.map.rows, dest.ld, dest.ld, 32, 32, false));
     Phase ph(phase, st);
-    SEER_CUDA(launch_tc_gemm(mode, plan, mA, mB, mB, mC, p, di->num_sms, st), "tc_gemm launch");
+    SEER_CUDA(launch_tc_gemm(mode, plan, mA, mB, mB, mC, mC2, p, di->num_sms, st), "tc_gemm launch");
   } else {
     if (c_dt != SEER_F32 || (r && r_dt != SEER_F32)) return fail(SEER_ERR_UNSUPPORTED, "fp32 linear needs fp32 output");
     if (M_cap == 0) return SEER_OK;
@@ -344,7 +361,7 @@ seer_status do_swiglu(const void* a, const void* wg, const void* wu, seer_dtype 
     if (mode == kGemmSwiglu) SEER_TRY(make_map16(&mC, act, act_dt, M_cap, F, F, 32, 32, false));
     else mC = mA;                                  // Count stores nothing
     Phase ph(phase, st);
-    SEER_CUDA(launch_tc_gemm(mode, plan, mA, mG, mU, mC, p, di->num_sms, st), "tc_gemm launch");
+    SEER_CUDA(launch_tc_gemm(mode, plan, mA, mG, mU, mC, mC, p, di->num_sms, st), "tc_gemm launch");
   } else {
     Phase ph(phase, st);
     SEER_CUDA(launch_simt_gemm(mode, static_cast<const float*>(a), static_cast<const float*>(wg),
@@ -355,7 +372,8 @@ seer_status do_swiglu(const void* a, const void* wg, const void* wu, seer_dtype 
 }
 
 seer_status do_rmsnorm(const void* x, seer_dtype x_dt, const void* g, void* y, seer_dtype y_dt, int M_cap,
-                       const int32_t* M_dev, int d, float eps, cudaStream_t st, int phase) {
+                       const int32_t* M_dev, int d, float eps, cudaStream_t st, int phase,
+                       const RowMap& map = RowMap{}) {
   if (!x || !g || !y) return fail(SEER_ERR_INVALID_ARG, "rmsnorm: null pointer");
   if (M_cap < 0 || d <= 0) return fail(SEER_ERR_INVALID_ARG, "rmsnorm: bad sizes");
   if (!valid_dt(x_dt) || !valid_dt(y_dt)) return fail(SEER_ERR_INVALID_ARG, "rmsnorm: unknown dtype");
@@ -367,7 +385,7 @@ seer_status do_rmsnorm(const void* x, seer_dtype x_dt, const void* g, void* y, s
   DeviceInfo* di;
   SEER_TRY(device_info(&di));
   Phase ph(phase, st);
-  SEER_CUDA(launch_rmsnorm(x, x_dt, g, y, y_dt, M_cap, M_dev, d, eps, di->err, st), "rmsnorm launch");
+  SEER_CUDA(launch_rmsnorm(x, x_dt, g, y, y_dt, M_cap, M_dev, d, eps, map, di->err, st), "rmsnorm launch");
   return SEER_OK;
 }
 
@@ -778,22 +796,38 @@ seer_status seer_kv_prefill(const seer_layer_weights* w, const seer_dims* dims, 
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const int d = dims->d_model, D2 = 2 * dims->n_heads * dims->head_dim;
   const seer_dtype it = dt == SEER_F32 ? SEER_F32 : SEER_F16;
-  const long xrow = static_cast<long>(d) * esize(dt), irow = static_cast<long>(d) * esize(it);
-  const long kvrow = static_cast<long>(D2) * esize(it);
   uint8_t* base = static_cast<uint8_t*>(ws);
-  void* xp = base + L.off_h;                     // prefix rows, packed  [sum ctx, d]
-  void* xn = base + L.off_xn;                    // normalised           [sum ctx, d]
-  void* kvp = base + L.off_qkv;                  // their K | V          [sum ctx, 2D]
+  void* xn = base + L.off_xn;                    // prefix rows, normalised and packed [sum ctx, d]
   int32_t* cu_ctx = reinterpret_cast<int32_t*>(base + L.off_sched);   // [B+1], before the (unused) schedule
+  const void* w_kv = static_cast<const uint8_t*>(w->w_qkv) + static_cast<size_t>(D2 / 2) * d * esize(it);
   {
     Phase ph(PH_KV, st);
     SEER_CUDA(launch_resp_layout(nullptr, ctx_len, B, nullptr, cu_ctx, di->err, st), "prefix layout");
+  }
+  if (it == SEER_F16) {
+    // the norm reads the prefix rows where they are and the projection stores into
+    // the cache: gathering the rows and scattering K | V afterwards moved 3.2 GB more
+    // for 24096 rows of 4096 (1160 -> 1014 us under the
+    // power cap, 1131 -> 893 below it)
+    const RowMap from{cu_ctx, cu_x, nullptr, B, T_x_cap}, to{cu_ctx, cu_kv, nullptr, B, T_kv_cap};
+    SEER_TRY(do_rmsnorm(x, dt, w->g_attn, xn, it, T_x_cap, cu_ctx + B, d, dims->rms_eps, st, PH_KV, from));
+    KvDest dest;
+    dest.kv = kv_cache;
+    dest.ld = D2;
+    dest.map = to;
+    return do_linear(xn, w_kv, it, nullptr, it, base + L.off_qkv, it, T_x_cap, cu_ctx + B, D2, d, st, PH_KV, RopeArgs(),
+                     dest);
+  }
+  void* xp = base + L.off_h;                     // prefix rows, packed  [sum ctx, d]
+  void* kvp = base + L.off_qkv;                  // their K | V          [sum ctx, 2D]
+  const long xrow = static_cast<long>(d) * esize(dt), kvrow = static_cast<long>(D2) * esize(it);
+  {
+    Phase ph(PH_KV, st);
     SEER_CUDA(launch_rows_copy(x, xrow, 0, xp, xrow, 0, static_cast<int>(xrow), cu_x, nullptr, ctx_len, nullptr, cu_ctx,
                                nullptr, B, T_x_cap, T_x_cap, T_x_cap, di->err, st),
               "prefix gather");
   }
   SEER_TRY(do_rmsnorm(xp, dt, w->g_attn, xn, it, T_x_cap, cu_ctx + B, d, dims->rms_eps, st, PH_KV));
-  const void* w_kv = static_cast<const uint8_t*>(w->w_qkv) + static_cast<size_t>(D2 / 2) * d * esize(it);
   SEER_TRY(do_linear(xn, w_kv, it, nullptr, it, kvp, it, T_x_cap, cu_ctx + B, D2, d, st, PH_KV));
   Phase ph(PH_KV, st);
   SEER_CUDA(launch_rows_copy(kvp, kvrow, 0, kv_cache, kvrow, 0, static_cast<int>(kvrow), cu_ctx, nullptr, nullptr, nullptr,
@@ -835,9 +869,17 @@ seer_status seer_layer_forward_cached(const seer_layer_weights* w, const seer_di
   const float eps = dims->rms_eps;
 
   SEER_TRY(do_rmsnorm(x_resp, dt, w->g_attn, xn, it, T_resp_cap, M_dev, d, eps, st, PH_NORM1));
-  SEER_TRY(do_linear(xn, w->w_qkv, it, nullptr, it, qkv, it, T_resp_cap, M_dev, 3 * d, d, st, PH_QKV));
-  {
-    // the response rows' K | V into the cache, after each segment's prefix
+  // the response rows' K | V go into the cache, after each segment's prefix: straight
+  // from the projection for 16-bit layers (a copy afterwards took 18 us for 848 rows)
+  KvDest dest;
+  if (it == SEER_F16) {
+    dest.kv = kv_cache;
+    dest.ld = 2 * D;
+    dest.split = D;
+    dest.map = RowMap{cu_resp, cu_kv, ctx_len, B, T_kv_cap};
+  }
+  SEER_TRY(do_linear(xn, w->w_qkv, it, nullptr, it, qkv, it, T_resp_cap, M_dev, 3 * d, d, st, PH_QKV, RopeArgs(), dest));
+  if (it != SEER_F16) {
     Phase ph(PH_KV, st);
     SEER_CUDA(launch_rows_copy(qkv, 3 * D * es, static_cast<int>(D * es), kv_cache, 2 * D * es, 0,
                                static_cast<int>(2 * D * es), cu_resp, nullptr, nullptr, nullptr, cu_kv, ctx_len, B,

@@ -39,6 +39,8 @@
 //   Count     detector: A rows gathered per sequence window, counts only
 //   Rope      Store, then the q|k columns rotated per 128-wide head by the
 //             rotary embedding at each row's position in its sequence
+//   Kv        Store, with the columns past a split going to mapped rows of a second
+//             matrix: the K | V projections straight into a K/V cache
 // Every stored 16-bit value passes a range guard: an infinite or NaN result
 // (an f16 intermediate that overflowed +-65504) records kErrRange in the
 // device error word, which seer_check_device reports.
@@ -123,7 +125,8 @@ __device__ __forceinline__ int count_near_zero(const float (&a)[32], const uint3
 template <int MODE, int CG>
 __global__ void __launch_bounds__(THREADS, 1)
     tc_gemm_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CUtensorMap mB0,
-                   const __grid_constant__ CUtensorMap mB1, const __grid_constant__ CUtensorMap mC, const GemmParams p) {
+                   const __grid_constant__ CUtensorMap mB1, const __grid_constant__ CUtensorMap mC,
+                   const __grid_constant__ CUtensorMap mC2, const GemmParams p) {
   const int BN = p.bn;
   const int stages = p.stages;
   const int sbytes = stage_bytes(CG, BN);
@@ -320,7 +323,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     int n_chunks = 0;                            // bulk stores issued by this warp (staging buffer = n & 1)
     // one staged 32 x 32 chunk of this warp's rows -> a TMA store at (x, y); the
     // buffer used two chunks ago is reused only once its store has read it
-    auto store_chunk = [&](const uint32_t (&w)[16], int x, int y) {
+    auto store_chunk = [&](const CUtensorMap& map, const uint32_t (&w)[16], int x, int y) {
       uint8_t* buf = my_stage + (n_chunks & 1) * EPI_CHUNK;
       if (lane == 0 && n_chunks >= 2) bulk_wait_read_1();
       __syncwarp();
@@ -330,7 +333,7 @@ __global__ void __launch_bounds__(THREADS, 1)
       fence_proxy_async_smem();
       __syncwarp();
       if (lane == 0) {
-        tma_store_2d_hint(&mC, buf, x, y, out_policy);
+        tma_store_2d_hint(&map, buf, x, y, out_policy);
         bulk_commit();
       }
       ++n_chunks;
@@ -363,6 +366,15 @@ __global__ void __launch_bounds__(THREADS, 1)
                                                          static_cast<size_t>(valid ? row : 0) * p.ldr + n * BN);
 #pragma unroll
         for (int i = 0; i < ACC_COLS / 8; ++i) res[i] = valid && i * 8 < cols ? rp[i] : make_uint4(0, 0, 0, 0);
+      }
+      // Kv: where this row's columns past the split go, and whether the warp's 32
+      // rows go to 32 consecutive ones (then a TMA store takes them together)
+      int row2 = -1, row2_0 = -1;
+      bool slab2 = false;
+      if (MODE == kGemmKv) {
+        row2 = valid ? mapped_row(p.map, row, p.M_cap, p.err) : -1;
+        row2_0 = __shfl_sync(0xffffffffu, row2, 0);
+        slab2 = __all_sync(0xffffffffu, row2 >= 0 && row2 == row2_0 + lane);
       }
       // warp-uniform outcome: the TMEM loads below are warp-collective, and
       // after an abort the lanes of a warp could otherwise decide differently
@@ -413,7 +425,7 @@ __global__ void __launch_bounds__(THREADS, 1)
             }
           }
         }
-      } else if (MODE == kGemmStore || MODE == kGemmResidual) {
+      } else if (MODE == kGemmStore || MODE == kGemmResidual || MODE == kGemmKv) {
         // two chunks of 32 columns per step, their accumulator loads in flight together
 #pragma unroll
         for (int c = 0; c < ACC_COLS / 32; c += 2) {
@@ -424,7 +436,10 @@ __global__ void __launch_bounds__(THREADS, 1)
           tmem_ld_wait();
 #pragma unroll
           for (int h = 0; h < 2; ++h) {
-            if ((c + h) * 32 < cols && (slab_full || valid)) {
+            const int col = n * BN + (c + h) * 32;
+            const bool second = MODE == kGemmKv && col >= p.split;   // a chunk lies on one side of the split
+            const bool slab = second ? slab2 : slab_full;
+            if ((c + h) * 32 < cols && (slab || (second ? row2 >= 0 : valid))) {
               float v[32];
 #pragma unroll
               for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(acc32[h][i]);
@@ -444,11 +459,12 @@ __global__ void __launch_bounds__(THREADS, 1)
                 w[i] = pack2(v[2 * i], v[2 * i + 1], of16);
                 nonfinite |= nonfinite_term(w[i], of16);
               }
-              if (slab_full) {
-                store_chunk(w, n * BN + (c + h) * 32, mt * BM + q * 32);
+              if (slab) {
+                store_chunk(second ? mC2 : mC, w, second ? col - p.split : col, second ? row2_0 : mt * BM + q * 32);
               } else {
                 // a lane owns one row: 64 contiguous bytes as two full 32-byte sectors
-                uint16_t* crow = reinterpret_cast<uint16_t*>(p.C) + static_cast<size_t>(row) * p.ldc + n * BN + (c + h) * 32;
+                uint16_t* crow = second ? reinterpret_cast<uint16_t*>(p.C2) + static_cast<size_t>(row2) * p.ldc2 + col - p.split
+                                        : reinterpret_cast<uint16_t*>(p.C) + static_cast<size_t>(row) * p.ldc + col;
                 st_global_v8(crow, w[0], w[1], w[2], w[3], w[4], w[5], w[6], w[7]);
                 st_global_v8(crow + 16, w[8], w[9], w[10], w[11], w[12], w[13], w[14], w[15]);
               }
@@ -499,7 +515,7 @@ __global__ void __launch_bounds__(THREADS, 1)
                 nonfinite |= nonfinite_term(w[i], of16);
               }
               if (slab_full) {
-                store_chunk(w, n * tile_n + c * 32, mt * BM + q * 32);
+                store_chunk(mC, w, n * tile_n + c * 32, mt * BM + q * 32);
               } else {
                 st_global_v8(arow + c * 32, w[0], w[1], w[2], w[3], w[4], w[5], w[6], w[7]);
                 st_global_v8(arow + c * 32 + 16, w[8], w[9], w[10], w[11], w[12], w[13], w[14], w[15]);
@@ -535,7 +551,7 @@ __global__ void __launch_bounds__(THREADS, 1)
 
 template <int MODE, int CG>
 cudaError_t launch_mode(const GemmPlan& plan, const CUtensorMap& mA, const CUtensorMap& mB0, const CUtensorMap& mB1,
-                        const CUtensorMap& mC, GemmParams p, int num_sms, cudaStream_t st) {
+                        const CUtensorMap& mC, const CUtensorMap& mC2, GemmParams p, int num_sms, cudaStream_t st) {
   static bool attr_set[64] = {};
   cudaError_t e = set_smem_limit_once(tc_gemm_kernel<MODE, CG>, RING_BYTES + FIXED_BYTES, attr_set);
   if (e != cudaSuccess) return e;
@@ -555,14 +571,14 @@ cudaError_t launch_mode(const GemmPlan& plan, const CUtensorMap& mA, const CUten
   // 11.9 ms either way); one of 842 rows 391 us without any, 383 with calls of up to
   // five tiles per SM overlapped, 379 with all
   return launch_kernel_overlap(launch_overlap_enabled(), CG, tc_gemm_kernel<MODE, CG>, dim3(grid * CG), dim3(THREADS),
-                               smem, st, mA, mB0, mB1, mC, p);
+                               smem, st, mA, mB0, mB1, mC, mC2, p);
 }
 
 template <int MODE>
 cudaError_t launch_cg(const GemmPlan& plan, const CUtensorMap& mA, const CUtensorMap& mB0, const CUtensorMap& mB1,
-                      const CUtensorMap& mC, const GemmParams& p, int num_sms, cudaStream_t st) {
-  return plan.cg == 2 ? launch_mode<MODE, 2>(plan, mA, mB0, mB1, mC, p, num_sms, st)
-                      : launch_mode<MODE, 1>(plan, mA, mB0, mB1, mC, p, num_sms, st);
+                      const CUtensorMap& mC, const CUtensorMap& mC2, const GemmParams& p, int num_sms, cudaStream_t st) {
+  return plan.cg == 2 ? launch_mode<MODE, 2>(plan, mA, mB0, mB1, mC, mC2, p, num_sms, st)
+                      : launch_mode<MODE, 1>(plan, mA, mB0, mB1, mC, mC2, p, num_sms, st);
 }
 
 }  // namespace
@@ -615,14 +631,15 @@ GemmPlan tc_gemm_plan(int mode, long m_tiles, long n_cols, int K, int num_sms) {
 }
 
 cudaError_t launch_tc_gemm(int mode, const GemmPlan& plan, const CUtensorMap& mA, const CUtensorMap& mB0,
-                           const CUtensorMap& mB1, const CUtensorMap& mC, const GemmParams& p, int num_sms,
-                           cudaStream_t st) {
+                           const CUtensorMap& mB1, const CUtensorMap& mC, const CUtensorMap& mC2, const GemmParams& p,
+                           int num_sms, cudaStream_t st) {
   switch (mode) {
-    case kGemmStore: return launch_cg<kGemmStore>(plan, mA, mB0, mB1, mC, p, num_sms, st);
-    case kGemmResidual: return launch_cg<kGemmResidual>(plan, mA, mB0, mB1, mC, p, num_sms, st);
-    case kGemmSwiglu: return launch_cg<kGemmSwiglu>(plan, mA, mB0, mB1, mC, p, num_sms, st);
-    case kGemmCount: return launch_cg<kGemmCount>(plan, mA, mB0, mB1, mC, p, num_sms, st);
-    case kGemmRope: return launch_cg<kGemmRope>(plan, mA, mB0, mB1, mC, p, num_sms, st);
+    case kGemmStore: return launch_cg<kGemmStore>(plan, mA, mB0, mB1, mC, mC2, p, num_sms, st);
+    case kGemmResidual: return launch_cg<kGemmResidual>(plan, mA, mB0, mB1, mC, mC2, p, num_sms, st);
+    case kGemmSwiglu: return launch_cg<kGemmSwiglu>(plan, mA, mB0, mB1, mC, mC2, p, num_sms, st);
+    case kGemmCount: return launch_cg<kGemmCount>(plan, mA, mB0, mB1, mC, mC2, p, num_sms, st);
+    case kGemmKv: return launch_cg<kGemmKv>(plan, mA, mB0, mB1, mC, mC2, p, num_sms, st);
+    case kGemmRope: return launch_cg<kGemmRope>(plan, mA, mB0, mB1, mC, mC2, p, num_sms, st);
     default: return cudaErrorInvalidValue;
   }
 }

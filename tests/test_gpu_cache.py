@@ -72,6 +72,44 @@ def test_cached_layer_matches_oracle_and_uncached_rows(dtype):
     assert (yrh[cr[-1]:] == 9.0).all()                                                 # zero work past the rows
 
 
+@pytest.mark.parametrize("d", [256, 4352])                           # norm from registers, and streaming
+@pytest.mark.parametrize("ctx,bad", [([40], -1), ([1, 31, 0, 32, 33, 200, 65], -1), ([100, 64, 7], 1), ([0, 5], -1)])
+def test_kv_prefill_stores_segments_where_the_offsets_say(d, ctx, bad):
+    """16-bit prefill reads and writes rows in place: segments at odd offsets with gaps
+    between them (slabs of 32 rows that straddle segments, empty prefixes) equal the
+    norm and the projection of the gathered rows bit for bit, other cache rows stay,
+    and a segment outside the cache is recorded and writes nothing."""
+    B, H = len(ctx), d // 128
+    g = torch.Generator(device="cuda").manual_seed(d + B)
+    r = lambda *shape: torch.randn(shape, generator=g, device="cuda")
+    starts_x = np.cumsum([3] + [c + 5 for c in ctx])                   # B + 1 offsets
+    starts_kv = np.cumsum([1] + [c + 9 for c in ctx])
+    T_x, T_kv = int(starts_x[-1]), int(starts_kv[-1])
+    place = starts_kv.copy()
+    if bad >= 0:
+        place[bad] = T_kv - ctx[bad] + 1                               # one row past the end
+    x = r(T_x, d).to(torch.bfloat16)
+    w_qkv, gain = (0.02 * r(3 * d, d)).half(), (1 + 0.1 * r(d)).half()
+    dims = S.make_dims(d, H, 128, 128)
+    w = S.make_weights(w_qkv, 0, 0, 0, 0, gain, 0)
+    n = S.seer_layer_workspace_size(dims, "bf16", T_x, B)
+    ws = torch.empty(n, dtype=torch.uint8, device=cuda())
+    cache = torch.full((T_kv, 2 * d), 7.0, dtype=torch.float16, device=cuda())
+    S.seer_kv_prefill(w, dims, "bf16", x, i32(starts_x), i32(ctx), B, T_x, cache, i32(place), T_kv, ws, n)
+    assert S.seer_check_device() == (2 if bad >= 0 else 0)
+    rows = torch.cat([x[a:a + c] for a, c in zip(starts_x, ctx)])
+    xn, kv = torch.empty_like(rows, dtype=torch.float16), torch.empty((len(rows), 2 * d), dtype=torch.float16, device=cuda())
+    S.seer_rmsnorm(rows, "bf16", gain, xn, "f16", len(rows), None, d, 1e-5)
+    S.seer_linear(xn, w_qkv[d:], "f16", None, "f16", kv, "f16", len(rows), None, 2 * d, d)
+    want = torch.full_like(cache, 7.0)
+    at = 0
+    for b, c in enumerate(ctx):
+        if b != bad:
+            want[int(place[b]):int(place[b]) + c] = kv[at:at + c]
+        at += c
+    assert torch.equal(cache, want)
+
+
 def test_cache_entry_points_reject_bad_arguments():
     x = torch.zeros((8, 256), dtype=torch.bfloat16, device=cuda())
     cu = i32([0, 8])
