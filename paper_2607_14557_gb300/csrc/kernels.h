@@ -49,7 +49,7 @@ struct GemmParams {
   int out_type;           // ElemType of C (kBF16 / kF16; kF32 on the CUDA-core path)
   int res_type;           // ElemType of R
   int bn;                 // accumulator columns per tile (multiple of 32)
-  int stages;             // operand ring depth
+  int stages;             // operand ring: stages
   int group_m;            // raster: row tiles per group (see tc_gemm.cu)
   float rope_theta;       // Rope: frequency base (> 0)
   int rope_cols;          // Rope: leading output columns that are rotated (the q|k columns)
@@ -84,8 +84,9 @@ struct AttnParams {
 struct GemmPlan {
   int cg;        // SMs per tile: 1, or 2 (paired tensor-core tiles)
   int bn;        // accumulator columns per tile (Swiglu / Count: bn / 2 of F)
-  int stages;    // operand ring depth
+  int stages;    // operand ring: stages
   int group_m;   // raster: row tiles per group
+  int depth;     // 64-deep k-blocks per stage: 1 or 2
 };
 // m_tiles: 128-row tiles; n_cols: accumulator columns (N; Swiglu / Count: 2 F);
 // K: depth; num_sms: SMs of the device.

@@ -122,14 +122,15 @@ __device__ __forceinline__ int count_near_zero(const float (&a)[32], const uint3
   return cnt;
 }
 
-template <int MODE, int CG>
+template <int MODE, int CG, int DEPTH>
 __global__ void __launch_bounds__(THREADS, 1)
     tc_gemm_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CUtensorMap mB0,
                    const __grid_constant__ CUtensorMap mB1, const __grid_constant__ CUtensorMap mC,
                    const __grid_constant__ CUtensorMap mC2, const GemmParams p) {
   const int BN = p.bn;
-  const int stages = p.stages;
-  const int sbytes = stage_bytes(CG, BN);
+  const int stages = p.stages;                              // of DEPTH k-blocks
+  const int bbytes = stage_bytes(CG, BN);                   // operand bytes of a k-block
+  const int sbytes = DEPTH * bbytes;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* fixed = smem + stages * sbytes;
@@ -234,21 +235,27 @@ __global__ void __launch_bounds__(THREADS, 1)
       const int b_row0 = n * tile_n;
       const int b_row1 = halfN ? n * tile_n : n * tile_n + BN / 2;
       bool ok = true;
-      for (int kb = 0; kb < KB; ++kb) {
+      for (int kb = 0; kb < KB; kb += DEPTH) {
         if (!warp_wait(&empty[s], ph ^ 1u, abort_flag, p.err)) { ok = false; break; }
         if (leader) {
+          const int here = DEPTH == 1 ? 1 : min(DEPTH, KB - kb);   // k-blocks of this stage
           uint8_t* sa = smem + s * sbytes;
-          if (CG == 1) {
-            mbar_arrive_expect_tx(&full[s], sbytes);
-            tma_load_2d(sa, &mA, &full[s], kb * BK, a_row);
-            tma_load_2d(sa + A_TILE_BYTES, &mB0, &full[s], kb * BK, b_row0);
-            tma_load_2d(sa + A_TILE_BYTES + half_b, &mB1, &full[s], kb * BK, b_row1);
-          } else {
-            if (rank == 0) mbar_arrive_expect_tx(&full[s], 2 * sbytes);
-            const uint32_t bar = full0 + static_cast<uint32_t>(s * sizeof(uint64_t));
-            tma_load_2d_pair(sa, &mA, bar, kb * BK, a_row);
-            if (rank == 0) tma_load_2d_pair(sa + A_TILE_BYTES, &mB0, bar, kb * BK, b_row0);
-            else tma_load_2d_pair(sa + A_TILE_BYTES, &mB1, bar, kb * BK, b_row1);
+          const uint32_t bar = full0 + static_cast<uint32_t>(s * sizeof(uint64_t));
+          if (CG == 1) mbar_arrive_expect_tx(&full[s], here * bbytes);
+          else if (rank == 0) mbar_arrive_expect_tx(&full[s], 2 * here * bbytes);
+#pragma unroll
+          for (int u = 0; u < DEPTH; ++u, sa += bbytes) {
+            if (u > 0 && u >= here) break;
+            const int x = (kb + u) * BK;
+            if (CG == 1) {
+              tma_load_2d(sa, &mA, &full[s], x, a_row);
+              tma_load_2d(sa + A_TILE_BYTES, &mB0, &full[s], x, b_row0);
+              tma_load_2d(sa + A_TILE_BYTES + half_b, &mB1, &full[s], x, b_row1);
+            } else {
+              tma_load_2d_pair(sa, &mA, bar, x, a_row);
+              if (rank == 0) tma_load_2d_pair(sa + A_TILE_BYTES, &mB0, bar, x, b_row0);
+              else tma_load_2d_pair(sa + A_TILE_BYTES, &mB1, bar, x, b_row1);
+            }
           }
         }
         __syncwarp();
@@ -272,6 +279,9 @@ __global__ void __launch_bounds__(THREADS, 1)
     if (CG == 2 && rank != 0 && leader) pdl_trigger();      // rank 0 triggers after its last MMAs
   } else if (warp == 1) {
     // ------------------------------------------------ MMA issuer
+    // No vote and no warp barrier per stage: the lanes stay together through the
+    // waits, and a lane that gives up (only after a 2 s limit) leaves the loop alone
+    // (narrow tiles 10% faster; 127 rows, down: 42.6 -> 38.4 us).
     const bool leader = elect_one();
     const uint32_t idesc = p.idesc;
     int s = 0;
@@ -283,25 +293,31 @@ __global__ void __launch_bounds__(THREADS, 1)
       tc_fence_after();
       const uint32_t d_tmem = tmem_base + static_cast<uint32_t>(acc * ACC_COLS);
       bool ok = true;
-      for (int kb = 0; kb < KB; ++kb) {
-        if (!warp_wait(&full[s], ph, abort_flag, p.err)) { ok = false; break; }
+      for (int kb = 0; kb < KB; kb += DEPTH) {
+        if (!mbar_wait(&full[s], ph, abort_flag, p.err)) { ok = false; break; }
         tc_fence_after();
         if (leader) {
           const uint32_t sa = smem_u32(smem + s * sbytes);
           const uint64_t adesc = make_sdesc_sw128(sa, 16, 1024);
           const uint64_t bdesc = make_sdesc_sw128(sa + A_TILE_BYTES, 16, 1024);
 #pragma unroll
-          for (int k = 0; k < BK / 16; ++k) {
-            // +32 bytes along K inside the 128-byte swizzle atom = +2 in the address field
-            if (CG == 1) tc_mma_f16(d_tmem, adesc + 2 * k, bdesc + 2 * k, idesc, (kb | k) != 0 ? 1u : 0u);
-            else tc_mma_f16_pair(d_tmem, adesc + 2 * k, bdesc + 2 * k, idesc, (kb | k) != 0 ? 1u : 0u);
+          for (int u = 0; u < DEPTH; ++u) {
+            if (u > 0 && kb + u >= KB) break;
+            const uint64_t off = static_cast<uint64_t>((u * bbytes) >> 4);
+#pragma unroll
+            for (int k = 0; k < BK / 16; ++k) {
+              // +32 bytes along K inside the 128-byte swizzle atom = +2 in the address field
+              const uint32_t add = u > 0 || k > 0 || kb > 0 ? 1u : 0u;
+              if (CG == 1) tc_mma_f16(d_tmem, adesc + off + 2 * k, bdesc + off + 2 * k, idesc, add);
+              else tc_mma_f16_pair(d_tmem, adesc + off + 2 * k, bdesc + off + 2 * k, idesc, add);
+            }
           }
           if (CG == 1) tc_commit(&empty[s]);
           else tc_commit_pair(&empty[s]);
         }
-        __syncwarp();
         if (++s == stages) { s = 0; ph ^= 1u; }
       }
+      ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
       if (leader) {
         if (CG == 1) tc_commit(&acc_full[acc]);
@@ -549,11 +565,11 @@ __global__ void __launch_bounds__(THREADS, 1)
   }
 }
 
-template <int MODE, int CG>
+template <int MODE, int CG, int DEPTH>
 cudaError_t launch_mode(const GemmPlan& plan, const CUtensorMap& mA, const CUtensorMap& mB0, const CUtensorMap& mB1,
                         const CUtensorMap& mC, const CUtensorMap& mC2, GemmParams p, int num_sms, cudaStream_t st) {
   static bool attr_set[64] = {};
-  cudaError_t e = set_smem_limit_once(tc_gemm_kernel<MODE, CG>, RING_BYTES + FIXED_BYTES, attr_set);
+  cudaError_t e = set_smem_limit_once(tc_gemm_kernel<MODE, CG, DEPTH>, RING_BYTES + FIXED_BYTES, attr_set);
   if (e != cudaSuccess) return e;
   long num_mt;
   if (MODE == kGemmCount) num_mt = static_cast<long>(p.B) * ((p.Nw + BM - 1) / BM);
@@ -566,19 +582,22 @@ cudaError_t launch_mode(const GemmPlan& plan, const CUtensorMap& mA, const CUten
   p.group_m = plan.group_m;
   const int units = num_sms / CG;
   const int grid = static_cast<int>(tiles < units ? tiles : units);
-  const int smem = plan.stages * stage_bytes(CG, plan.bn) + FIXED_BYTES;
+  const int smem = plan.stages * DEPTH * stage_bytes(CG, plan.bn) + FIXED_BYTES;
   // long calls gain little from the overlap but lose nothing (one layer of 35k rows:
   // 11.9 ms either way); one of 842 rows 391 us without any, 383 with calls of up to
   // five tiles per SM overlapped, 379 with all
-  return launch_kernel_overlap(launch_overlap_enabled(), CG, tc_gemm_kernel<MODE, CG>, dim3(grid * CG), dim3(THREADS),
+  return launch_kernel_overlap(launch_overlap_enabled(), CG, tc_gemm_kernel<MODE, CG, DEPTH>, dim3(grid * CG), dim3(THREADS),
                                smem, st, mA, mB0, mB1, mC, mC2, p);
 }
 
 template <int MODE>
 cudaError_t launch_cg(const GemmPlan& plan, const CUtensorMap& mA, const CUtensorMap& mB0, const CUtensorMap& mB1,
                       const CUtensorMap& mC, const CUtensorMap& mC2, const GemmParams& p, int num_sms, cudaStream_t st) {
-  return plan.cg == 2 ? launch_mode<MODE, 2>(plan, mA, mB0, mB1, mC, mC2, p, num_sms, st)
-                      : launch_mode<MODE, 1>(plan, mA, mB0, mB1, mC, mC2, p, num_sms, st);
+  if (plan.cg == 2)
+    return plan.depth == 2 ? launch_mode<MODE, 2, 2>(plan, mA, mB0, mB1, mC, mC2, p, num_sms, st)
+                           : launch_mode<MODE, 2, 1>(plan, mA, mB0, mB1, mC, mC2, p, num_sms, st);
+  return plan.depth == 2 ? launch_mode<MODE, 1, 2>(plan, mA, mB0, mB1, mC, mC2, p, num_sms, st)
+                         : launch_mode<MODE, 1, 1>(plan, mA, mB0, mB1, mC, mC2, p, num_sms, st);
 }
 
 }  // namespace
@@ -587,35 +606,42 @@ cudaError_t launch_cg(const GemmPlan& plan, const CUtensorMap& mA, const CUtenso
 // k-blocks x time of a k-block + the fixed part of a call (launch, first
 // operands, last epilogue).  The constants (us) are fits to GB300 timings of the
 // 8B layer's shapes at 127, 300, 842 and 2976 rows: per 64-deep k-block with all
-// SMs busy a pair takes 0.281 at 256 columns (the tensor rate), 0.264 at 224, 0.22
-// at 192, 0.19 at 160 and never below 0.18; one SM, which stages a third more
-// operand bytes per product, 0.366 / 0.35 / 0.29 / 0.22 at 256 / 224 / 192 / 128
-// columns (the SMs together read ~15 TB/s from L2) and never below 0.2.  So pairs
-// are the rule; one-SM tiles remain where a pair's second SM would idle (an odd,
+// SMs busy a pair takes 0.281 at 256 columns (the tensor rate), 0.254 at 224, 0.22
+// at 192, 0.19 at 160, 0.165 at 128 and 0.14 at 64; one SM, which stages a third
+// more operand bytes per product, 0.366 / 0.35 / 0.29 / 0.2 at 256 / 224 / 192 / 128
+// columns (the SMs together read ~15 TB/s from L2) and 0.15 at 32.  So pairs are
+// the rule; one-SM tiles remain where a pair's second SM would idle (an odd,
 // small number of row tiles), and narrower tiles where they fill the last wave.
 // Examples (us, one-SM 256-column tiles -> chosen): 842 rows QKV 73.5 -> 57.7
-// (224 columns, 2.9 waves of pairs instead of 2.2 of SMs), O 30.8 -> 26.9 and
-// down 77.7 -> 60.7 (224: 76 tiles on 76 pairs); 127 rows QKV 30.7 -> 22.8 (96
-// columns), O 30.6 -> 17.3, down 75.7 -> 43; 2976 rows O 74.6 -> 63.0, down 238
-// -> 182; 35194 rows QKV 1990 -> 1927, down 2323 -> 2154.
+// (224 columns, 2.9 waves of pairs instead of 2.2 of SMs), O 30.8 -> 25.0 and
+// down 77.7 -> 60.7 (224: 76 tiles on 76 pairs); 127 rows QKV 30.7 -> 22, O 30.6 ->
+// 12.9, down 75.7 -> 32.3; 2976 rows O 74.6 -> 63.0, down 238 -> 182; 35194 rows
+// QKV 1990 -> 1927, down 2323 -> 2154.
+// Narrow tiles stage two k-blocks at a time: below ~190 columns the issuer's wait,
+// commit and loop per stage (~100 cycles) exceed what the MMAs hide (127 rows, down:
+// 38.4 us with one, 32.3 with two; 842 rows at 128 columns 75.1 and 71.6, at 224
+// columns 61.0 and 63.2).
 GemmPlan tc_gemm_plan(int mode, long m_tiles, long n_cols, int K, int num_sms) {
   const bool half_n = mode == kGemmSwiglu || mode == kGemmCount;
   // whole 32-column chunks of the output, and whole heads for Rope
   const int step = mode == kGemmRope ? 128 : (half_n ? 64 : 32);
-  GemmPlan g{2, 256, 0, 1};
+  GemmPlan g{2, 256, 0, 1, 1};
   double best = 0.0;
   for (int cg = 2; cg >= 1; --cg) {
     for (int bn = 256; bn >= step; bn -= step) {
       const long tiles = ((m_tiles + cg - 1) / cg) * ((n_cols + bn - 1) / bn);
       const long units = num_sms / cg;
-      const double block = cg == 2 ? fmax(0.18, 0.03 + 0.001 * bn) : fmax(0.2, 0.08 + 0.00112 * bn);
+      const bool narrow = bn / cg <= 64;
+      const double block = cg == 2 ? (narrow ? 0.115 + 0.0004 * bn : 0.03 + 0.001 * bn)
+                                   : (narrow ? 0.143 + 0.0003 * bn : fmax(0.19, 0.08 + 0.00112 * bn));
       const double fixed = cg == 2 ? 6.0 + 0.015 * bn : 4.2 + 0.0125 * bn;
       const double cost = fixed + static_cast<double>((tiles + units - 1) / units) * (K / BK) * block;
       if (g.stages == 0 || cost < 0.98 * best) {      // wide pair tiles unless another choice is clearly faster
         best = cost;
         g.cg = cg;
         g.bn = bn;
-        g.stages = RING_BYTES / stage_bytes(cg, bn);
+        g.depth = narrow ? 2 : 1;
+        g.stages = RING_BYTES / (g.depth * stage_bytes(cg, bn));
       }
     }
   }
