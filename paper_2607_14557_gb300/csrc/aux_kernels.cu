@@ -105,8 +105,9 @@ __global__ void __launch_bounds__(256) rmsnorm_kernel(const void* __restrict__ x
 // loads in flight (35194 x 4096 rows: 6.36 TB/s, against 5.4 for the
 // two-pass streaming kernel and 4.9 at one block per SM).  The gain vector g,
 // the same for every row, is staged once per block in shared memory (8 KB at
-// d = 4096); read from global memory per row, its loads were hoisted beside
-// the row's 64 registers and spilled.
+// d = 4096) while the block's first rows are in flight (9973 rows: 29.9 -> 27.9 us
+// against staging it first); read from global memory per row, its loads were
+// hoisted beside the row's 64 registers and spilled.
 template <int IN, int OUT, int VPL, bool MAP>
 __global__ void __launch_bounds__(256, 2) rmsnorm_rows_kernel(const void* __restrict__ x, const void* __restrict__ g,
                                                            void* __restrict__ y, int M_cap, const int* M_dev, int d,
@@ -127,20 +128,25 @@ __global__ void __launch_bounds__(256, 2) rmsnorm_rows_kernel(const void* __rest
   const int d8 = d / 8;
   const uint4* xv = reinterpret_cast<const uint4*>(x);
   __shared__ uint4 g_sh[32 * VPL];
-  for (int v = threadIdx.x; v < d8; v += blockDim.x) g_sh[v] = __ldg(reinterpret_cast<const uint4*>(g) + v);
-  __syncthreads();
   uint4* yv = reinterpret_cast<uint4*>(y);
   uint32_t nonfinite = 0;
-  for (int row = blockIdx.x * 8 + warp; row < M; row += nwarps) {
-    const size_t base8 = static_cast<size_t>(row) * d8;
+  uint4 raw[VPL];
+  auto load_row = [&](int row) {
     const int src = MAP ? mapped_row(map, row, M_cap, err) : row;
     const size_t src8 = static_cast<size_t>(src) * d8;
-    uint4 raw[VPL];
 #pragma unroll
     for (int i = 0; i < VPL; ++i) {
       const int v = lane + 32 * i;
       raw[i] = v < d8 && src >= 0 ? __ldg(xv + src8 + v) : make_uint4(0, 0, 0, 0);
     }
+  };
+  // the first row's loads are under way while the gain is staged
+  int row = blockIdx.x * 8 + warp;
+  if (row < M) load_row(row);
+  for (int v = threadIdx.x; v < d8; v += blockDim.x) g_sh[v] = __ldg(reinterpret_cast<const uint4*>(g) + v);
+  __syncthreads();
+  while (row < M) {
+    const size_t base8 = static_cast<size_t>(row) * d8;
     // the sum of squares unpacks through an opaque copy of each word, so the
     // scaling below unpacks again instead of keeping 8 floats per vector live
     // from here (that reuse needed 128 float registers and spilled)
@@ -177,6 +183,8 @@ __global__ void __launch_bounds__(256, 2) rmsnorm_rows_kernel(const void* __rest
         yv[base8 + v] = make_uint4(o[0], o[1], o[2], o[3]);
       }
     }
+    row += nwarps;
+    if (row < M) load_row(row);
   }
   report_range(nonfinite, err);
 }
@@ -323,31 +331,41 @@ __global__ void wait_selftest_kernel(uint64_t limit_ns, int* err) {
 
 // ------------------------------------------------------------------ SNR scan
 constexpr int kScanSmemInts = 12288;   // 48 KB of staged counts per sequence at most
+constexpr int kScanThreads = 128;
 // Sec. 3.3: first 0-based i in [1, N-w] with
 //   jump  = min(s_i .. s_{i+w-1}) - s_{i-1} >= tau_jump
 //   noise = max(s_i .. s_{i+w-1}) - min(..)  <= gamma * jump,   s = c / F,
 // evaluated in IEEE fp64 with explicit round-to-nearest operations (no FMA
 // contraction) so the decision is exactly reproducible.  L* = i* + 1, or N.
-__global__ void __launch_bounds__(32) snr_scan_kernel(const int* __restrict__ counts, int N, int F, double tau_jump,
-                                                      double gamma, int window, int* __restrict__ L_star,
-                                                      int* __restrict__ i_star) {
+// A block per sequence; its threads take candidates in turn, kScanThreads at a
+// time, until one passes.  The fp64 quotients (the part has few fp64 units: three
+// per candidate paced a warp-per-sequence scan, 12 us for 512 candidates) are only
+// formed for candidates that pass the test in fp32 with slack: the exact test
+// compares (lo - prev) / F with tau_jump and (hi - lo) / F with gamma (lo - prev) / F
+// up to a few roundings of 2^-53 of s <= 1, the fp32 one the same numbers times F
+// with every rounding of its own below 2^-22 of either side; 1e-5 of the larger
+// side plus 1e-3 counts covers both.
+__global__ void __launch_bounds__(kScanThreads) snr_scan_kernel(const int* __restrict__ counts, int N, int F,
+                                                                double tau_jump, double gamma, int window,
+                                                                int* __restrict__ L_star, int* __restrict__ i_star) {
   pdl_enter();
   const int b = blockIdx.x;
-  const int lane = threadIdx.x;
   const int* c = counts + static_cast<size_t>(b) * N;
   // the sequence's counts staged in shared memory by one coalesced pass (all
   // loads in flight at once) when they fit; the scan then reads them there
   extern __shared__ int staged[];
+  __shared__ int first[kScanThreads / 32];
   if (N <= kScanSmemInts) {
-    for (int i = lane; i < N; i += 32) staged[i] = c[i];
-    __syncwarp();
+    for (int i = threadIdx.x; i < N; i += kScanThreads) staged[i] = c[i];
+    __syncthreads();
     c = staged;
   }
   const double Fd = static_cast<double>(F);
+  const float need = static_cast<float>(tau_jump * Fd), g = static_cast<float>(gamma);
   int found = -1;
   const int last = N - window;   // inclusive
-  for (int base = 1; base <= last; base += 32) {
-    const int i = base + lane;
+  for (int base = 1; base <= last; base += kScanThreads) {
+    const int i = base + static_cast<int>(threadIdx.x);
     bool hit = false;
     if (i <= last) {
       int lo = c[i], hi = c[i];
@@ -356,20 +374,31 @@ __global__ void __launch_bounds__(32) snr_scan_kernel(const int* __restrict__ co
         lo = min(lo, v);
         hi = max(hi, v);
       }
-      const double s_lo = __ddiv_rn(static_cast<double>(lo), Fd);
-      const double s_hi = __ddiv_rn(static_cast<double>(hi), Fd);
-      const double s_prev = __ddiv_rn(static_cast<double>(c[i - 1]), Fd);
-      const double jump = __dsub_rn(s_lo, s_prev);
-      const double noise = __dsub_rn(s_hi, s_lo);
-      hit = (jump >= tau_jump) && (noise <= __dmul_rn(gamma, jump));
+      const int prev = c[i - 1];
+      const float jump_f = static_cast<float>(lo) - static_cast<float>(prev);
+      const float noise_f = static_cast<float>(hi) - static_cast<float>(lo), room = g * jump_f;
+      // counts above 2^24 are rounded here: their slack is 1e-5 of the counts themselves
+      const float slack = 1e-5f * fmaxf(fabsf(static_cast<float>(hi)), fabsf(static_cast<float>(prev))) + 1e-3f;
+      const bool maybe = jump_f >= need - 1e-5f * fabsf(need) - slack && noise_f <= room + 1e-5f * fabsf(room) + slack * (1.f + fabsf(g));
+      if (maybe) {
+        const double s_lo = __ddiv_rn(static_cast<double>(lo), Fd);
+        const double s_hi = __ddiv_rn(static_cast<double>(hi), Fd);
+        const double s_prev = __ddiv_rn(static_cast<double>(prev), Fd);
+        const double jump = __dsub_rn(s_lo, s_prev);
+        const double noise = __dsub_rn(s_hi, s_lo);
+        hit = (jump >= tau_jump) && (noise <= __dmul_rn(gamma, jump));
+      }
     }
     const unsigned mask = __ballot_sync(0xffffffffu, hit);
-    if (mask) {
-      found = base + __ffs(mask) - 1;
-      break;
-    }
+    if ((threadIdx.x & 31) == 0) first[threadIdx.x >> 5] = mask ? base + static_cast<int>(threadIdx.x) + __ffs(mask) - 1 : -1;
+    __syncthreads();
+#pragma unroll
+    for (int w = kScanThreads / 32 - 1; w >= 0; --w)
+      if (first[w] >= 0) found = first[w];
+    if (found >= 0) break;                       // the same in every thread
+    __syncthreads();                             // `first` is rewritten by the next round
   }
-  if (lane == 0) {
+  if (threadIdx.x == 0) {
     L_star[b] = found >= 0 ? found + 1 : N;
     if (i_star) i_star[b] = found;
   }
@@ -382,8 +411,8 @@ struct RouteSmem {
   int count[kCtrlMaxGroups];
   long long sum[kCtrlMaxGroups];
   int path[kCtrlMaxGroups];
-  int rho_ppm[kCtrlMaxGroups];
-  int total, max_seg, pad_rows, path_mask, n_groups;
+  int words[kCtrlWords];         // the control word
+  int total, max_seg;
 };
 
 __device__ __forceinline__ int graph_capacity(int total) {
@@ -396,8 +425,11 @@ __device__ __forceinline__ int graph_capacity(int total) {
 }
 
 // Every block recomputes the (tiny) routing decision in shared memory, block 0
-// publishes it, then all blocks copy rows.  Dynamic smem: seg/cu/bucket-index
-// arrays of B+1 ints each.
+// publishes it, then all blocks copy rows.  Segments, buckets and control words are
+// each handled side by side by the block's threads: with one thread walking them (its
+// loads, fp64 quotients and the 135 words it stored to host memory) a batch of one
+// took 13 us, now 8.7; 32 segments, 77k rows of 8 KB 205.6 -> 201.5 us.  Dynamic smem: seg/cu/bucket-index arrays of
+// B+1 ints each.
 __global__ void __launch_bounds__(256, 4) pack_route_kernel(const uint8_t* __restrict__ x_full, int row_bytes,
                                                          const int* __restrict__ cu_full,
                                                          const int* __restrict__ ctx_len,
@@ -411,17 +443,32 @@ __global__ void __launch_bounds__(256, 4) pack_route_kernel(const uint8_t* __res
   int* cus = dyn + B;          // [B+1]
   int* bidx = dyn + 2 * B + 1; // [B]
   __shared__ RouteSmem rs;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
-  if (threadIdx.x == 0) {
-    int nb = 0;
-    for (int b = bucket_min; b < N && nb < kCtrlMaxGroups - 1; b *= 2) rs.bucket[nb++] = b;
-    rs.bucket[nb++] = N;
-    rs.n_buckets = nb;
-    for (int k = 0; k < nb; ++k) { rs.count[k] = 0; rs.sum[k] = 0; }
+  // this thread's first segment, its loads in flight together (further ones, past
+  // the block's width, are loaded where they are used)
+  const int mine = threadIdx.x;
+  int my_L = 0, my_ctx = 0, my_avail = 0;
+  if (mine < B) {
+    my_L = L_star[mine];
+    my_ctx = ctx_len[mine];
+    my_avail = cu_full[mine + 1] - cu_full[mine];
   }
+
+  // buckets bucket_min * 2^k below N (at most kCtrlMaxGroups - 1), then N
+  if (warp == 0) {
+    const long long size = static_cast<long long>(bucket_min) << lane;
+    const bool below = lane < kCtrlMaxGroups - 1 && size < N;
+    const int nb = __popc(__ballot_sync(0xffffffffu, below));
+    rs.bucket[lane] = lane < nb ? static_cast<int>(size) : N;
+    rs.count[lane] = 0;
+    rs.sum[lane] = 0;
+    if (lane == 0) rs.n_buckets = nb + 1;
+  }
+  for (int i = threadIdx.x; i < kCtrlWords; i += blockDim.x) rs.words[i] = 0;
   __syncthreads();
   for (int i = threadIdx.x; i < B; i += blockDim.x) {
-    int Ls = L_star[i];
+    int Ls = i == mine ? my_L : L_star[i];
     if (Ls < 1 || Ls > N) {
       if (blockIdx.x == 0) record_error(err, kErrBoundary);
       Ls = Ls < 1 ? 1 : N;
@@ -433,32 +480,44 @@ __global__ void __launch_bounds__(256, 4) pack_route_kernel(const uint8_t* __res
     atomicAdd(reinterpret_cast<unsigned long long*>(&rs.sum[k]), static_cast<unsigned long long>(Ls));
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    int mask = 0, ng = 0;
-    for (int k = 0; k < rs.n_buckets; ++k) {
-      if (rs.count[k] == 0) { rs.path[k] = -1; continue; }
+  if (warp == 0) {
+    // a lane per bucket
+    const bool used = lane < rs.n_buckets && rs.count[lane] > 0;
+    int path = -1, rho_ppm = 0;
+    if (used) {
       // Eq. 4, in fp64 exactly as written
-      const double rho = 1.0 - static_cast<double>(rs.sum[k]) / static_cast<double>(static_cast<long long>(rs.count[k]) * rs.bucket[k]);
-      int path;
-      if (rs.bucket[k] <= eager_max_bucket || rs.count[k] == 1) path = 2;
+      const double rho = 1.0 - static_cast<double>(rs.sum[lane]) /
+                                   static_cast<double>(static_cast<long long>(rs.count[lane]) * rs.bucket[lane]);
+      if (rs.bucket[lane] <= eager_max_bucket || rs.count[lane] == 1) path = 2;
       else if (rho <= tau_pad) path = 0;
       else path = 1;
-      rs.path[k] = path;
-      rs.rho_ppm[k] = static_cast<int>(floor(rho * 1e6));
-      mask |= 1 << path;
-      ++ng;
+      rho_ppm = static_cast<int>(floor(rho * 1e6));
     }
-    rs.path_mask = mask;
-    rs.n_groups = ng;
+    rs.path[lane] = path;
+    const unsigned groups = __ballot_sync(0xffffffffu, used);
+    const int mask = __reduce_or_sync(0xffffffffu, used ? 1u << path : 0u);
+    if (used) {
+      int* w = rs.words + 8 + 4 * __popc(groups & ((1u << lane) - 1u));
+      w[0] = rs.bucket[lane];
+      w[1] = rs.count[lane];
+      w[2] = path;
+      w[3] = rho_ppm;
+    }
+    if (lane == 0) {
+      rs.words[4] = __popc(groups);
+      rs.words[5] = mask;
+    }
   }
   __syncthreads();
   for (int i = threadIdx.x; i < B; i += blockDim.x) {
-    int Ls = L_star[i];
+    int Ls = i == mine ? my_L : L_star[i];
     Ls = Ls < 1 ? 1 : (Ls > N ? N : Ls);
     const int k = bidx[i];
-    const int keep = rs.path[k] == 0 ? rs.bucket[k] : Ls;
-    const int ctx = ctx_len[i];
-    const int avail = cu_full[i + 1] - cu_full[i];
+    const bool padded = rs.path[k] == 0;
+    const int keep = padded ? rs.bucket[k] : Ls;
+    if (padded && blockIdx.x == 0) atomicAdd(&rs.words[6], keep - Ls);
+    const int ctx = i == mine ? my_ctx : ctx_len[i];
+    const int avail = i == mine ? my_avail : cu_full[i + 1] - cu_full[i];
     if (ctx < 0 || ctx + N > avail) {
       if (blockIdx.x == 0) record_error(err, kErrLayout);
     }
@@ -466,50 +525,50 @@ __global__ void __launch_bounds__(256, 4) pack_route_kernel(const uint8_t* __res
     if (blockIdx.x == 0) kv_out[i] = max(0, min(ctx + Ls, avail));
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    int acc = 0, mx = 0, pad = 0;
-    for (int i = 0; i < B; ++i) {
-      cus[i] = acc;
-      acc += seg[i];
-      mx = max(mx, seg[i]);
-      int Ls = L_star[i];
-      Ls = Ls < 1 ? 1 : (Ls > N ? N : Ls);
-      if (rs.path[bidx[i]] == 0) pad += rs.bucket[bidx[i]] - Ls;
+  if (warp == 0) {
+    // offsets: inclusive scans of 32 segments at a time
+    int acc = 0, mx = 0;
+    for (int i0 = 0; i0 < B; i0 += 32) {
+      const int i = i0 + lane;
+      const int n = i < B ? seg[i] : 0;
+      int sum = n;
+#pragma unroll
+      for (int off = 1; off < 32; off <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, sum, off);
+        if (lane >= off) sum += v;
+      }
+      if (i < B) cus[i] = acc + sum - n;
+      acc += __shfl_sync(0xffffffffu, sum, 31);
+      mx = max(mx, __reduce_max_sync(0xffffffffu, n));
     }
-    cus[B] = acc;
-    rs.total = acc;
-    rs.max_seg = mx;
-    rs.pad_rows = pad;
-    if (acc > T_cap && blockIdx.x == 0) record_error(err, kErrCapacity);
+    if (lane == 0) {
+      cus[B] = acc;
+      rs.total = acc;
+      rs.max_seg = mx;
+      if (acc > T_cap && blockIdx.x == 0) record_error(err, kErrCapacity);
+    }
   }
   __syncthreads();
 
   if (blockIdx.x == 0) {
     for (int i = threadIdx.x; i <= B; i += blockDim.x) cu_out[i] = cus[i];
     if (threadIdx.x == 0) {
-      // the control word is assembled in place in meta_out (a local array of
-      // kCtrlWords ints would live on the stack and cost registers in every block)
-      for (int i = 0; i < kCtrlWords; ++i) meta_out[i] = 0;
-      meta_out[1] = rs.total;
-      meta_out[2] = rs.max_seg;
-      meta_out[3] = graph_capacity(rs.total);
-      meta_out[4] = rs.n_groups;
-      meta_out[5] = rs.path_mask;
-      meta_out[6] = rs.pad_rows;
-      int g = 0;
-      for (int k = 0; k < rs.n_buckets && g < kCtrlMaxGroups; ++k) {
-        if (rs.count[k] == 0) continue;
-        meta_out[8 + 4 * g + 0] = rs.bucket[k];
-        meta_out[8 + 4 * g + 1] = rs.count[k];
-        meta_out[8 + 4 * g + 2] = rs.path[k];
-        meta_out[8 + 4 * g + 3] = rs.rho_ppm[k];
-        ++g;
-      }
-      meta_out[0] = epoch;
-      if (host_ctrl != nullptr) {
-        volatile int* hc = host_ctrl;
-        for (int i = 1; i < kCtrlWords; ++i) hc[i] = meta_out[i];
-        __threadfence_system();
+      rs.words[0] = epoch;
+      rs.words[1] = rs.total;
+      rs.words[2] = rs.max_seg;
+      rs.words[3] = graph_capacity(rs.total);
+    }
+    __syncthreads();
+    // a thread per word; the host's word 0 follows once the others are visible there
+    volatile int* hc = host_ctrl;
+    for (int i = threadIdx.x; i < kCtrlWords; i += blockDim.x) {
+      meta_out[i] = rs.words[i];
+      if (hc != nullptr && i > 0) hc[i] = rs.words[i];
+    }
+    if (hc != nullptr) {
+      __threadfence_system();
+      __syncthreads();
+      if (threadIdx.x == 0) {
         hc[0] = epoch;
         __threadfence_system();
       }
@@ -519,7 +578,6 @@ __global__ void __launch_bounds__(256, 4) pack_route_kernel(const uint8_t* __res
   // ---- copy rows, one warp per row, 16-byte vectors; four loads in flight
   // per lane before their stores
   const int total = min(rs.total, T_cap);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int vec = row_bytes / 16;
   for (int r = blockIdx.x * 8 + warp; r < total; r += gridDim.x * 8) {
     int lo = 0, hi = B;
@@ -637,7 +695,7 @@ cudaError_t launch_snr_scan(const int* counts, int B, int N, int F, double tau_j
                             int* L_star, int* i_star, cudaStream_t st) {
   if (B <= 0) return cudaSuccess;
   const size_t sm = N <= kScanSmemInts ? static_cast<size_t>(N) * sizeof(int) : 0;
-  return launch_kernel(snr_scan_kernel, dim3(B), dim3(32), sm, st, counts, N, F, tau_jump, gamma, window, L_star, i_star);
+  return launch_kernel(snr_scan_kernel, dim3(B), dim3(kScanThreads), sm, st, counts, N, F, tau_jump, gamma, window, L_star, i_star);
 }
 
 cudaError_t launch_pack_route(const void* x_full, int elem_bytes, const int* cu_full, const int* ctx_len,

@@ -540,3 +540,37 @@ def test_pack_route_bucket_set_variants(bucket_min):
     ctx = [100, 50, 70, 30, 10, 64, 64, 20]
     L = [120, 128, 110, 125, 300, 5, 16, 3]
     _pack_case("bf16", ctx, L, 1024, 256, seed=30 + bucket_min, bucket_min=bucket_min)
+
+
+@pytest.mark.parametrize("N,w", [(2, 1), (4, 3), (129, 3), (130, 1), (257, 10), (12289, 3)])
+@pytest.mark.parametrize("F,tau,gamma", [(12288, 0.03, 0.6), (100, 0.07, 0.5), (3 * 12288, 0.0, 0.0), (7, 3 / 7, 1.0)])
+def test_snr_scan_at_the_thresholds(N, w, F, tau, gamma):
+    """Counts whose jump and noise land on, just under and just over tau F and gamma
+    jump (where the fp32 filter must leave the decision to the fp64 test), hits in
+    every round of candidates and none; bit-exact against the oracle."""
+    rng = _rng(N + w + F)
+    B = 24
+    c = np.zeros((B, N), dtype=np.int64)
+    for b in range(B):
+        i = int(rng.integers(1, N)) if b % 4 else N - w
+        jump = int(np.ceil(tau * F)) + int(rng.integers(-1, 2))
+        noise = int(gamma * max(jump, 0)) + int(rng.integers(-1, 2))
+        base = int(rng.integers(0, 3))
+        c[b, :i] = base
+        c[b, i:] = base + max(jump, 0)
+        tail = c[b, i:]
+        tail[rng.random(len(tail)) < 0.3] += max(noise, 0)
+    counts = np.clip(c, 0, F).astype(np.int32)
+    L, I = torch.empty(B, dtype=torch.int32, device=cuda()), torch.empty(B, dtype=torch.int32, device=cuda())
+    S.seer_snr_scan(torch.from_numpy(counts).to(cuda()), B, N, F, S.make_params(0.0, tau_jump=tau, gamma=gamma, window=w), L, I)
+    i_ref, L_ref = oracle.snr_boundaries(counts, F, tau, gamma, w)
+    np.testing.assert_array_equal(I.cpu().numpy(), i_ref)
+    np.testing.assert_array_equal(L.cpu().numpy(), L_ref)
+
+
+@pytest.mark.parametrize("B,N,bucket_min", [(1, 1, 1), (33, 1000, 8), (64, 64, 1), (300, 4096, 3), (1000, 17, 8)])
+def test_pack_route_many_segments(B, N, bucket_min):
+    """More segments than a warp, every bucket count, rows of 48 bytes .. 8 KB."""
+    rng = _rng(B + N)
+    ctx, L = rng.integers(0, 20, B), rng.integers(1, N + 1, B)
+    _pack_case("bf16", ctx, L, N, 24 if B > 100 else 4096, seed=B, bucket_min=bucket_min)
