@@ -75,6 +75,8 @@ struct AttnParams {
   const int4* work;       // schedule: (b, h, first q-tile, q-tiles)
   const int* work_count;  // units in `work`
   int* work_next;         // next unit to hand out (zeroed by the schedule kernel)
+  int kv_rows;            // rows of the K/V source (capacity)
+  int parts;              // CTAs sharing a unit's keys (set by launch_tc_attn)
   int* err;
 };
 
@@ -99,9 +101,10 @@ cudaError_t launch_tc_gemm(int mode, const GemmPlan& plan, const CUtensorMap& mA
                            const CUtensorMap& mB1, const CUtensorMap& mC, const CUtensorMap& mC2, const GemmParams& p,
                            int num_sms, cudaStream_t st);
 int tc_attn_smem_bytes();
-// grid: persistent CTAs (at most one per SM); they take the units of the
-// schedule from p.work_next until *p.work_count are done
-cudaError_t launch_tc_attn(const CUtensorMap& mQ, const CUtensorMap& mKV, const AttnParams& p, int grid, bool f16,
+// persistent CTAs (at most one per SM) that take the units of the schedule from
+// p.work_next until *p.work_count are done, or, where units are few and keys many,
+// a cluster of CTAs per unit
+cudaError_t launch_tc_attn(const CUtensorMap& mQ, const CUtensorMap& mKV, AttnParams p, bool f16, int num_sms,
                            cudaStream_t st);
 // Bytes of schedule workspace the 16-bit attention kernels need for a launch
 // sized for T_cap rows, B segments and H heads: H * (ceil(T_cap/128) + B) work

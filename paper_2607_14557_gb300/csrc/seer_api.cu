@@ -424,6 +424,7 @@ seer_status do_attention(const void* qkv, void* o, seer_dtype dt, const int32_t*
   p.ld_kv = kvs.kv ? kvs.ld : 3 * H * dh;
   p.xk0 = kvs.kv ? kvs.xk0 : H * dh;
   p.xv0 = kvs.kv ? kvs.xv0 : 2 * H * dh;
+  p.kv_rows = kvs.kv ? kvs.T_kv_cap : T_cap;
   if (is16(dt)) {
     if (dh != 128) return fail(SEER_ERR_UNSUPPORTED, "16-bit attention needs head_dim == 128");
     if (kvs.kv && (!aligned16(kvs.kv) || (static_cast<long>(kvs.ld) * 2) % 16 != 0 || kvs.xk0 % 64 != 0 || kvs.xv0 % 64 != 0))
@@ -448,8 +449,7 @@ seer_status do_attention(const void* qkv, void* o, seer_dtype dt, const int32_t*
     // the attention phase brackets the attention kernel alone (the one-block
     // schedule kernel before it takes a few microseconds)
     Phase ph(PH_ATTN, st);
-    // persistent: one CTA per SM (at most one per unit)
-    SEER_CUDA(launch_tc_attn(m, kvs.kv ? mkv : m, p, std::min(max_units, di->num_sms), dt == SEER_F16, st),
+    SEER_CUDA(launch_tc_attn(m, kvs.kv ? mkv : m, p, dt == SEER_F16, di->num_sms, st),
               "tc_attn launch");
   } else {
     if (dh > 128 || dh % 4 != 0) return fail(SEER_ERR_UNSUPPORTED, "fp32 attention needs head_dim <= 128, %% 4 == 0");

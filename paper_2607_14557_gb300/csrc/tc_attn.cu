@@ -80,6 +80,7 @@ constexpr int OFF_K = NT * TILE_BYTES;
 constexpr int OFF_V = OFF_K + K_STAGES * TILE_BYTES;
 constexpr int OFF_BAR = OFF_V + V_STAGES * TILE_BYTES;
 constexpr int BAR_BYTES = 512;
+// 198144 bytes leave 60 KB of the SM to L1; 2 KB more would leave 28 (1.8% slower)
 constexpr int SMEM_BYTES = OFF_BAR + BAR_BYTES + 1024;
 static_assert(SMEM_BYTES <= 232448, "shared memory per CTA");
 constexpr uint32_t TMEM_COLS = 512;
@@ -189,6 +190,27 @@ __device__ __forceinline__ Unit decode_unit(const AttnParams& p, int u) {
   return d;
 }
 
+// Of a unit whose keys are split over a cluster of `parts` CTAs: the share of CTA
+// `part`, a run of whole key tiles (possibly none: nkv = 0).
+__device__ __forceinline__ Unit split_unit(Unit d, int part, int parts) {
+  const int t0 = d.nkv * part / parts, t1 = d.nkv * (part + 1) / parts;
+  d.kv0 += t0 * BKV;
+  d.kvL = min(d.kvL - t0 * BKV, (t1 - t0) * BKV);
+  d.nkv = t1 - t0;
+  return d;
+}
+
+__device__ __forceinline__ float ld_cluster_f32(uint32_t addr) {
+  float v;
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr));
+  return v;
+}
+__device__ __forceinline__ float4 ld_cluster_f32x4(uint32_t addr) {
+  float4 v;
+  asm volatile("ld.shared::cluster.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr));
+  return v;
+}
+
 // Unit index of this CTA's i-th unit, read from the shared ring (-1: no more
 // units or an abort); `arrive` releases the slot for this reader.
 __device__ __forceinline__ int read_unit(uint64_t* u_full, uint64_t* u_empty, const int* unit_slot, int i,
@@ -200,13 +222,26 @@ __device__ __forceinline__ int read_unit(uint64_t* u_full, uint64_t* u_empty, co
   return u;
 }
 
-template <bool F16>
+// SPLIT: launched as clusters of `parts` CTAs, one unit per cluster; each CTA runs
+// the unit over its share of the key tiles (the same loops), and the shares are
+// merged through distributed shared memory: every CTA leaves its unnormalised
+// rows of O and their (max, sum) in its own shared memory and combines 128 / parts
+// columns of all of them, in rank order.
+template <bool F16, bool SPLIT>
 __global__ void __launch_bounds__(THREADS, 1)
     tc_attn_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__ CUtensorMap mKV, const AttnParams p) {
   pdl_enter();
   const int count = *p.work_count;
-  if (static_cast<int>(blockIdx.x) >= count) return;
+  const int parts = SPLIT ? p.parts : 1;
+  const int part = SPLIT ? static_cast<int>(cluster_ctarank()) : 0;
+  const int first_unit = SPLIT ? static_cast<int>(blockIdx.x) / parts : static_cast<int>(blockIdx.x);
+  if (first_unit >= count) return;                 // the same in every CTA of a cluster
   const int G = gridDim.x;
+  const auto unit_at = [&](int u) {
+    const Unit d = decode_unit(p, u);
+    return SPLIT ? split_unit(d, part, parts) : d;
+  };
+  const bool idle = SPLIT && unit_at(first_unit).nkv == 0;   // no key tiles for this CTA: it only merges
 
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -264,7 +299,9 @@ __global__ void __launch_bounds__(THREADS, 1)
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
 
-  if (warp == 0) {
+  float m_part = -INFINITY, l_part = 0.f;    // SPLIT: this thread's row (softmax warps)
+  if (idle) {
+  } else if (warp == 0) {
     // -------------------------------------------------- TMA producer
     // The whole warp runs the loop in lockstep (every wait by all lanes, with
     // a warp-uniform outcome) and the elected lane issues: it takes the units
@@ -279,15 +316,15 @@ __global__ void __launch_bounds__(THREADS, 1)
     if (leader) {
       tma_prefetch_desc(&mQ);
       tma_prefetch_desc(&mKV);
-      unit_slot[0] = blockIdx.x;
+      unit_slot[0] = first_unit;
       mbar_arrive(&u_full[0]);
     }
     __syncwarp();
     int q_issued = 0, k_issued = 0, v_issued = 0;
     bool ok = true;
-    int u = blockIdx.x;
+    int u = first_unit;
     for (int i = 0; ok && u >= 0; ++i) {
-      const Unit d = decode_unit(p, u);
+      const Unit d = unit_at(u);
       if (i > 0 && !warp_wait(q_empty, (i - 1) & 1, abort_flag, p.err)) break;
       if (leader) {
         mbar_arrive_expect_tx(q_full, d.nt * TILE_BYTES);
@@ -303,7 +340,7 @@ __global__ void __launch_bounds__(THREADS, 1)
       if (n >= U_SLOTS && !warp_wait(&u_empty[sl], (n / U_SLOTS - 1) & 1, abort_flag, p.err)) break;
       int un = 0;
       if (leader) {
-        un = G + atomicAdd(p.work_next, 1);
+        un = SPLIT ? -1 : G + atomicAdd(p.work_next, 1);
         if (un >= count) un = -1;
         unit_slot[sl] = un;
         mbar_arrive(&u_full[sl]);
@@ -404,7 +441,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     for (int i = 0; ok; ++i) {
       const int u = __shfl_sync(0xffffffffu, read_unit(u_full, u_empty, unit_slot, i, abort_flag, p.err, lane == 0), 0);
       if (u < 0) break;
-      const Unit d = decode_unit(p, u);
+      const Unit d = unit_at(u);
       if (!warp_wait(q_full, i & 1, abort_flag, p.err)) break;
       if (t >= d.nt) {
         // idle this unit: release Q and every K / V stage as they pass
@@ -498,7 +535,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     for (int i = 0; ok; ++i) {
       const int u = __shfl_sync(0xffffffffu, read_unit(u_full, u_empty, unit_slot, i, abort_flag, p.err, lane == 0), 0);
       if (u < 0) break;
-      const Unit d = decode_unit(p, u);
+      const Unit d = unit_at(u);
       if (t >= d.nt) {
         cv += d.nkv;
         continue;
@@ -543,14 +580,16 @@ __global__ void __launch_bounds__(THREADS, 1)
         const bool any_need = __any_sync(0xffffffffu, need);
         float alpha = 1.f;
         if (need) {
-          alpha = (j == 0) ? 0.f : ex2(m_ref - m_new);
+          alpha = (j == 0 || (SPLIT && m_ref == -INFINITY)) ? 0.f : ex2(m_ref - m_new);
           m_ref = m_new;
         }
         // P_t,j: keys 32c .. 32c+31 -> 16 packed columns 16c .. 16c+15 of S_t
         // (the scores were all read above; O_t += P_t,j-1 V_j-1 has completed),
         // released to the PV MMAs in two halves of 64 keys, so the first
         // half's MMAs run while the second half is exponentiated
-        const float neg = -m_ref;
+        // a share that has met only scores of -inf adds nothing (the merge may still
+        // find finite ones elsewhere)
+        const float neg = SPLIT && m_ref == -INFINITY ? 0.f : -m_ref;
         float rs[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
         for (int hf = 0; hf < 2; ++hf) {
@@ -605,6 +644,11 @@ __global__ void __launch_bounds__(THREADS, 1)
       }
       if (!ok) break;
       if (!__all_sync(0xffffffffu, mbar_wait(&o_done[t], co & 1, abort_flag, p.err))) break;
+      if (SPLIT) {
+        m_part = m_ref;
+        l_part = l;
+        break;                                    // merged below
+      }
       tc_fence_after();
       const float inv_l = 1.f / l;
       const int qrow = (d.qt0 + t) * BQ + r;      // row inside the segment
@@ -637,6 +681,81 @@ __global__ void __launch_bounds__(THREADS, 1)
       cv += d.nkv;
     }
     report_range(nonfinite, p.err);               // an output value was infinite or NaN
+  }
+
+  if (SPLIT) {
+    // every role is done, so the operand buffers are free: tile t's O goes to the
+    // 64 KB at t * 64 KB as [column / 4][row] float4, the rows' (max, sum) to the V
+    // tiles, for the other CTAs to read
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const Unit d = unit_at(first_unit);
+    const int t = (warp - 4) >> 2, r = (warp & 3) * 32 + lane;
+    float2* ml = reinterpret_cast<float2*>(smem + OFF_V);
+    if (warp >= 4 && t < d.nt) {
+      const uint32_t tO = tmem + (static_cast<uint32_t>((warp & 3) * 32) << 16) + TM_O + 128 * t;
+      float4* mine = reinterpret_cast<float4*>(smem + t * 2 * TILE_BYTES);
+      ml[t * 128 + r] = make_float2(m_part, l_part);
+      if (!idle) {
+#pragma unroll 1
+        for (int cc = 0; cc < DH / 32; ++cc) {
+          uint32_t rr[32];
+          tmem_ld32(tO + 32 * cc, rr);
+          tmem_ld_wait();
+#pragma unroll
+          for (int e = 0; e < 8; ++e)
+            mine[(8 * cc + e) * 128 + r] = make_float4(__uint_as_float(rr[4 * e]), __uint_as_float(rr[4 * e + 1]),
+                                                       __uint_as_float(rr[4 * e + 2]), __uint_as_float(rr[4 * e + 3]));
+        }
+      }
+    }
+    cluster_sync();
+    uint32_t nonfinite = 0;
+    if (warp >= 4 && t < d.nt) {
+      const int qrow = (d.qt0 + t) * BQ + r;
+      constexpr int MAX_PARTS = 8;
+      float w[MAX_PARTS];
+      float m_all = -INFINITY, l_all = 0.f;
+#pragma unroll
+      for (int k = 0; k < MAX_PARTS; ++k)
+        if (k < parts) {
+          const uint32_t a = cluster_addr(&ml[t * 128 + r], k);
+          w[k] = ld_cluster_f32(a);
+          m_all = fmaxf(m_all, w[k]);
+        }
+#pragma unroll
+      for (int k = 0; k < MAX_PARTS; ++k)
+        if (k < parts) {
+          const float l_k = ld_cluster_f32(cluster_addr(&ml[t * 128 + r], k) + 4);
+          // a share without keys has sum 0 and no rows to read
+          w[k] = l_k == 0.f ? 0.f : ex2(w[k] - m_all);
+          l_all += l_k * w[k];
+        }
+      const float inv_l = 1.f / l_all;
+      if (qrow < d.L) {
+        uint16_t* orow = reinterpret_cast<uint16_t*>(p.out) + static_cast<size_t>(d.seq0 + qrow) * p.ldo + d.h * DH;
+        const int per = DH / 4 / parts;              // 4-column groups of this CTA
+        for (int g = part * per; g < (part + 1) * per; ++g) {
+          float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+          const float4* src = reinterpret_cast<const float4*>(smem + t * 2 * TILE_BYTES) + g * 128 + r;
+#pragma unroll
+          for (int k = 0; k < MAX_PARTS; ++k)
+            if (k < parts && w[k] != 0.f) {
+              const float4 v = ld_cluster_f32x4(cluster_addr(src, k));
+              acc.x = fmaf(w[k], v.x, acc.x);
+              acc.y = fmaf(w[k], v.y, acc.y);
+              acc.z = fmaf(w[k], v.z, acc.z);
+              acc.w = fmaf(w[k], v.w, acc.w);
+            }
+          const uint32_t q0 = pack2(acc.x * inv_l, acc.y * inv_l, F16), q1 = pack2(acc.z * inv_l, acc.w * inv_l, F16);
+          nonfinite |= nonfinite_term(q0, F16) | nonfinite_term(q1, F16);
+          reinterpret_cast<uint2*>(orow)[g] = make_uint2(q0, q1);
+        }
+      }
+    }
+    if (warp >= 4) report_range(nonfinite, p.err);
+    cluster_sync();                                  // no CTA leaves while its rows are read
   }
 
   tc_fence_before();
@@ -707,22 +826,47 @@ __global__ void attn_schedule_kernel(const int* cu, const int* cu_kv, const int*
   }
 }
 
-template <bool F16>
+template <bool F16, bool SPLIT>
 cudaError_t launch_typed(const CUtensorMap& mQ, const CUtensorMap& mKV, const AttnParams& p, int grid, cudaStream_t st) {
   static bool attr_set[64] = {};
-  cudaError_t e = set_smem_limit_once(tc_attn_kernel<F16>, SMEM_BYTES, attr_set);
+  cudaError_t e = set_smem_limit_once(tc_attn_kernel<F16, SPLIT>, SMEM_BYTES, attr_set);
   if (e != cudaSuccess) return e;
   if (grid <= 0) return cudaSuccess;
-  return launch_kernel(tc_attn_kernel<F16>, dim3(grid), dim3(THREADS), SMEM_BYTES, st, mQ, mKV, p);
+  return launch_kernel_overlap(launch_overlap_enabled(), p.parts, tc_attn_kernel<F16, SPLIT>, dim3(grid), dim3(THREADS),
+                               SMEM_BYTES, st, mQ, mKV, p);
 }
 
 }  // namespace
 
 int tc_attn_smem_bytes() { return SMEM_BYTES; }
 
-cudaError_t launch_tc_attn(const CUtensorMap& mQ, const CUtensorMap& mKV, const AttnParams& p, int grid, bool f16,
+// CTAs that share a unit's keys, from what the host knows: the most units the
+// call can have (a segment of L rows has ceil(L / 256) per head) and the average
+// number of key tiles.  Split only where units leave most SMs idle, each share keeps
+// four key tiles (six of two), and the clusters fit at once (152 SMs hold 76 clusters of 2, 36
+// of 4, 15 of 8).  us, one CTA per unit -> split: the cached 8B layer of one sequence,
+// 50 rows over 3062 keys 160 -> 139 (4 CTAs), 120 over 12120 272 -> 165; 2 heads of
+// 3000 rows 40.5 -> 23.6 (4), of 5900 + 300 rows 71 -> 49; at 8 tiles 2 CTAs gain
+// nothing (2 heads of 1100 rows 21.0 -> 22.4).
+int attn_parts(long max_units, long kv_rows, int B) {
+  const long tiles = kv_rows / B / BKV;
+  if (max_units <= 15 && tiles >= 32) return 8;
+  if (max_units <= 36 && tiles >= 16) return 4;
+  if (max_units <= 76 && tiles >= 12) return 2;
+  return 1;
+}
+
+cudaError_t launch_tc_attn(const CUtensorMap& mQ, const CUtensorMap& mKV, AttnParams p, bool f16, int num_sms,
                            cudaStream_t st) {
-  return f16 ? launch_typed<true>(mQ, mKV, p, grid, st) : launch_typed<false>(mQ, mKV, p, grid, st);
+  const long max_units = static_cast<long>(p.n_heads) * (p.T_cap / (NT * BQ) + p.B);
+  p.parts = attn_parts(max_units, p.kv_rows, p.B);
+  if (p.parts > 1) {
+    const int grid = static_cast<int>(max_units) * p.parts;
+    return f16 ? launch_typed<true, true>(mQ, mKV, p, grid, st) : launch_typed<false, true>(mQ, mKV, p, grid, st);
+  }
+  // persistent: one CTA per SM (at most one per unit)
+  const int grid = static_cast<int>(max_units < num_sms ? max_units : num_sms);
+  return f16 ? launch_typed<true, false>(mQ, mKV, p, grid, st) : launch_typed<false, false>(mQ, mKV, p, grid, st);
 }
 
 cudaError_t launch_attn_schedule(const int* cu, const int* cu_kv, const int* kv_len, int B, int n_heads, int T_cap,

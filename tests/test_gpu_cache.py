@@ -110,6 +110,35 @@ def test_kv_prefill_stores_segments_where_the_offsets_say(d, ctx, bad):
     assert torch.equal(cache, want)
 
 
+@pytest.mark.parametrize("ctx,resp", [([4200], [40]), ([5000, 4300], [200, 7]), ([9000], [300])])
+def test_cached_layer_long_prefixes_few_rows(ctx, resp):
+    """Few query tiles over long caches: each unit's keys are split over 8 or 4 CTAs."""
+    wl = _workload("bf16")
+    w = synth.layer_weights(wl, 0)
+    d, H, B = wl.d, wl.n_heads, len(ctx)
+    dims = S.make_dims(d, H, wl.head_dim, wl.d_ff)
+    from paper_2607_14557_gb300 import driver as D
+    W = D.LayerWeights.from_host(w, "bf16")
+    rng = np.random.default_rng(sum(ctx))
+    cu = np.concatenate([[0], np.cumsum([a + b for a, b in zip(ctx, resp)])])
+    cr = np.concatenate([[0], np.cumsum(resp)])
+    T, R = int(cu[-1]), int(cr[-1])
+    x = synth.round_storage(rng.standard_normal((R, d)), "bf16")
+    kv = torch.from_numpy(rng.standard_normal((T, 2 * d)).astype(np.float32)).half()
+    cache = kv.to(cuda())
+    y = torch.full((R, d), 9.0, dtype=torch.bfloat16, device=cuda())
+    n = S.seer_layer_workspace_size(dims, "bf16", R, B)
+    ws = torch.empty(n, dtype=torch.uint8, device=cuda())
+    S.seer_layer_forward_cached(W.struct(), dims, "bf16", to_dev(x, "bf16"), y, i32(cr), i32(ctx), B, R, cache, i32(cu),
+                                None, T, ws, n)
+    assert S.seer_check_device() == 0
+    k, got = kv.numpy().astype(np.float64), host(y)
+    for b, c in enumerate(ctx):
+        pre = k[cu[b]:cu[b] + c]
+        ref = oracle.layer_forward_cached(x[cr[b]:cr[b + 1]], pre[:, :d], pre[:, d:], w, H)
+        check_close(got[cr[b]:cr[b + 1]], ref, "bf16", f"cached block segment {b}")
+
+
 def test_cache_entry_points_reject_bad_arguments():
     x = torch.zeros((8, 256), dtype=torch.bfloat16, device=cuda())
     cu = i32([0, 8])

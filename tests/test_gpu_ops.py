@@ -296,6 +296,34 @@ def test_attention_growing_max_forces_rescale(dt):
     _attention_case(dt, 2, 128, lens, lens, 1.0, 15, structured=True)
 
 
+@pytest.mark.parametrize("dt", ["f16", "bf16"])
+@pytest.mark.parametrize("H,lens,kv", [
+    (4, [1700], [1700]), (3, [2500, 700], [2401, 700]),                        # keys of a unit over 2 CTAs
+    (2, [4200], [4133]), (1, [3000], [3000]), (1, [4000, 300], [3900, 77]),    # over 4, some without keys
+    (1, [3700], [129])])
+def test_attention_split_keys(dt, H, lens, kv):
+    _attention_case(dt, H, 128, lens, kv, 1.0, 17)
+
+
+@pytest.mark.parametrize("dt", ["f16", "bf16"])
+def test_attention_split_keys_with_infinite_scores(dt):
+    """Shares (and first tiles of shares) whose every score is -inf add nothing: the
+    result is the attention over the finite keys."""
+    n, keep = 3000, [*range(0, 700), *range(1000, 1300)]          # 4 shares of 6 tiles; two without a finite score
+    g = torch.Generator(device="cuda").manual_seed(3)
+    qkv = torch.randn((n, 3 * 128), generator=g, device="cuda").to(tdtype(dt))
+    qkv[:, 0] = 1.0
+    dead = torch.ones(n, dtype=torch.bool, device="cuda")
+    dead[keep] = False
+    qkv[dead, 128] = float("-inf")
+    out = torch.empty((n, 128), dtype=qkv.dtype, device="cuda")
+    ws = torch.empty(1 << 16, dtype=torch.uint8, device="cuda")
+    S.seer_attention(qkv, out, dt, i32([0, n]), None, 1, n, 1, 128, ws, 1 << 16)
+    q = qkv.double()
+    ref = torch.softmax(q[:, :128] @ q[keep, 128:256].T / 128 ** 0.5, dim=-1) @ q[keep, 256:]
+    check_close(host(out), host(ref.float()), "bf16", "attention, infinite scores")
+
+
 def test_attention_many_heads():
     _attention_case("f16", 4, 128, [200, 90], [200, 90], 1.0, 12)
 
