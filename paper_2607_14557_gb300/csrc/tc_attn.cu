@@ -845,9 +845,9 @@ int tc_attn_smem_bytes() { return SMEM_BYTES; }
 // number of key tiles.  Split only where units leave most SMs idle, each share keeps
 // four key tiles (six of two), and the clusters fit at once (152 SMs hold 76 clusters of 2, 36
 // of 4, 15 of 8).  us, one CTA per unit -> split: the cached 8B layer of one sequence,
-// 50 rows over 3062 keys 160 -> 139 (4 CTAs), 120 over 12120 272 -> 165; 2 heads of
-// 3000 rows 40.5 -> 23.6 (4), of 5900 + 300 rows 71 -> 49; at 8 tiles 2 CTAs gain
-// nothing (2 heads of 1100 rows 21.0 -> 22.4).
+// 50 rows over 3062 keys 154 -> 140 (4 CTAs), 120 over 12120 241 -> 166; 2 heads of
+// 3000 rows 40.2 -> 22.9 (4), of 5900 + 300 rows 70.7 -> 48.4; at 8 tiles 2 CTAs gain
+// nothing (2 heads of 1100 rows 20.8 -> 22.4).
 int attn_parts(long max_units, long kv_rows, int B) {
   const long tiles = kv_rows / B / BKV;
   if (max_units <= 15 && tiles >= 32) return 8;

@@ -123,20 +123,27 @@ def _p(t) -> Optional[int]:
     return t.data_ptr()
 
 
+_DTYPES = {SEER_F32: SEER_F32, SEER_BF16: SEER_BF16, SEER_F16: SEER_F16, "bf16": SEER_BF16,
+           torch.bfloat16: SEER_BF16, "f16": SEER_F16, torch.float16: SEER_F16, "f32": SEER_F32,
+           torch.float32: SEER_F32}
+
+
 def _dt(dt) -> int:
-    if dt in (SEER_F32, SEER_BF16, SEER_F16):
-        return dt
-    if dt in ("bf16", torch.bfloat16):
-        return SEER_BF16
-    if dt in ("f16", torch.float16):
-        return SEER_F16
-    if dt in ("f32", torch.float32):
-        return SEER_F32
-    raise ValueError(f"unsupported dtype {dt!r}")
+    code = _DTYPES.get(dt)
+    if code is None:
+        raise ValueError(f"unsupported dtype {dt!r}")
+    return code
+
+
+# The current stream's handle without building a torch.cuda.Stream around it (2.8 us
+# of a small call's ~11 us on the host; 0.4 this way).
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
 
 
 def _stream(stream) -> Optional[int]:
     if stream is None:
+        if _raw_stream is not None:
+            return _raw_stream(torch.cuda.current_device())
         return torch.cuda.current_stream().cuda_stream
     if isinstance(stream, int):
         return stream
