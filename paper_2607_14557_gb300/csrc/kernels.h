@@ -50,6 +50,9 @@ struct GemmParams {
   int res_type;           // ElemType of R
   int bn;                 // accumulator columns per tile (multiple of 32)
   int stages;             // operand ring: stages
+  int few_m;              // with at most this many row tiles (of cg * 128 rows), instead of bn ...
+  int few_bn;             // ... this many columns per tile (single-weight modes; mB1 has its boxes) ...
+  int few_stages;         // ... and stages
   int group_m;            // raster: row tiles per group (see tc_gemm.cu)
   float rope_theta;       // Rope: frequency base (> 0)
   int rope_cols;          // Rope: leading output columns that are rotated (the q|k columns)
@@ -89,13 +92,17 @@ struct GemmPlan {
   int stages;    // operand ring: stages
   int group_m;   // raster: row tiles per group
   int depth;     // 64-deep k-blocks per stage: 1 or 2
+  int few_m;     // tile choice of a call whose device row count leaves at most few_m row
+  int few_bn;    // tiles: few_bn columns (few_m = 0: no second choice)
 };
 // m_tiles: 128-row tiles; n_cols: accumulator columns (N; Swiglu / Count: 2 F);
-// K: depth; num_sms: SMs of the device.
-GemmPlan tc_gemm_plan(int mode, long m_tiles, long n_cols, int K, int num_sms);
+// K: depth; device_rows: the row count is read on the device (m_tiles is a bound);
+// num_sms: SMs of the device.
+GemmPlan tc_gemm_plan(int mode, long m_tiles, long n_cols, int K, bool device_rows, int num_sms);
 // mC: the 16-bit output C (Store, Residual, Rope) or act (Swiglu) with 32 x 32
 // boxes and no swizzle, for the epilogue's TMA stores (unused by Count).  mA
-// has boxes of 128 rows, mB0 and mB1 boxes of bn / 2 rows; mC2 is C2 in boxes
+// has boxes of 128 rows, mB0 and mB1 boxes of bn / 2 rows (mB1 of few_bn / 2 where
+// the plan has a second choice); mC2 is C2 in boxes
 // like mC's (Kv only).
 cudaError_t launch_tc_gemm(int mode, const GemmPlan& plan, const CUtensorMap& mA, const CUtensorMap& mB0,
                            const CUtensorMap& mB1, const CUtensorMap& mC, const CUtensorMap& mC2, const GemmParams& p,

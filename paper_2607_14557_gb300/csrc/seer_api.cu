@@ -285,16 +285,18 @@ seer_status do_linear(const void* a, const void* w, seer_dtype op_dt, const void
     if (!aligned16(a) || !aligned16(w) || !aligned16(c) || (r && !aligned16(r)))
       return fail(SEER_ERR_UNSUPPORTED, "16-bit linear needs 16-byte aligned pointers");
     if (M_cap == 0) return SEER_OK;
-    const GemmPlan plan = tc_gemm_plan(mode, (M_cap + 127l) / 128, N, K, di->num_sms);
+    const GemmPlan plan = tc_gemm_plan(mode, (M_cap + 127l) / 128, N, K, M_dev != nullptr, di->num_sms);
     p.idesc = make_idesc(128 * plan.cg, plan.bn, 0, op_dt == SEER_F16);
     CUtensorMap mA, mB, mC;
     SEER_TRY(make_map16(&mA, a, op_dt, M_cap, K, K, 128));
     SEER_TRY(make_map16(&mB, w, op_dt, N, K, K, plan.bn / 2));
+    CUtensorMap mB2 = mB;
+    if (plan.few_m > 0) SEER_TRY(make_map16(&mB2, w, op_dt, N, K, K, plan.few_bn / 2));
     SEER_TRY(make_map16(&mC, c, c_dt, M_cap, N, N, 32, 32, false));
     CUtensorMap mC2 = mC;
     if (dest.kv) SEER_TRY(make_map16(&mC2, dest.kv, c_dt, dest.map.rows, dest.ld, dest.ld, 32, 32, false));
     Phase ph(phase, st);
-    SEER_CUDA(launch_tc_gemm(mode, plan, mA, mB, mB, mC, mC2, p, di->num_sms, st), "tc_gemm launch");
+    SEER_CUDA(launch_tc_gemm(mode, plan, mA, mB, mB2, mC, mC2, p, di->num_sms, st), "tc_gemm launch");
   } else {
     if (c_dt != SEER_F32 || (r && r_dt != SEER_F32)) return fail(SEER_ERR_UNSUPPORTED, "fp32 linear needs fp32 output");
     if (M_cap == 0) return SEER_OK;
@@ -352,7 +354,7 @@ seer_status do_swiglu(const void* a, const void* wg, const void* wu, seer_dtype 
   if (M_cap == 0) return SEER_OK;
   if (is16(op_dt)) {
     const long m_tiles = mode == kGemmCount ? static_cast<long>(B) * ((N + 127l) / 128) : (M_cap + 127l) / 128;
-    const GemmPlan plan = tc_gemm_plan(mode, m_tiles, 2l * F, K, di->num_sms);
+    const GemmPlan plan = tc_gemm_plan(mode, m_tiles, 2l * F, K, mode != kGemmCount && M_dev != nullptr, di->num_sms);
     p.idesc = make_idesc(128 * plan.cg, plan.bn, 0, op_dt == SEER_F16);
     CUtensorMap mA, mG, mU, mC;
     SEER_TRY(make_map16(&mA, a, op_dt, M_cap, K, K, 128));

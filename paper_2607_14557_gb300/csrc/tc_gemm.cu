@@ -127,13 +127,9 @@ __global__ void __launch_bounds__(THREADS, 1)
     tc_gemm_kernel(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CUtensorMap mB0,
                    const __grid_constant__ CUtensorMap mB1, const __grid_constant__ CUtensorMap mC,
                    const __grid_constant__ CUtensorMap mC2, const GemmParams p) {
-  const int BN = p.bn;
-  const int stages = p.stages;                              // of DEPTH k-blocks
-  const int bbytes = stage_bytes(CG, BN);                   // operand bytes of a k-block
-  const int sbytes = DEPTH * bbytes;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  uint8_t* fixed = smem + stages * sbytes;
+  uint8_t* fixed = smem + RING_BYTES;
   uint64_t* full = reinterpret_cast<uint64_t*>(fixed);
   uint64_t* empty = full + MAX_STAGES;
   uint64_t* acc_full = empty + MAX_STAGES;
@@ -148,7 +144,7 @@ __global__ void __launch_bounds__(THREADS, 1)
   const uint32_t rank = CG == 2 ? cluster_ctarank() : 0u;   // CTA of the pair; rank 0 issues the MMAs
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < stages; ++s) {
+    for (int s = 0; s < MAX_STAGES; ++s) {
       mbar_init(&full[s], 1);
       mbar_init(&empty[s], 1);
     }
@@ -192,6 +188,13 @@ __global__ void __launch_bounds__(THREADS, 1)
     num_mt = (M + BM - 1) / BM;
   }
   constexpr bool halfN = (MODE == kGemmSwiglu || MODE == kGemmCount);
+  // the tile choice for the rows there are: a call sized for more may be better off
+  // with other tiles (tc_gemm_plan)
+  const bool few = !halfN && MODE != kGemmRope && (num_mt + CG - 1) / CG <= p.few_m;
+  const int BN = few ? p.few_bn : p.bn;
+  const int stages = few ? p.few_stages : p.stages;         // of DEPTH k-blocks
+  const int bbytes = stage_bytes(CG, BN);                   // operand bytes of a k-block
+  const int sbytes = DEPTH * bbytes;
   const int tile_n = halfN ? BN / 2 : BN;                   // columns of p.N covered by a tile
   const int num_m = (num_mt + CG - 1) / CG;
   const int num_n = (p.N + tile_n - 1) / tile_n;
@@ -214,6 +217,9 @@ __global__ void __launch_bounds__(THREADS, 1)
     const bool leader = elect_one();
     const uint32_t full0 = CG == 2 ? cluster_addr(full, 0) : 0u;
     const int half_b = BN / 2 * BK * 2;                     // bytes of one half of B's rows
+    // both halves come from one matrix unless they are gate and up rows
+    const CUtensorMap* mapB0 = few ? &mB1 : &mB0;
+    const CUtensorMap* mapB1 = halfN ? &mB1 : mapB0;
     int s = 0;
     uint32_t ph = 0;
     long issued = 0;
@@ -249,12 +255,12 @@ __global__ void __launch_bounds__(THREADS, 1)
             const int x = (kb + u) * BK;
             if (CG == 1) {
               tma_load_2d(sa, &mA, &full[s], x, a_row);
-              tma_load_2d(sa + A_TILE_BYTES, &mB0, &full[s], x, b_row0);
-              tma_load_2d(sa + A_TILE_BYTES + half_b, &mB1, &full[s], x, b_row1);
+              tma_load_2d(sa + A_TILE_BYTES, mapB0, &full[s], x, b_row0);
+              tma_load_2d(sa + A_TILE_BYTES + half_b, mapB1, &full[s], x, b_row1);
             } else {
               tma_load_2d_pair(sa, &mA, bar, x, a_row);
-              if (rank == 0) tma_load_2d_pair(sa + A_TILE_BYTES, &mB0, bar, x, b_row0);
-              else tma_load_2d_pair(sa + A_TILE_BYTES, &mB1, bar, x, b_row1);
+              if (rank == 0) tma_load_2d_pair(sa + A_TILE_BYTES, mapB0, bar, x, b_row0);
+              else tma_load_2d_pair(sa + A_TILE_BYTES, mapB1, bar, x, b_row1);
             }
           }
         }
@@ -283,7 +289,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     // waits, and a lane that gives up (only after a 2 s limit) leaves the loop alone
     // (narrow tiles 10% faster; 127 rows, down: 42.6 -> 38.4 us).
     const bool leader = elect_one();
-    const uint32_t idesc = p.idesc;
+    const uint32_t idesc = (p.idesc & ~(0x3Fu << 17)) | (static_cast<uint32_t>(BN >> 3) << 17);   // N of the tile
     int s = 0;
     uint32_t ph = 0;
     int acc = 0;
@@ -565,6 +571,11 @@ __global__ void __launch_bounds__(THREADS, 1)
   }
 }
 
+int plan_stages(int cg, int bn, int depth) {
+  const int fit = RING_BYTES / (depth * stage_bytes(cg, bn));
+  return fit < MAX_STAGES ? fit : MAX_STAGES;
+}
+
 template <int MODE, int CG, int DEPTH>
 cudaError_t launch_mode(const GemmPlan& plan, const CUtensorMap& mA, const CUtensorMap& mB0, const CUtensorMap& mB1,
                         const CUtensorMap& mC, const CUtensorMap& mC2, GemmParams p, int num_sms, cudaStream_t st) {
@@ -574,20 +585,30 @@ cudaError_t launch_mode(const GemmPlan& plan, const CUtensorMap& mA, const CUten
   long num_mt;
   if (MODE == kGemmCount) num_mt = static_cast<long>(p.B) * ((p.Nw + BM - 1) / BM);
   else num_mt = (p.M_cap + BM - 1) / BM;
-  const int tile_n = (MODE == kGemmSwiglu || MODE == kGemmCount) ? plan.bn / 2 : plan.bn;
-  const long tiles = ((num_mt + CG - 1) / CG) * ((p.N + tile_n - 1) / tile_n);
+  const auto tiles_of = [&](long m, int bn) {
+    const int tile_n = (MODE == kGemmSwiglu || MODE == kGemmCount) ? bn / 2 : bn;
+    return m * ((p.N + tile_n - 1) / tile_n);
+  };
+  const long num_m = (num_mt + CG - 1) / CG;
+  long tiles = tiles_of(num_m, plan.bn);
   if (tiles <= 0) return cudaSuccess;
+  if (plan.few_m > 0) {
+    const long few = tiles_of(plan.few_m < num_m ? plan.few_m : num_m, plan.few_bn);
+    if (few > tiles) tiles = few;
+  }
   p.bn = plan.bn;
+  p.few_m = plan.few_m;
+  p.few_bn = plan.few_bn;
+  p.few_stages = plan.few_m > 0 ? plan_stages(CG, plan.few_bn, DEPTH) : 0;
   p.stages = plan.stages;
   p.group_m = plan.group_m;
   const int units = num_sms / CG;
   const int grid = static_cast<int>(tiles < units ? tiles : units);
-  const int smem = plan.stages * DEPTH * stage_bytes(CG, plan.bn) + FIXED_BYTES;
   // long calls gain little from the overlap but lose nothing (one layer of 35k rows:
   // 11.9 ms either way); one of 842 rows 391 us without any, 383 with calls of up to
   // five tiles per SM overlapped, 379 with all
   return launch_kernel_overlap(launch_overlap_enabled(), CG, tc_gemm_kernel<MODE, CG, DEPTH>, dim3(grid * CG), dim3(THREADS),
-                               smem, st, mA, mB0, mB1, mC, mC2, p);
+                               RING_BYTES + FIXED_BYTES, st, mA, mB0, mB1, mC, mC2, p);
 }
 
 template <int MODE>
@@ -621,31 +642,57 @@ cudaError_t launch_cg(const GemmPlan& plan, const CUtensorMap& mA, const CUtenso
 // commit and loop per stage (~100 cycles) exceed what the MMAs hide (127 rows, down:
 // 38.4 us with one, 32.3 with two; 842 rows at 128 columns 75.1 and 71.6, at 224
 // columns 61.0 and 63.2).
-GemmPlan tc_gemm_plan(int mode, long m_tiles, long n_cols, int K, int num_sms) {
+// A row count read on the device may leave fewer row tiles than the call is sized
+// for (a packed batch in buffers for its full windows): single-weight modes then get
+// a second width for four fifths of the tiles, and among choices within 8% of the
+// best at full size the one that is best over both is taken (the path at batch 1, 842
+// rows in buffers for 1049: 377 -> 371 us).
+GemmPlan tc_gemm_plan(int mode, long m_tiles, long n_cols, int K, bool device_rows, int num_sms) {
   const bool half_n = mode == kGemmSwiglu || mode == kGemmCount;
   // whole 32-column chunks of the output, and whole heads for Rope
   const int step = mode == kGemmRope ? 128 : (half_n ? 64 : 32);
-  GemmPlan g{2, 256, 0, 1, 1};
-  double best = 0.0;
-  for (int cg = 2; cg >= 1; --cg) {
-    for (int bn = 256; bn >= step; bn -= step) {
-      const long tiles = ((m_tiles + cg - 1) / cg) * ((n_cols + bn - 1) / bn);
-      const long units = num_sms / cg;
-      const bool narrow = bn / cg <= 64;
-      const double block = cg == 2 ? (narrow ? 0.115 + 0.0004 * bn : 0.03 + 0.001 * bn)
-                                   : (narrow ? 0.143 + 0.0003 * bn : fmax(0.19, 0.08 + 0.00112 * bn));
-      const double fixed = cg == 2 ? 6.0 + 0.015 * bn : 4.2 + 0.0125 * bn;
-      const double cost = fixed + static_cast<double>((tiles + units - 1) / units) * (K / BK) * block;
-      if (g.stages == 0 || cost < 0.98 * best) {      // wide pair tiles unless another choice is clearly faster
-        best = cost;
-        g.cg = cg;
-        g.bn = bn;
-        g.depth = narrow ? 2 : 1;
-        g.stages = RING_BYTES / (g.depth * stage_bytes(cg, bn));
-      }
+  const auto cost = [&](int cg, int bn, long mt) {
+    const long tiles = ((mt + cg - 1) / cg) * ((n_cols + bn - 1) / bn);
+    const long units = num_sms / cg;
+    const bool narrow = bn / cg <= 64;
+    const double block = cg == 2 ? (narrow ? 0.115 + 0.0004 * bn : 0.03 + 0.001 * bn)
+                                 : (narrow ? 0.143 + 0.0003 * bn : fmax(0.19, 0.08 + 0.00112 * bn));
+    const double fixed = cg == 2 ? 6.0 + 0.015 * bn : 4.2 + 0.0125 * bn;
+    return fixed + static_cast<double>((tiles + units - 1) / units) * (K / BK) * block;
+  };
+  // cheapest width for mt row tiles; narrower than 256 only where clearly faster
+  const auto width = [&](int cg, long mt, int depth) {
+    int best = 0;
+    for (int bn = 256; bn >= step; bn -= step)
+      if ((depth == 0 || depth == (bn / cg <= 64 ? 2 : 1)) && (best == 0 || cost(cg, bn, mt) < 0.98 * cost(cg, best, mt)))
+        best = bn;
+    return best;
+  };
+  const auto depth_of = [](int cg, int bn) { return bn / cg <= 64 ? 2 : 1; };
+  const long few = device_rows && m_tiles > 2 ? (4 * m_tiles + 4) / 5 : m_tiles;
+  const bool second = !half_n && mode != kGemmRope;
+
+  GemmPlan g{2, width(2, m_tiles, 0), 0, 1, 1, 0, 0};
+  int one = width(1, m_tiles, 0);                      // the one-SM choice
+  const double pair_full = cost(2, g.bn, m_tiles), one_full = cost(1, one, m_tiles);
+  bool use_one = one_full < 0.98 * pair_full;
+  if (few < m_tiles) {
+    const int pair_bn = second ? width(2, few, depth_of(2, g.bn)) : g.bn;
+    const int one_bn = second ? width(1, few, depth_of(1, one)) : one;
+    const double pair_few = cost(2, pair_bn > 0 ? pair_bn : g.bn, few), one_few = cost(1, one_bn > 0 ? one_bn : one, few);
+    if (fmax(pair_full, one_full) <= 1.08 * fmin(pair_full, one_full)) use_one = one_full + one_few < pair_full + pair_few;
+    const int other = use_one ? one_bn : pair_bn, cg = use_one ? 1 : 2;
+    if (second && other > 0 && other != (use_one ? one : g.bn)) {
+      g.few_bn = other;
+      g.few_m = static_cast<int>((few + cg - 1) / cg);
     }
   }
-  if (g.stages > MAX_STAGES) g.stages = MAX_STAGES;
+  if (use_one) {
+    g.cg = 1;
+    g.bn = one;
+  }
+  g.depth = depth_of(g.cg, g.bn);
+  g.stages = plan_stages(g.cg, g.bn, g.depth);
   // L2 raster: the 76 pair tiles in flight form a block of about 16 x 5, so each
   // operand slab is shared by many SMs at once: 16 columns of tiles swept per row
   // tile where the matrix has no more, else groups of 16 row tiles.  Swept on GB300

@@ -96,6 +96,23 @@ def test_linear_tile_choices(M, N, K, res):
     assert torch.isnan(c[M]).all()                                  # nothing past the last row
 
 
+@pytest.mark.parametrize("M_cap,N,K", [(640, 12288, 128), (640, 4096, 192), (900, 4096, 64), (1049, 4096, 128),
+                                       (1500, 4096, 64), (1500, 12288, 64)])
+@pytest.mark.parametrize("fill", [0.0, 0.01, 0.5, 0.78, 0.8, 0.82, 1.0])
+def test_linear_second_tile_choice_for_fewer_device_rows(M_cap, N, K, fill):
+    """Calls whose device row count is below the size they are planned for use the
+    plan's second tile width up to four fifths of the row tiles: exact on integers,
+    rows past the count untouched."""
+    M = int(M_cap * fill)
+    rng = _rng(M_cap + N + K)
+    a, w = (to_dev(rng.integers(-2, 3, s).astype(np.float32), "f16") for s in ((M_cap, K), (N, K)))
+    r = to_dev(rng.integers(-8, 9, (M_cap, N)).astype(np.float32), "f16")
+    c = torch.full((M_cap, N), float("nan"), dtype=torch.bfloat16, device=cuda())
+    S.seer_linear(a, w, "f16", r, "f16", c, "bf16", M_cap, i32([M]), N, K)
+    assert torch.equal(c[:M], (a[:M].double() @ w.double().T + r[:M].double()).to(torch.bfloat16))
+    assert torch.isnan(c[M:]).all()
+
+
 @pytest.mark.parametrize("M,F,K", [(1, 128, 64), (127, 1280, 64), (200, 384, 128), (300, 12288, 64), (900, 1408, 64)])
 def test_swiglu_tile_choices(M, F, K):
     """Gate/up tiles of every width, the last one narrower than the others."""
