@@ -17,7 +17,7 @@ CSRC = os.path.join(PKG, "csrc")
 BUILD = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libseer.so")
 SOURCES = ["seer_api.cu", "tc_gemm.cu", "tc_attn.cu", "simt.cu", "aux_kernels.cu", "seer_noalloc.cu"]
-HEADERS = ["common.cuh", "kernels.h"]
+HEADERS = ["common.cuh", "kernels.h", "attn_schedule.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

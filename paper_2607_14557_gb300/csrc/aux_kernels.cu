@@ -6,6 +6,7 @@
 //                    with device-resident compaction and the pinned control word
 #include <math.h>
 
+#include "attn_schedule.cuh"
 #include "common.cuh"
 #include "kernels.h"
 
@@ -98,6 +99,26 @@ __global__ void __launch_bounds__(256) rmsnorm_kernel(const void* __restrict__ x
   if (OUT != kF32) report_range(nonfinite, err);
 }
 
+// One block's share of a rotary table: its rows, 64 pairs each.
+__device__ __forceinline__ void rope_table_block(const RopeTable& t, int block, int blocks, int* err, float2* freq) {
+  if (threadIdx.x < 64) freq[threadIdx.x] = rope_inv_freq(threadIdx.x, 128, t.theta);
+  __syncthreads();
+  int M = t.cu[t.B];
+  if (M < 0 || M > t.T_cap) M = M < 0 ? 0 : t.T_cap;           // recorded by the row kernels
+  const int i = threadIdx.x & 63, step = blocks * (blockDim.x >> 6);
+  for (int row = block * (blockDim.x >> 6) + (threadIdx.x >> 6); row < M; row += step) {
+    float c, sn;
+    rope_cos_sin(static_cast<float>(row_position(t.cu, t.B, row)), freq[i], c, sn);
+    t.tab[static_cast<size_t>(row) * 64 + i] = make_float2(c, sn);
+  }
+}
+
+__global__ void __launch_bounds__(256) rope_table_kernel(const RopeTable t, int* err) {
+  pdl_enter();
+  __shared__ float2 freq[64];
+  rope_table_block(t, blockIdx.x, gridDim.x, err, freq);
+}
+
 // 16-bit rows of up to 256 * VPL elements: the row is read once into
 // registers (VPL 16-byte vectors per lane, all loads in flight together), the
 // sum of squares reduced across the warp, and the row scaled from registers.
@@ -108,26 +129,40 @@ __global__ void __launch_bounds__(256) rmsnorm_kernel(const void* __restrict__ x
 // d = 4096) while the block's first rows are in flight (9973 rows: 29.9 -> 27.9 us
 // against staging it first); read from global memory per row, its loads were
 // hoisted beside the row's 64 registers and spilled.
-template <int IN, int OUT, int VPL, bool MAP>
+// PRE: the first `extra` blocks leave the rows to the others and do the prelude's work
+// (block 0 the attention schedule, the rest the rotary table): neither depends on the
+// rows, and as launches of their own they stood in the layer's chain of kernels (us,
+// without rotation: cached 8B layer of 848 rows 378.6 -> 376.0, 150 rows of a 256-wide
+// layer 31.5 -> 30.0; with: 450 rows of it 47.3 -> 40.0, 240 rows of the 8B layer
+// 154.5 -> 148.0).
+template <int IN, int OUT, int VPL, bool MAP, bool PRE>
 __global__ void __launch_bounds__(256, 2) rmsnorm_rows_kernel(const void* __restrict__ x, const void* __restrict__ g,
                                                            void* __restrict__ y, int M_cap, const int* M_dev, int d,
-                                                           float eps, const RowMap map, int* err) {
+                                                           float eps, const RowMap map, const Prelude pre, int extra,
+                                                           int* err) {
   pdl_enter();
+  __shared__ uint4 g_sh[32 * VPL];
+  if (PRE && static_cast<int>(blockIdx.x) < extra) {
+    const int sched = pre.sched.work != nullptr ? 1 : 0;
+    if (static_cast<int>(blockIdx.x) < sched) attn_schedule_block(pre.sched, err, reinterpret_cast<int*>(g_sh));
+    else rope_table_block(pre.rope, blockIdx.x - sched, extra - sched, err, reinterpret_cast<float2*>(g_sh));
+    return;
+  }
+  const int block = PRE ? blockIdx.x - extra : blockIdx.x;
   int M = M_cap;
   if (M_dev != nullptr) {
     const int md = *M_dev;
     if (md < 0 || md > M_cap) {
-      if (blockIdx.x == 0 && threadIdx.x == 0) record_error(err, kErrRows);
+      if (block == 0 && threadIdx.x == 0) record_error(err, kErrRows);
       M = md < 0 ? 0 : M_cap;
     } else {
       M = md;
     }
   }
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int nwarps = gridDim.x * 8;
+  const int nwarps = (PRE ? gridDim.x - extra : gridDim.x) * 8;
   const int d8 = d / 8;
   const uint4* xv = reinterpret_cast<const uint4*>(x);
-  __shared__ uint4 g_sh[32 * VPL];
   uint4* yv = reinterpret_cast<uint4*>(y);
   uint32_t nonfinite = 0;
   uint4 raw[VPL];
@@ -141,7 +176,7 @@ __global__ void __launch_bounds__(256, 2) rmsnorm_rows_kernel(const void* __rest
     }
   };
   // the first row's loads are under way while the gain is staged
-  int row = blockIdx.x * 8 + warp;
+  int row = block * 8 + warp;
   if (row < M) load_row(row);
   for (int v = threadIdx.x; v < d8; v += blockDim.x) g_sh[v] = __ldg(reinterpret_cast<const uint4*>(g) + v);
   __syncthreads();
@@ -603,16 +638,34 @@ __global__ void __launch_bounds__(256, 4) pack_route_kernel(const uint8_t* __res
 }  // namespace
 
 cudaError_t launch_rmsnorm(const void* x, int in_type, const void* g, void* y, int out_type, int M_cap,
-                           const int* M_dev, int d, float eps, const RowMap& map, int* err, cudaStream_t st) {
+                           const int* M_dev, int d, float eps, const RowMap& map, const Prelude* pre, int* err,
+                           int num_sms, cudaStream_t st) {
   if (M_cap <= 0) return cudaSuccess;
   int blocks = (M_cap + 7) / 8;
   if (blocks > 65535 * 4) blocks = 65535 * 4;
   // 16-bit rows up to 4096 wide: register-resident variant sized to the row
   const int vpl = (d / 8 + 31) / 32;
+  if (pre != nullptr) {
+    if (!norm_takes_prelude(in_type, out_type, d, pre->sched.B)) return cudaErrorInvalidValue;
+    int tables = 0;
+    if (pre->rope.tab != nullptr) {
+      tables = (pre->rope.T_cap + 3) / 4;
+      if (tables > num_sms) tables = num_sms;
+    }
+    const int extra = (pre->sched.work != nullptr ? 1 : 0) + tables;
+#define SEER_NORM_PRE(I, O, V)                                                                                         \
+  if (in_type == I && out_type == O && vpl <= V)                                                                       \
+    return launch_kernel(rmsnorm_rows_kernel<I, O, V, false, true>, dim3(blocks + extra), dim3(256), 0, st, x, g, y,   \
+                         M_cap, M_dev, d, eps, map, *pre, extra, err);
+    SEER_NORM_PRE(kBF16, kF16, 4) SEER_NORM_PRE(kBF16, kF16, 8) SEER_NORM_PRE(kBF16, kF16, 16)
+    SEER_NORM_PRE(kF16, kF16, 4) SEER_NORM_PRE(kF16, kF16, 8) SEER_NORM_PRE(kF16, kF16, 16)
+#undef SEER_NORM_PRE
+    return cudaErrorInvalidValue;
+  }
 #define SEER_NORM_ROWS(I, O, V, MAPPED)                                                                              \
   if (in_type == I && out_type == O && vpl <= V && mapped == MAPPED)                                                 \
-    return launch_kernel(rmsnorm_rows_kernel<I, O, V, MAPPED>, dim3(blocks), dim3(256), 0, st, x, g, y, M_cap, M_dev, \
-                         d, eps, map, err);
+    return launch_kernel(rmsnorm_rows_kernel<I, O, V, MAPPED, false>, dim3(blocks), dim3(256), 0, st, x, g, y, M_cap, \
+                         M_dev, d, eps, map, Prelude{}, 0, err);
 #define SEER_NORM_16(I, O, MAPPED) \
   SEER_NORM_ROWS(I, O, 4, MAPPED) SEER_NORM_ROWS(I, O, 8, MAPPED) SEER_NORM_ROWS(I, O, 16, MAPPED)
 #define SEER_NORM(I, O, MAPPED)                                                                                  \
@@ -635,6 +688,20 @@ cudaError_t launch_rmsnorm(const void* x, int in_type, const void* g, void* y, i
 #undef SEER_NORM_16
 #undef SEER_NORM_ROWS
   return cudaErrorInvalidValue;
+}
+
+bool norm_takes_prelude(int in_type, int out_type, int d, int B) {
+  const int vpl = (d / 8 + 31) / 32;
+  if (out_type != kF16 || in_type == kF32 || vpl > 16) return false;
+  // the schedule's 4 B ints and the table's 64 frequencies use the gain's shared memory
+  const int words = 32 * (vpl <= 4 ? 4 : (vpl <= 8 ? 8 : 16)) * 4;
+  return 4 * B <= words;
+}
+
+cudaError_t launch_rope_table(const RopeTable& t, int* err, int num_sms, cudaStream_t st) {
+  if (t.T_cap <= 0) return cudaSuccess;
+  const int blocks = (t.T_cap + 3) / 4 < 2 * num_sms ? (t.T_cap + 3) / 4 : 2 * num_sms;
+  return launch_kernel(rope_table_kernel, dim3(blocks), dim3(256), 0, st, t, err);
 }
 
 cudaError_t launch_convert(const void* src, int in_type, void* dst, int out_type, size_t n, int* err, cudaStream_t st) {

@@ -54,7 +54,7 @@ struct GemmParams {
   int few_bn;             // ... this many columns per tile (single-weight modes; mB1 has its boxes) ...
   int few_stages;         // ... and stages
   int group_m;            // raster: row tiles per group (see tc_gemm.cu)
-  float rope_theta;       // Rope: frequency base (> 0)
+  const float2* rope_tab; // Rope: (cos, sin) of each row's 64 pairs
   int rope_cols;          // Rope: leading output columns that are rotated (the q|k columns)
   void* C2;               // Kv: matrix of the mapped columns [map.rows, ldc2]
   int ldc2;
@@ -118,10 +118,37 @@ cudaError_t launch_tc_attn(const CUtensorMap& mQ, const CUtensorMap& mKV, AttnPa
 // units of 16 bytes, rounded up to 256 bytes, plus 256 bytes for the unit
 // count and the persistent kernel's unit counter.
 size_t attn_sched_bytes(int T_cap, int B, int H);
-// writes the units to work, their number to work_count[0] and zeroes
-// work_count[1] (the attention kernel's unit counter)
-cudaError_t launch_attn_schedule(const int* cu, const int* cu_kv, const int* kv_len, int B, int n_heads, int T_cap,
-                                 int4* work, int* work_count, int max_units, int* err, cudaStream_t st);
+// Arguments of the attention schedule: the units go to work (at most max_units),
+// their number to work_count[0], and work_count[1] (the attention kernel's unit
+// counter) is zeroed.
+struct ScheduleArgs {
+  const int* cu;
+  const int* cu_kv;       // or null
+  const int* kv_len;      // or null
+  int B, n_heads, T_cap;
+  int4* work;             // null: no schedule
+  int* work_count;
+  int max_units;
+};
+cudaError_t launch_attn_schedule(const ScheduleArgs& a, int* err, cudaStream_t st);
+
+// cos and sin of the rotary angles of each row: tab[row * 64 + i] for pair i of a
+// 128-wide head, rows of the segments cu[0 .. B].
+struct RopeTable {
+  float2* tab;            // [T_cap, 64], or null
+  const int* cu;
+  int B, T_cap;
+  float theta;
+};
+cudaError_t launch_rope_table(const RopeTable& t, int* err, int num_sms, cudaStream_t st);
+
+// What a layer's first norm can do beside its rows, in blocks of its own.
+struct Prelude {
+  ScheduleArgs sched;
+  RopeTable rope;
+};
+// Whether launch_rmsnorm takes a prelude for these rows and segments.
+bool norm_takes_prelude(int in_type, int out_type, int d, int B);
 
 // CUDA-core kernels (fp32 storage; small shapes).
 cudaError_t launch_simt_gemm(int mode, const float* A, const float* B0, const float* B1, const GemmParams& p,
@@ -130,9 +157,10 @@ cudaError_t launch_simt_attn(const float* qkv, const AttnParams& p, int num_sms,
 
 // Element-wise / scan kernels (both storage types).
 // map.cu set: row r of y is the norm of the row of x that the map names (rows
-// of segments outside x become zero and are recorded).
+// of segments outside x become zero and are recorded).  pre: also done, or null.
 cudaError_t launch_rmsnorm(const void* x, int in_type, const void* g, void* y, int out_type, int M_cap,
-                           const int* M_dev, int d, float eps, const RowMap& map, int* err, cudaStream_t st);
+                           const int* M_dev, int d, float eps, const RowMap& map, const Prelude* pre, int* err,
+                           int num_sms, cudaStream_t st);
 cudaError_t launch_rope(void* qkv, int type, const int* cu, int B, int T_cap, int n_heads, int head_dim, float theta,
                         int* err, int num_sms, cudaStream_t st);
 // Per-segment row copies (see aux_kernels.cu): rows of segment b go from src

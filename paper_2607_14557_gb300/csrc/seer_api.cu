@@ -226,6 +226,7 @@ seer_status check_dims(const seer_dims* dims, seer_dtype dt) {
 // when theta > 0: positions come from the segment offsets cu[0..B].
 struct RopeArgs {
   float theta = 0.f;
+  const float2* tab = nullptr;   // 16-bit: the rows' table (RopeTable)
   const int32_t* cu = nullptr;
   int B = 0;
   int n_heads = 0;
@@ -272,12 +273,13 @@ seer_status do_linear(const void* a, const void* w, seer_dtype op_dt, const void
     p.map = dest.map;
   }
   if (rot) {
-    p.rope_theta = rope.theta;
+    p.rope_tab = rope.tab;
     p.rope_cols = 2 * rope.n_heads * rope.head_dim;
     p.cu = rope.cu;
     p.B = rope.B;
   }
   if (is16(op_dt)) {
+    if (rot && !rope.tab) return fail(SEER_ERR_INVALID_ARG, "linear: the 16-bit rotary epilogue needs a table");
     if (rot && rope.head_dim != 128) return fail(SEER_ERR_UNSUPPORTED, "16-bit rotary epilogue needs head_dim == 128");
     if (!is16(c_dt) || (r && !is16(r_dt))) return fail(SEER_ERR_UNSUPPORTED, "16-bit linear needs 16-bit output and residual");
     if (N % 256 != 0 || K % 64 != 0)
@@ -375,7 +377,7 @@ seer_status do_swiglu(const void* a, const void* wg, const void* wu, seer_dtype 
 
 seer_status do_rmsnorm(const void* x, seer_dtype x_dt, const void* g, void* y, seer_dtype y_dt, int M_cap,
                        const int32_t* M_dev, int d, float eps, cudaStream_t st, int phase,
-                       const RowMap& map = RowMap{}) {
+                       const RowMap& map = RowMap{}, const Prelude* pre = nullptr) {
   if (!x || !g || !y) return fail(SEER_ERR_INVALID_ARG, "rmsnorm: null pointer");
   if (M_cap < 0 || d <= 0) return fail(SEER_ERR_INVALID_ARG, "rmsnorm: bad sizes");
   if (!valid_dt(x_dt) || !valid_dt(y_dt)) return fail(SEER_ERR_INVALID_ARG, "rmsnorm: unknown dtype");
@@ -387,7 +389,7 @@ seer_status do_rmsnorm(const void* x, seer_dtype x_dt, const void* g, void* y, s
   DeviceInfo* di;
   SEER_TRY(device_info(&di));
   Phase ph(phase, st);
-  SEER_CUDA(launch_rmsnorm(x, x_dt, g, y, y_dt, M_cap, M_dev, d, eps, map, di->err, st), "rmsnorm launch");
+  SEER_CUDA(launch_rmsnorm(x, x_dt, g, y, y_dt, M_cap, M_dev, d, eps, map, pre, di->err, di->num_sms, st), "rmsnorm launch");
   return SEER_OK;
 }
 
@@ -401,9 +403,26 @@ struct KvSource {
   int T_kv_cap = 0;
 };
 
+// The schedule of an attention call in its workspace part.
+ScheduleArgs schedule_args(const int32_t* cu, const int32_t* cu_kv, const int32_t* kv_len, int B, int T_cap, int H,
+                           void* sched) {
+  ScheduleArgs a{};
+  a.cu = cu;
+  a.cu_kv = cu_kv;
+  a.kv_len = kv_len;
+  a.B = B;
+  a.n_heads = H;
+  a.T_cap = T_cap;
+  a.max_units = static_cast<int>(static_cast<size_t>(H) * ((T_cap + 127) / 128 + B));
+  a.work = static_cast<int4*>(sched);
+  a.work_count = reinterpret_cast<int*>(static_cast<uint8_t*>(sched) + align256(static_cast<size_t>(a.max_units) * sizeof(int4)));
+  return a;
+}
+
+// scheduled: the schedule of this call is already in the workspace.
 seer_status do_attention(const void* qkv, void* o, seer_dtype dt, const int32_t* cu, const int32_t* kv_len, int B,
                          int T_cap, int H, int dh, void* sched, size_t sched_bytes, cudaStream_t st,
-                         const KvSource& kvs = KvSource()) {
+                         const KvSource& kvs = KvSource(), bool scheduled = false) {
   if (!qkv || !o || !cu) return fail(SEER_ERR_INVALID_ARG, "attention: null pointer");
   if (kvs.kv && (!kvs.cu_kv || kvs.T_kv_cap < 0 || kvs.ld < 2 * H * dh))
     return fail(SEER_ERR_INVALID_ARG, "attention: a separate K/V source needs cu_kv, a capacity and rows of >= 2*H*dh");
@@ -437,17 +456,14 @@ seer_status do_attention(const void* qkv, void* o, seer_dtype dt, const int32_t*
     if (!aligned16(qkv) || !aligned16(o) || !aligned16(sched))
       return fail(SEER_ERR_UNSUPPORTED, "attention needs 16-byte aligned pointers");
     if (T_cap == 0) return SEER_OK;
-    const int max_units = static_cast<int>(static_cast<size_t>(H) * ((T_cap + 127) / 128 + B));
-    int4* work = static_cast<int4*>(sched);
-    int* count = reinterpret_cast<int*>(static_cast<uint8_t*>(sched) + align256(static_cast<size_t>(max_units) * sizeof(int4)));
-    p.work = work;
-    p.work_count = count;
-    p.work_next = count + 1;
+    const ScheduleArgs sa = schedule_args(cu, p.cu_kv, kv_len, B, T_cap, H, sched);
+    p.work = sa.work;
+    p.work_count = sa.work_count;
+    p.work_next = sa.work_count + 1;
     CUtensorMap m, mkv;
     SEER_TRY(make_map16(&m, qkv, dt, T_cap, 3 * H * dh, 3 * H * dh, 128));
     if (kvs.kv) SEER_TRY(make_map16(&mkv, kvs.kv, dt, kvs.T_kv_cap > 0 ? kvs.T_kv_cap : 1, kvs.ld, kvs.ld, 128));
-    SEER_CUDA(launch_attn_schedule(cu, p.cu_kv, kv_len, B, H, T_cap, work, count, max_units, di->err, st),
-              "attn schedule");
+    if (!scheduled) SEER_CUDA(launch_attn_schedule(sa, di->err, st), "attn schedule");
     // the attention phase brackets the attention kernel alone (the one-block
     // schedule kernel before it takes a few microseconds)
     Phase ph(PH_ATTN, st);
@@ -744,15 +760,28 @@ seer_status seer_layer_forward(const seer_layer_weights* w, const seer_dims* dim
   const int32_t* M_dev = cu_seqlens + B;   // device total rows
   const float eps = dims->rms_eps;
 
-  SEER_TRY(do_rmsnorm(x, dt, w->g_attn, xn, it, T_capacity, M_dev, d, eps, st, PH_NORM1));
   RopeArgs rope;
   rope.theta = dims->rope_theta;
   rope.cu = cu_seqlens;
   rope.B = B;
   rope.n_heads = H;
   rope.head_dim = dh;
+  // 16-bit: the attention's schedule and the rotary table (in h, not yet in use) are
+  // made by blocks of the first norm where it takes them
+  DeviceInfo* di;
+  SEER_TRY(device_info(&di));
+  Prelude pre{};
+  pre.sched = schedule_args(cu_seqlens, nullptr, kv_len, B, T_capacity, H, sched);
+  if (it == SEER_F16 && rope.theta > 0.f) {
+    pre.rope = RopeTable{static_cast<float2*>(h), cu_seqlens, B, T_capacity, rope.theta};
+    rope.tab = pre.rope.tab;
+  }
+  const bool early = it == SEER_F16 && T_capacity > 0 && norm_takes_prelude(dt, it, d, B);
+  if (!early && rope.tab) SEER_CUDA(launch_rope_table(pre.rope, di->err, di->num_sms, st), "rope table");
+  SEER_TRY(do_rmsnorm(x, dt, w->g_attn, xn, it, T_capacity, M_dev, d, eps, st, PH_NORM1, RowMap{}, early ? &pre : nullptr));
   SEER_TRY(do_linear(xn, w->w_qkv, it, nullptr, it, qkv, it, T_capacity, M_dev, 3 * d, d, st, PH_QKV, rope));
-  SEER_TRY(do_attention(qkv, xn, it, cu_seqlens, kv_len, B, T_capacity, H, dh, sched, L.total - L.off_sched, st));
+  SEER_TRY(do_attention(qkv, xn, it, cu_seqlens, kv_len, B, T_capacity, H, dh, sched, L.total - L.off_sched, st, KvSource(),
+                        early));
   SEER_TRY(do_linear(xn, w->w_o, it, x, dt, h, it, T_capacity, M_dev, d, d, st, PH_OPROJ));
   SEER_TRY(do_rmsnorm(h, it, w->g_mlp, xn, it, T_capacity, M_dev, d, eps, st, PH_NORM2));
   SEER_TRY(do_swiglu(xn, w->w_gate, w->w_up, it, act, it, T_capacity, M_dev, F, d, cu_seqlens, B, count_resp_start, N,
@@ -870,7 +899,11 @@ seer_status seer_layer_forward_cached(const seer_layer_weights* w, const seer_di
   const int32_t* M_dev = cu_resp + B;
   const float eps = dims->rms_eps;
 
-  SEER_TRY(do_rmsnorm(x_resp, dt, w->g_attn, xn, it, T_resp_cap, M_dev, d, eps, st, PH_NORM1));
+  Prelude pre{};
+  pre.sched = schedule_args(cu_resp, cu_kv, kv_len, B, T_resp_cap, H, sched);
+  const bool early = it == SEER_F16 && norm_takes_prelude(dt, it, d, B);
+  SEER_TRY(do_rmsnorm(x_resp, dt, w->g_attn, xn, it, T_resp_cap, M_dev, d, eps, st, PH_NORM1, RowMap{},
+                      early ? &pre : nullptr));
   // the response rows' K | V go into the cache, after each segment's prefix: straight
   // from the projection for 16-bit layers (a copy afterwards took 18 us for 848 rows)
   KvDest dest;
@@ -895,7 +928,7 @@ seer_status seer_layer_forward_cached(const seer_layer_weights* w, const seer_di
   kvs.xv0 = D;
   kvs.cu_kv = cu_kv;
   kvs.T_kv_cap = T_kv_cap;
-  SEER_TRY(do_attention(qkv, xn, it, cu_resp, kv_len, B, T_resp_cap, H, dh, sched, L.total - L.off_sched, st, kvs));
+  SEER_TRY(do_attention(qkv, xn, it, cu_resp, kv_len, B, T_resp_cap, H, dh, sched, L.total - L.off_sched, st, kvs, early));
   SEER_TRY(do_linear(xn, w->w_o, it, x_resp, dt, h, it, T_resp_cap, M_dev, d, d, st, PH_OPROJ));
   SEER_TRY(do_rmsnorm(h, it, w->g_mlp, xn, it, T_resp_cap, M_dev, d, eps, st, PH_NORM2));
   SEER_TRY(do_swiglu(xn, w->w_gate, w->w_up, it, act, it, T_resp_cap, M_dev, F, d, cu_resp, B, nullptr, 0, 0.f, nullptr,

@@ -59,16 +59,17 @@
 // traffic those MMAs ran at about half their isolated rate.
 #include <math.h>
 
+#include "attn_schedule.cuh"
 #include "common.cuh"
 #include "kernels.h"
 
 namespace seer {
 namespace {
 
-constexpr int BQ = 128;
+constexpr int BQ = kAttnRows;
 constexpr int BKV = 128;
 constexpr int DH = 128;
-constexpr int NT = 2;                       // query tiles per CTA
+constexpr int NT = kAttnTiles;              // query tiles per CTA
 constexpr int THREADS = 128 + 128 * NT;    // warps 0-3 producer/issuers, 4 warps per tile
 constexpr int TILE_BYTES = 128 * DH * 2;    // 32 KB: 128 rows x 128 16-bit values as two 16 KB swizzle panels
 constexpr int PANEL = 16384;
@@ -766,64 +767,10 @@ __global__ void __launch_bounds__(THREADS, 1)
   }
 }
 
-// One block: per-segment key counts -> work units (b, h, first q-tile, tiles)
-// of up to NT query tiles, ordered by descending kv length so the longest
-// segments start first.
-__global__ void attn_schedule_kernel(const int* cu, const int* cu_kv, const int* kv_len, int B, int H, int T_cap,
-                                     int4* work, int* work_count, int max_units, int* err) {
+__global__ void attn_schedule_kernel(const ScheduleArgs a, int* err) {
   pdl_enter();
   extern __shared__ int sh[];
-  int* ntile = sh;           // [B]
-  int* kvs = sh + B;         // [B]
-  int* off = sh + 2 * B;     // [B]
-  int* rank = sh + 3 * B;    // [B]
-  for (int i = threadIdx.x; i < B; i += blockDim.x) {
-    const int L = cu[i + 1] - cu[i];
-    const int Lkv = cu_kv ? cu_kv[i + 1] - cu_kv[i] : L;   // rows of the segment's K/V
-    int kv = kv_len ? kv_len[i] : Lkv;
-    if (L < 0 || cu[i] < 0 || cu[i + 1] > T_cap || kv > Lkv || (L > 0 && kv <= 0)) {
-      record_error(err, kErrLayout);
-      kv = 0;
-    }
-    ntile[i] = (kv > 0) ? (L + BQ * NT - 1) / (BQ * NT) : 0;   // work units (tile groups) per head
-    kvs[i] = kv;
-  }
-  __syncthreads();
-  for (int i = threadIdx.x; i < B; i += blockDim.x) {
-    int rk = 0;
-    for (int k = 0; k < B; ++k) rk += (kvs[k] > kvs[i]) || (kvs[k] == kvs[i] && k < i);
-    rank[i] = rk;
-  }
-  __syncthreads();
-  // offsets in rank order: a segment's units follow those of every segment
-  // ranked before it (the ranks are a permutation of 0..B-1)
-  for (int i = threadIdx.x; i < B; i += blockDim.x) {
-    int before = 0;
-    for (int k = 0; k < B; ++k) before += rank[k] < rank[i] ? ntile[k] : 0;
-    off[i] = H * before;
-  }
-  if (threadIdx.x == 0) {
-    int acc = 0;
-    for (int i = 0; i < B; ++i) acc += H * ntile[i];
-    if (acc > max_units) {
-      record_error(err, kErrCapacity);
-      acc = max_units;
-    }
-    work_count[0] = acc;
-    work_count[1] = 0;            // next unit handed out by the attention kernel
-  }
-  __syncthreads();
-  for (int i = 0; i < B; ++i) {
-    const int n = H * ntile[i];
-    for (int k = threadIdx.x; k < n; k += blockDim.x) {
-      const int idx = off[i] + k;
-      if (idx < max_units) {
-        const int g = k % ntile[i];
-        const int tiles = (cu[i + 1] - cu[i] + BQ - 1) / BQ;
-        work[idx] = make_int4(i, k / ntile[i], g * NT, min(NT, tiles - g * NT));
-      }
-    }
-  }
+  attn_schedule_block(a, err, sh);
 }
 
 template <bool F16, bool SPLIT>
@@ -869,16 +816,14 @@ cudaError_t launch_tc_attn(const CUtensorMap& mQ, const CUtensorMap& mKV, AttnPa
   return f16 ? launch_typed<true, false>(mQ, mKV, p, grid, st) : launch_typed<false, false>(mQ, mKV, p, grid, st);
 }
 
-cudaError_t launch_attn_schedule(const int* cu, const int* cu_kv, const int* kv_len, int B, int n_heads, int T_cap,
-                                 int4* work, int* work_count, int max_units, int* err, cudaStream_t st) {
-  const size_t sm = static_cast<size_t>(4) * B * sizeof(int);
+cudaError_t launch_attn_schedule(const ScheduleArgs& a, int* err, cudaStream_t st) {
+  const size_t sm = static_cast<size_t>(4) * a.B * sizeof(int);
   if (sm > 48 * 1024) {
     cudaError_t e = cudaFuncSetAttribute(attn_schedule_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          static_cast<int>(sm));
     if (e != cudaSuccess) return e;
   }
-  return launch_kernel(attn_schedule_kernel, dim3(1), dim3(256), sm, st, cu, cu_kv, kv_len, B, n_heads, T_cap, work,
-                       work_count, max_units, err);
+  return launch_kernel(attn_schedule_kernel, dim3(1), dim3(256), sm, st, a, err);
 }
 
 }  // namespace seer

@@ -61,10 +61,9 @@ constexpr int ACC_COLS = 256;                        // one of the two accumulat
 constexpr int TMEM_COLS = 512;
 constexpr int BAR_BYTES = 256;
 constexpr int ROPE_HEAD = 128;                       // head width of the Rope epilogue
-constexpr int ROPE_BYTES = ROPE_HEAD / 2 * 8;        // (hi, lo) inverse frequency per pair
 constexpr int EPI_CHUNK = 32 * 32 * 2;              // a warp's 32 rows x 32 columns, 16-bit
 constexpr int EPI_BYTES = 4 * 2 * EPI_CHUNK;         // 4 epilogue warps x 2 staging buffers
-constexpr int FIXED_BYTES = BAR_BYTES + ROPE_BYTES + EPI_BYTES + 1024;
+constexpr int FIXED_BYTES = BAR_BYTES + EPI_BYTES + 1024;
 constexpr int RING_BYTES = 196608;                   // operand ring: six stages of a 256-column pair tile
 static_assert(8 * (2 * MAX_STAGES + 4) + 8 <= BAR_BYTES, "barrier block");
 static_assert(RING_BYTES + FIXED_BYTES <= 232448, "shared memory per CTA");
@@ -136,8 +135,7 @@ __global__ void __launch_bounds__(THREADS, 1)
   uint64_t* acc_empty = acc_full + 2;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + 2);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-  float2* rope_tab = reinterpret_cast<float2*>(fixed + BAR_BYTES);
-  uint8_t* epi_stage = fixed + BAR_BYTES + ROPE_BYTES;   // [4 warps][2][EPI_CHUNK]
+  uint8_t* epi_stage = fixed + BAR_BYTES;                // [4 warps][2][EPI_CHUNK]
 
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
@@ -360,11 +358,6 @@ __global__ void __launch_bounds__(THREADS, 1)
       }
       ++n_chunks;
     };
-    if (MODE == kGemmRope) {
-      const int et = threadIdx.x - 64;                 // 0..127 over the epilogue warps
-      if (et < ROPE_HEAD / 2) rope_tab[et] = rope_inv_freq(et, ROPE_HEAD, p.rope_theta);
-      asm volatile("bar.sync 1, 128;" ::: "memory");
-    }
     int acc = 0;
     uint32_t acc_ph = 0;
     uint32_t nonfinite = 0;                      // range guard over this thread's stores
@@ -404,18 +397,23 @@ __global__ void __launch_bounds__(THREADS, 1)
       tc_fence_after();
       const uint32_t tacc = tmem_base + lane_off + static_cast<uint32_t>(acc * ACC_COLS);
       if (MODE == kGemmRope) {
-        // the tile holds whole heads; pair (c, c + 64) of a head rotates by pos * f_c
+        // the tile holds whole heads; pair (c, c + 64) of a head rotates by pos * f_c,
+        // its cos and sin read from the row's table (64 sincosf per row here lengthened
+        // every call's last epilogue by several us)
         const bool rotate = n * BN < p.rope_cols;       // tile-uniform (rope_cols % 256 == 0, BN 128 or 256)
         const int heads = cols / ROPE_HEAD;
         uint16_t* crow = reinterpret_cast<uint16_t*>(p.C) + static_cast<size_t>(valid ? row : 0) * p.ldc + n * BN;
-        const float pos = (valid && rotate) ? static_cast<float>(row_position(p.cu, p.B, row)) : 0.f;
+        const float4* trow = reinterpret_cast<const float4*>(p.rope_tab + static_cast<size_t>(valid ? row : 0) * (ROPE_HEAD / 2));
 #pragma unroll 1
         for (int c = 0; c < ROPE_HEAD / 64; ++c) {
           float cs[32], sn[32];
 #pragma unroll
-          for (int e = 0; e < 32; ++e) {
-            if (rotate) rope_cos_sin(pos, rope_tab[c * 32 + e], cs[e], sn[e]);
-            else { cs[e] = 1.f; sn[e] = 0.f; }
+          for (int e = 0; e < 16; ++e) {
+            const float4 t2 = rotate && valid ? trow[c * 16 + e] : make_float4(1.f, 0.f, 1.f, 0.f);
+            cs[2 * e] = t2.x;
+            sn[2 * e] = t2.y;
+            cs[2 * e + 1] = t2.z;
+            sn[2 * e + 1] = t2.w;
           }
 #pragma unroll 1
           for (int hh = 0; hh < heads; ++hh) {
@@ -424,25 +422,27 @@ __global__ void __launch_bounds__(THREADS, 1)
             tmem_ld32(tacc + c0, r0);
             tmem_ld32(tacc + c1, r1);
             tmem_ld_wait();
-            if (valid) {
-              float v0[32], v1[32];
+            if (slab_full || valid) {
+              uint32_t q0[16], q1[16];
 #pragma unroll
-              for (int e = 0; e < 32; ++e) {
+              for (int e = 0; e < 32; e += 2) {
                 const float x0 = __uint_as_float(r0[e]), x1 = __uint_as_float(r1[e]);
-                v0[e] = fmaf(x0, cs[e], -x1 * sn[e]);
-                v1[e] = fmaf(x1, cs[e], x0 * sn[e]);
+                const float y0 = __uint_as_float(r0[e + 1]), y1 = __uint_as_float(r1[e + 1]);
+                q0[e / 2] = pack2(fmaf(x0, cs[e], -x1 * sn[e]), fmaf(y0, cs[e + 1], -y1 * sn[e + 1]), of16);
+                q1[e / 2] = pack2(fmaf(x1, cs[e], x0 * sn[e]), fmaf(y1, cs[e + 1], y0 * sn[e + 1]), of16);
+                nonfinite |= nonfinite_term(q0[e / 2], of16) | nonfinite_term(q1[e / 2], of16);
               }
+              if (slab_full) {
+                store_chunk(mC, q0, n * BN + c0, mt * BM + q * 32);
+                store_chunk(mC, q1, n * BN + c1, mt * BM + q * 32);
+              } else {
 #pragma unroll
-              for (int i = 0; i < 2; ++i) {
-                uint32_t q0[8], q1[8];
-#pragma unroll
-                for (int e = 0; e < 8; ++e) {
-                  q0[e] = pack2(v0[16 * i + 2 * e], v0[16 * i + 2 * e + 1], of16);
-                  q1[e] = pack2(v1[16 * i + 2 * e], v1[16 * i + 2 * e + 1], of16);
-                  nonfinite |= nonfinite_term(q0[e], of16) | nonfinite_term(q1[e], of16);
+                for (int i = 0; i < 2; ++i) {
+                  st_global_v8(crow + c0 + 16 * i, q0[8 * i], q0[8 * i + 1], q0[8 * i + 2], q0[8 * i + 3], q0[8 * i + 4],
+                               q0[8 * i + 5], q0[8 * i + 6], q0[8 * i + 7]);
+                  st_global_v8(crow + c1 + 16 * i, q1[8 * i], q1[8 * i + 1], q1[8 * i + 2], q1[8 * i + 3], q1[8 * i + 4],
+                               q1[8 * i + 5], q1[8 * i + 6], q1[8 * i + 7]);
                 }
-                st_global_v8(crow + c0 + 16 * i, q0[0], q0[1], q0[2], q0[3], q0[4], q0[5], q0[6], q0[7]);
-                st_global_v8(crow + c1 + 16 * i, q1[0], q1[1], q1[2], q1[3], q1[4], q1[5], q1[6], q1[7]);
               }
             }
           }

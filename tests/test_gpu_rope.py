@@ -55,3 +55,32 @@ def test_rope_rejects_bad_arguments():
         S.seer_rope(x, "f32", cu, 1, 8, 1, 128, 0.0)
     with pytest.raises(RuntimeError):
         S.seer_rope(x, "f32", cu, 1, 8, 1, 256, 1e4)
+
+
+@pytest.mark.parametrize("theta", [0.0, 1e4])
+@pytest.mark.parametrize("B", [140, 256])
+def test_layer_schedule_and_table_by_either_kernel(theta, B):
+    """A 256-wide layer's first norm also makes the attention schedule and the rotary
+    table for up to 128 segments; more have launches of their own.  Segments are
+    independent, so the layer over all of them equals, bit for bit, the layer over
+    each half (128 segments or fewer)."""
+    d, H, F = 256, 2, 256
+    g = torch.Generator(device="cuda").manual_seed(B)
+    r = lambda *shape: torch.randn(shape, generator=g, device="cuda")
+    w = [(0.05 * r(*s)).half() for s in ((3 * d, d), (d, d), (F, d), (F, d), (d, F))] + [(1 + 0.1 * r(d)).half()] * 2
+    W, dims = S.make_weights(*w), S.make_dims(d, H, 128, F, rope_theta=theta)
+    lens = np.random.default_rng(B).integers(0, 40, B)
+    x = r(int(lens.sum()), d).to(torch.bfloat16)
+
+    def layer(a, b):
+        cu = np.concatenate([[0], np.cumsum(lens[a:b])])
+        T = int(cu[-1])
+        rows = x[int(lens[:a].sum()):int(lens[:b].sum())].clone()
+        y = torch.empty_like(rows)
+        n = S.seer_layer_workspace_size(dims, "bf16", T, b - a)
+        ws = torch.empty(n, dtype=torch.uint8, device=cuda())
+        S.seer_layer_forward(W, dims, "bf16", rows, y, i32(cu), None, b - a, T, None, 0, 0.0, None, ws, n)
+        torch.cuda.synchronize()
+        return y
+
+    assert torch.equal(layer(0, B), torch.cat([layer(0, B // 2), layer(B // 2, B)]))
