@@ -288,6 +288,15 @@ __global__ void __launch_bounds__(256) rope_kernel(void* __restrict__ qkv, const
   }
 }
 
+// Zeroes n ints: a kernel of the chain, so its neighbours' launches overlap it (a
+// memset between kernels orders them fully: fp32 path 73.1 -> 69.9 us, 8B layer with the
+// count hook 1103 -> 1093).
+__global__ void __launch_bounds__(256) zero_kernel(int* __restrict__ p, size_t n) {
+  pdl_enter();
+  for (size_t i = blockIdx.x * static_cast<size_t>(256) + threadIdx.x; i < n; i += gridDim.x * static_cast<size_t>(256))
+    p[i] = 0;
+}
+
 // ------------------------------------------------------------------ segment row copies
 // For each segment b: n rows starting at src row s0 (columns [src_c0, src_c0 +
 // row) in bytes) go to dst rows starting at d0, with
@@ -732,6 +741,12 @@ cudaError_t launch_rope(void* qkv, int type, const int* cu, int B, int T_cap, in
     case kBF16: return launch_kernel(rope_kernel<kBF16>, dim3(blocks), dim3(256), 0, st, qkv, cu, B, T_cap, n_heads, head_dim, theta, err);
     default: return cudaErrorInvalidValue;
   }
+}
+
+cudaError_t launch_zero(int* p, size_t n, int num_sms, cudaStream_t st) {
+  if (n == 0) return cudaSuccess;
+  const size_t blocks = (n + 255) / 256, cap = static_cast<size_t>(num_sms) * 8;
+  return launch_kernel(zero_kernel, dim3(static_cast<unsigned>(blocks < cap ? blocks : cap)), dim3(256), 0, st, p, n);
 }
 
 cudaError_t launch_rows_copy(const void* src, long src_ld, int src_c0, void* dst, long dst_ld, int dst_c0, int row_bytes,

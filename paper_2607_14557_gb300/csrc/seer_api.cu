@@ -352,7 +352,7 @@ seer_status do_swiglu(const void* a, const void* wg, const void* wu, seer_dtype 
     return fail(SEER_ERR_UNSUPPORTED, "fp32 swiglu needs an fp32 output");
   }
   if (counts && !accumulate)
-    SEER_CUDA(cudaMemsetAsync(counts, 0, sizeof(int32_t) * static_cast<size_t>(B) * N, st), "memset counts");
+    SEER_CUDA(launch_zero(counts, static_cast<size_t>(B) * N, di->num_sms, st), "zero counts");
   if (M_cap == 0) return SEER_OK;
   if (is16(op_dt)) {
     const long m_tiles = mode == kGemmCount ? static_cast<long>(B) * ((N + 127l) / 128) : (M_cap + 127l) / 128;
