@@ -75,7 +75,7 @@ struct AttnParams {
   int head_dim;
   void* out;              // [T, H*dh]
   int ldo;                // elements
-  const int4* work;       // schedule: (b, h, first q-tile, q-tiles)
+  const int4* work;       // schedule: (b, h, first q-tile, q-tiles), or null: made in the kernel
   const int* work_count;  // units in `work`
   int* work_next;         // next unit to hand out (zeroed by the schedule kernel)
   int kv_rows;            // rows of the K/V source (capacity)
@@ -113,6 +113,8 @@ int tc_attn_smem_bytes();
 // a cluster of CTAs per unit
 cudaError_t launch_tc_attn(const CUtensorMap& mQ, const CUtensorMap& mKV, AttnParams p, bool f16, int num_sms,
                            cudaStream_t st);
+// Whether the kernel makes the schedule of such a call itself (AttnParams::work null).
+bool attn_schedules_itself(int B, int n_heads, int T_cap, int num_sms);
 // Bytes of schedule workspace the 16-bit attention kernels need for a launch
 // sized for T_cap rows, B segments and H heads: H * (ceil(T_cap/128) + B) work
 // units of 16 bytes, rounded up to 256 bytes, plus 256 bytes for the unit

@@ -457,13 +457,16 @@ seer_status do_attention(const void* qkv, void* o, seer_dtype dt, const int32_t*
       return fail(SEER_ERR_UNSUPPORTED, "attention needs 16-byte aligned pointers");
     if (T_cap == 0) return SEER_OK;
     const ScheduleArgs sa = schedule_args(cu, p.cu_kv, kv_len, B, T_cap, H, sched);
-    p.work = sa.work;
-    p.work_count = sa.work_count;
-    p.work_next = sa.work_count + 1;
+    const bool inline_schedule = !scheduled && attn_schedules_itself(B, H, T_cap, di->num_sms);
+    if (!inline_schedule) {
+      p.work = sa.work;
+      p.work_count = sa.work_count;
+      p.work_next = sa.work_count + 1;
+    }
     CUtensorMap m, mkv;
     SEER_TRY(make_map16(&m, qkv, dt, T_cap, 3 * H * dh, 3 * H * dh, 128));
     if (kvs.kv) SEER_TRY(make_map16(&mkv, kvs.kv, dt, kvs.T_kv_cap > 0 ? kvs.T_kv_cap : 1, kvs.ld, kvs.ld, 128));
-    if (!scheduled) SEER_CUDA(launch_attn_schedule(sa, di->err, st), "attn schedule");
+    if (!scheduled && !inline_schedule) SEER_CUDA(launch_attn_schedule(sa, di->err, st), "attn schedule");
     // the attention phase brackets the attention kernel alone (the one-block
     // schedule kernel before it takes a few microseconds)
     Phase ph(PH_ATTN, st);

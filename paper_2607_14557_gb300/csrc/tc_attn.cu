@@ -6,8 +6,9 @@
 // beyond kv_len (bucket padding of the static path) are never keys.
 //
 // Work unit = (segment, head, pair of 128-query tiles).  Persistent CTAs, one
-// per SM (384 threads), take units from a global counter in schedule order
-// (longest segment first) until none are left; every ring and barrier phase
+// per SM (384 threads), take units in schedule order (longest segment first) until
+// none are left, from a global counter (each CTA one of every gridDim in alternating
+// direction instead: 3% slower on a ragged batch); every ring and barrier phase
 // runs on across units, so a unit's Q / K loads and first QK^T overlap the
 // previous unit's last PV and epilogue (a CTA per unit paid ~3.4 us of
 // setup and teardown per unit, the persistent loop ~0.3 us).
@@ -81,8 +82,12 @@ constexpr int OFF_K = NT * TILE_BYTES;
 constexpr int OFF_V = OFF_K + K_STAGES * TILE_BYTES;
 constexpr int OFF_BAR = OFF_V + V_STAGES * TILE_BYTES;
 constexpr int BAR_BYTES = 512;
-// 198144 bytes leave 60 KB of the SM to L1; 2 KB more would leave 28 (1.8% slower)
-constexpr int SMEM_BYTES = OFF_BAR + BAR_BYTES + 1024;
+constexpr int MAX_INLINE_B = 64;                           // segments of a schedule made in the kernel
+constexpr int OFF_SCHED = OFF_BAR + BAR_BYTES;             // four int arrays of MAX_INLINE_B (+ 1)
+constexpr int SCHED_BYTES = (4 * MAX_INLINE_B + 4) * 4;
+// up to 199680 bytes leave 60 KB of the SM to L1; more would leave 28 (1.8% slower)
+constexpr int SMEM_BYTES = OFF_SCHED + SCHED_BYTES + 1024;
+static_assert(SMEM_BYTES <= 199680, "L1 carve-out");
 static_assert(SMEM_BYTES <= 232448, "shared memory per CTA");
 constexpr uint32_t TMEM_COLS = 512;
 constexpr uint32_t TM_S = 0;                // S_t at TM_S + 128 t
@@ -172,15 +177,71 @@ struct Unit {
   int b, h, qt0, nt, seq0, L, kv0, kvL, q0, nkv, xq, xk, xv;
 };
 
-__device__ __forceinline__ Unit decode_unit(const AttnParams& p, int u) {
+// Schedule made by every CTA for itself, where no CTA gets a second unit: a kernel for
+// it alone took 2 us of a short call (32 heads of 420 rows 15.7 -> 13.8, 8 heads of 700 +
+// 700 17.9 -> 16.1).  Longer calls keep the list and its counter.  Segments by
+// descending key count as in attn_schedule_block; the units of the segment of rank r
+// are first[r] .. first[r + 1] - 1.
+struct InlineSchedule {
+  int* first;              // [B + 1]
+  int* seg;                // [B] segment of rank r
+};
+
+// All threads; returns the number of units.  scratch: two arrays of B ints.
+__device__ __forceinline__ int make_inline_schedule(const AttnParams& p, const InlineSchedule& s, int* scratch) {
+  int* kvs = scratch;
+  int* groups = scratch + MAX_INLINE_B;
+  const int i = threadIdx.x;
+  if (i < p.B) {
+    const int c0 = p.cu[i], c1 = p.cu[i + 1], L = c1 - c0;
+    const int Lkv = p.cu_kv ? p.cu_kv[i + 1] - p.cu_kv[i] : L;
+    int kv = p.kv_len ? p.kv_len[i] : Lkv;
+    if (L < 0 || c0 < 0 || c1 > p.T_cap || kv > Lkv || (L > 0 && kv <= 0)) {
+      record_error(p.err, kErrLayout);
+      kv = 0;
+    }
+    kvs[i] = kv;
+    groups[i] = kv > 0 ? (L + BQ * NT - 1) / (BQ * NT) : 0;
+  }
+  __syncthreads();
+  if (i < p.B) {
+    int rank = 0, before = 0;
+    for (int k = 0; k < p.B; ++k) {
+      const bool ahead = kvs[k] > kvs[i] || (kvs[k] == kvs[i] && k < i);
+      rank += ahead ? 1 : 0;
+      before += ahead ? groups[k] : 0;
+    }
+    s.seg[rank] = i;
+    s.first[rank] = p.n_heads * before;
+    if (rank == p.B - 1) s.first[p.B] = p.n_heads * (before + groups[i]);
+  }
+  __syncthreads();
+  return s.first[p.B];
+}
+
+template <bool INLINE>
+__device__ __forceinline__ Unit decode_unit(const AttnParams& p, const InlineSchedule& s, int u) {
   Unit d;
-  const int4 wk = p.work[u];
-  d.b = wk.x;
-  d.h = wk.y;
-  d.qt0 = wk.z;
-  d.nt = wk.w;
+  if (INLINE) {
+    int lo = 0, hi = p.B;
+    while (hi - lo > 1) {
+      const int mid = (lo + hi) >> 1;
+      if (s.first[mid] <= u) lo = mid; else hi = mid;
+    }
+    const int k = u - s.first[lo], groups = (s.first[lo + 1] - s.first[lo]) / p.n_heads;
+    d.b = s.seg[lo];
+    d.h = k / groups;
+    d.qt0 = (k - d.h * groups) * NT;
+  } else {
+    const int4 wk = p.work[u];
+    d.b = wk.x;
+    d.h = wk.y;
+    d.qt0 = wk.z;
+    d.nt = wk.w;
+  }
   d.seq0 = p.cu[d.b];
   d.L = p.cu[d.b + 1] - d.seq0;
+  if (INLINE) d.nt = min(NT, (d.L + BQ - 1) / BQ - d.qt0);
   d.kv0 = p.cu_kv ? p.cu_kv[d.b] : d.seq0;
   d.kvL = p.kv_len ? p.kv_len[d.b] : (p.cu_kv ? p.cu_kv[d.b + 1] - d.kv0 : d.L);
   d.q0 = d.seq0 + d.qt0 * BQ;
@@ -228,24 +289,26 @@ __device__ __forceinline__ int read_unit(uint64_t* u_full, uint64_t* u_empty, co
 // merged through distributed shared memory: every CTA leaves its unnormalised
 // rows of O and their (max, sum) in its own shared memory and combines 128 / parts
 // columns of all of them, in rank order.
-template <bool F16, bool SPLIT>
+template <bool F16, bool SPLIT, bool INLINE>
 __global__ void __launch_bounds__(THREADS, 1)
     tc_attn_kernel(const __grid_constant__ CUtensorMap mQ, const __grid_constant__ CUtensorMap mKV, const AttnParams p) {
   pdl_enter();
-  const int count = *p.work_count;
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  int* sched_smem = reinterpret_cast<int*>(smem + OFF_SCHED);
+  const InlineSchedule sched{sched_smem, sched_smem + MAX_INLINE_B + 1};
+  const int count = INLINE ? make_inline_schedule(p, sched, sched_smem + 2 * MAX_INLINE_B + 2) : *p.work_count;
   const int parts = SPLIT ? p.parts : 1;
   const int part = SPLIT ? static_cast<int>(cluster_ctarank()) : 0;
   const int first_unit = SPLIT ? static_cast<int>(blockIdx.x) / parts : static_cast<int>(blockIdx.x);
   if (first_unit >= count) return;                 // the same in every CTA of a cluster
   const int G = gridDim.x;
   const auto unit_at = [&](int u) {
-    const Unit d = decode_unit(p, u);
+    const Unit d = decode_unit<INLINE>(p, sched, u);
     return SPLIT ? split_unit(d, part, parts) : d;
   };
   const bool idle = SPLIT && unit_at(first_unit).nkv == 0;   // no key tiles for this CTA: it only merges
 
-  extern __shared__ uint8_t smem_raw[];
-  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + OFF_BAR);
   uint64_t* q_full = bars + 0;
   uint64_t* q_empty = bars + 1;              // both issuers are done with the Q tiles of a unit
@@ -341,7 +404,7 @@ __global__ void __launch_bounds__(THREADS, 1)
       if (n >= U_SLOTS && !warp_wait(&u_empty[sl], (n / U_SLOTS - 1) & 1, abort_flag, p.err)) break;
       int un = 0;
       if (leader) {
-        un = SPLIT ? -1 : G + atomicAdd(p.work_next, 1);
+        un = SPLIT || INLINE ? -1 : G + atomicAdd(p.work_next, 1);   // split / inline: one unit per cluster / CTA
         if (un >= count) un = -1;
         unit_slot[sl] = un;
         mbar_arrive(&u_full[sl]);
@@ -773,13 +836,13 @@ __global__ void attn_schedule_kernel(const ScheduleArgs a, int* err) {
   attn_schedule_block(a, err, sh);
 }
 
-template <bool F16, bool SPLIT>
+template <bool F16, bool SPLIT, bool INLINE>
 cudaError_t launch_typed(const CUtensorMap& mQ, const CUtensorMap& mKV, const AttnParams& p, int grid, cudaStream_t st) {
   static bool attr_set[64] = {};
-  cudaError_t e = set_smem_limit_once(tc_attn_kernel<F16, SPLIT>, SMEM_BYTES, attr_set);
+  cudaError_t e = set_smem_limit_once(tc_attn_kernel<F16, SPLIT, INLINE>, SMEM_BYTES, attr_set);
   if (e != cudaSuccess) return e;
   if (grid <= 0) return cudaSuccess;
-  return launch_kernel_overlap(launch_overlap_enabled(), p.parts, tc_attn_kernel<F16, SPLIT>, dim3(grid), dim3(THREADS),
+  return launch_kernel_overlap(launch_overlap_enabled(), p.parts, tc_attn_kernel<F16, SPLIT, INLINE>, dim3(grid), dim3(THREADS),
                                SMEM_BYTES, st, mQ, mKV, p);
 }
 
@@ -803,17 +866,27 @@ int attn_parts(long max_units, long kv_rows, int B) {
   return 1;
 }
 
+bool attn_schedules_itself(int B, int n_heads, int T_cap, int num_sms) {
+  return B <= MAX_INLINE_B && static_cast<long>(n_heads) * (T_cap / (NT * BQ) + B) <= num_sms;
+}
+
+namespace {
+template <bool SPLIT>
+cudaError_t launch_split(const CUtensorMap& mQ, const CUtensorMap& mKV, const AttnParams& p, bool f16, int grid,
+                         cudaStream_t st) {
+  if (p.work == nullptr)
+    return f16 ? launch_typed<true, SPLIT, true>(mQ, mKV, p, grid, st) : launch_typed<false, SPLIT, true>(mQ, mKV, p, grid, st);
+  return f16 ? launch_typed<true, SPLIT, false>(mQ, mKV, p, grid, st) : launch_typed<false, SPLIT, false>(mQ, mKV, p, grid, st);
+}
+}  // namespace
+
 cudaError_t launch_tc_attn(const CUtensorMap& mQ, const CUtensorMap& mKV, AttnParams p, bool f16, int num_sms,
                            cudaStream_t st) {
   const long max_units = static_cast<long>(p.n_heads) * (p.T_cap / (NT * BQ) + p.B);
   p.parts = attn_parts(max_units, p.kv_rows, p.B);
-  if (p.parts > 1) {
-    const int grid = static_cast<int>(max_units) * p.parts;
-    return f16 ? launch_typed<true, true>(mQ, mKV, p, grid, st) : launch_typed<false, true>(mQ, mKV, p, grid, st);
-  }
+  if (p.parts > 1) return launch_split<true>(mQ, mKV, p, f16, static_cast<int>(max_units) * p.parts, st);
   // persistent: one CTA per SM (at most one per unit)
-  const int grid = static_cast<int>(max_units < num_sms ? max_units : num_sms);
-  return f16 ? launch_typed<true, false>(mQ, mKV, p, grid, st) : launch_typed<false, false>(mQ, mKV, p, grid, st);
+  return launch_split<false>(mQ, mKV, p, f16, static_cast<int>(max_units < num_sms ? max_units : num_sms), st);
 }
 
 cudaError_t launch_attn_schedule(const ScheduleArgs& a, int* err, cudaStream_t st) {

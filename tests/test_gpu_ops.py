@@ -341,6 +341,29 @@ def test_attention_split_keys_with_infinite_scores(dt):
     check_close(host(out), host(ref.float()), "bf16", "attention, infinite scores")
 
 
+@pytest.mark.parametrize("B", [1, 4, 30, 44, 45, 64, 65, 200])
+def test_attention_schedule_made_by_either_kernel(B):
+    """Calls of up to 64 segments with a unit per SM at most make the schedule in the
+    attention kernel: equal lengths and masked tails against the oracle, and empty
+    segments between them change nothing."""
+    rng = _rng(B)
+    lens = rng.choice([1, 40, 130, 300], B)
+    lens[0] = 257
+    kv = np.where(rng.random(B) < 0.3, np.maximum(lens - 7, 1), lens)
+    _attention_case("f16", 2, 128, [int(v) for v in lens], [int(v) for v in kv], 1.0, B)
+    T, ws = int(lens.sum()), torch.empty(1 << 20, dtype=torch.uint8, device=cuda())
+    qkv = torch.randn((T, 3 * 256), generator=torch.Generator(device="cuda").manual_seed(B), device="cuda").half()
+    keep = np.sort(rng.choice(B + 20, B, replace=False))              # B + 20 segments, 20 of them empty
+    more, more_kv = np.zeros(B + 20, dtype=np.int64), np.zeros(B + 20, dtype=np.int64)
+    more[keep], more_kv[keep] = lens, kv
+    out = []
+    for n, k in ((lens, kv), (more, more_kv)):
+        o = torch.empty((T, 256), dtype=torch.float16, device="cuda")
+        S.seer_attention(qkv, o, "f16", i32(np.concatenate([[0], np.cumsum(n)])), i32(k), len(n), T, 2, 128, ws, 1 << 20)
+        out.append(o)
+    assert torch.equal(*out)
+
+
 def test_attention_many_heads():
     _attention_case("f16", 4, 128, [200, 90], [200, 90], 1.0, 12)
 
