@@ -117,18 +117,22 @@ __device__ __forceinline__ uint32_t ex2_h2(uint32_t x) {
   asm("ex2.approx.f16x2 %0, %1;" : "=r"(y) : "r"(x));
   return y;
 }
-// acc + (f16 half of v), in fp32 (mixed-precision add).
-__device__ __forceinline__ float add_f16_lo(uint32_t v, float acc) {
+// acc + the low / high 16-bit half of v (f16 or bf16), in fp32: one mixed-precision
+// addition each.
+template <bool F16>
+__device__ __forceinline__ float add_lo16(uint32_t v, float acc) {
   float d;
-  asm("{\n\t.reg .b16 l, h;\n\tmov.b32 {l, h}, %1;\n\tadd.rn.f32.f16 %0, l, %2;\n\t}" : "=f"(d) : "r"(v), "f"(acc));
+  if (F16) asm("{\n\t.reg .b16 l, h;\n\tmov.b32 {l, h}, %1;\n\tadd.rn.f32.f16 %0, l, %2;\n\t}" : "=f"(d) : "r"(v), "f"(acc));
+  else asm("{\n\t.reg .b16 l, h;\n\tmov.b32 {l, h}, %1;\n\tadd.rn.f32.bf16 %0, l, %2;\n\t}" : "=f"(d) : "r"(v), "f"(acc));
   return d;
 }
-__device__ __forceinline__ float add_f16_hi(uint32_t v, float acc) {
+template <bool F16>
+__device__ __forceinline__ float add_hi16(uint32_t v, float acc) {
   float d;
-  asm("{\n\t.reg .b16 l, h;\n\tmov.b32 {l, h}, %1;\n\tadd.rn.f32.f16 %0, h, %2;\n\t}" : "=f"(d) : "r"(v), "f"(acc));
+  if (F16) asm("{\n\t.reg .b16 l, h;\n\tmov.b32 {l, h}, %1;\n\tadd.rn.f32.f16 %0, h, %2;\n\t}" : "=f"(d) : "r"(v), "f"(acc));
+  else asm("{\n\t.reg .b16 l, h;\n\tmov.b32 {l, h}, %1;\n\tadd.rn.f32.bf16 %0, h, %2;\n\t}" : "=f"(d) : "r"(v), "f"(acc));
   return d;
 }
-
 
 // Two fp32 fused multiply-adds in one instruction (packed f32x2, sm_100+).
 __device__ __forceinline__ void ffma2(float a0, float a1, float b0, float b1, float c0, float c1, float& d0, float& d1) {
@@ -142,34 +146,28 @@ __device__ __forceinline__ void ffma2(float a0, float a1, float b0, float b1, fl
 }
 
 // Packed probabilities of keys 32c .. 32c+31 of one row: p = 2^(s * scale - m),
-// accumulated into the row sum.  f16: the exponents x of a pair come from one
-// packed f32x2 FMA, are rounded to f16, and two probabilities come from one
-// MUFU operation (ex2.approx.f16x2); P is stored in f16 anyway.  bf16: one
-// fp32 ex2 per probability.  Either way the row sum adds the stored (rounded)
-// probabilities.  The softmax of a tile sits on its tile's critical chain, so
-// its instruction count matters: the packed FMA is 2.5% faster on GB300, while
-// moving a quarter of the exponentials to a polynomial on the FMA pipes was 9%
-// slower (more instructions, no MUFU relief).
+// accumulated into the row sum.  The exponents of a pair come from one packed f32x2
+// FMA.  f16: they are rounded to f16, and two probabilities come from one MUFU
+// operation (ex2.approx.f16x2); P is stored in f16 anyway.  bf16: one fp32 ex2 per
+// probability.  Either way the row sum adds the stored (rounded) probabilities by
+// mixed-precision additions, so numerator and normaliser carry the same rounding.
+// The softmax of a tile sits on its tile's critical chain, so its instruction count is
+// what matters (8 x 3100 rows, 32 heads): bf16 0.950 ms with scalar FMAs and unpacked
+// sums, 0.857 with packed FMAs, 0.807 so; with an eighth / a quarter of its exponentials
+// as a polynomial on the FMA pipes 0.900 / 1.003; f16 0.836, with fp32 ex2 0.814 (not
+// taken: the near-zero counts of a layer behind it would move by more than the ties
+// that a change of order may move).
 template <bool F16>
 __device__ __forceinline__ void row_probs(const float* s, float scale_log2, float neg, float (&rs)[4],
                                           uint32_t (&pk)[16]) {
 #pragma unroll
   for (int i = 0; i < 16; ++i) {
-    if (F16) {
-      float x0, x1;
-      ffma2(s[2 * i], s[2 * i + 1], scale_log2, scale_log2, neg, neg, x0, x1);
-      const uint32_t ph = ex2_h2(pack_f16x2(x0, x1));
-      rs[(2 * i) & 3] = add_f16_lo(ph, rs[(2 * i) & 3]);
-      rs[(2 * i + 1) & 3] = add_f16_hi(ph, rs[(2 * i + 1) & 3]);
-      pk[i] = ph;
-    } else {
-      const float x0 = fmaf(s[2 * i], scale_log2, neg), x1 = fmaf(s[2 * i + 1], scale_log2, neg);
-      // the row sum adds the rounded probabilities the PV product reads, so
-      // numerator and normaliser carry the same rounding
-      const uint32_t ph = pack_bf16x2(ex2(x0), ex2(x1));
-      rs[i & 3] += bf16_lo(ph) + bf16_hi(ph);
-      pk[i] = ph;
-    }
+    float x0, x1;
+    ffma2(s[2 * i], s[2 * i + 1], scale_log2, scale_log2, neg, neg, x0, x1);
+    const uint32_t ph = F16 ? ex2_h2(pack_f16x2(x0, x1)) : pack_bf16x2(ex2(x0), ex2(x1));
+    rs[(2 * i) & 3] = add_lo16<F16>(ph, rs[(2 * i) & 3]);
+    rs[(2 * i + 1) & 3] = add_hi16<F16>(ph, rs[(2 * i + 1) & 3]);
+    pk[i] = ph;
   }
 }
 
