@@ -287,8 +287,12 @@ seer_status seer_convert(const void* src, seer_dtype src_dt, void* dst, seer_dty
  * segment's first kv_len[b] keys (Eqs. 6-7, no causal mask).  qkv [T, 3*H*dh]
  * holds q | k | v.  ws as for seer_layer_forward (only the scheduling part:
  * the work units, their count and the counter from which the attention
- * kernel's persistent CTAs take units; all rewritten by every call, so calls
- * that share a workspace must not overlap on the GPU). */
+ * kernel's persistent CTAs take units; rewritten by every call that does not
+ * make its schedule inside the kernel, so calls that share a workspace must
+ * not overlap on the GPU).  Where a call has few units (segment, head, 256
+ * query rows) and many keys, each unit's keys are shared by a cluster of CTAs
+ * and the shares merged in fp32: such a call's results differ from those of a
+ * call that keeps them together by fp32 rounding before the 16-bit store. */
 seer_status seer_attention(const void* qkv, void* o, seer_dtype dt, const int32_t* cu_seqlens,
                            const int32_t* kv_len, int B, int T_capacity, int n_heads, int head_dim,
                            void* ws, size_t ws_bytes, void* stream);
@@ -361,9 +365,9 @@ seer_status seer_selftest_wait_timeout(int limit_us, void* stream);
  * each kernel of the library is launched as a programmatic dependent of the
  * previous kernel in its stream: the GPU may place its blocks while that
  * kernel finishes, which hides most of the launch gap between consecutive
- * kernels.  Every kernel waits at entry until the kernels before it have
- * completed and their writes are visible, so results are the same with the
- * setting on or off.  Process-wide; returns the previous setting (1 or 0). */
+ * kernels.  Every kernel waits, before it touches global memory, until the
+ * kernels before it have completed and their writes are visible, so results
+ * are the same with the setting on or off.  Process-wide; returns the previous setting (1 or 0). */
 int seer_set_launch_overlap(int on);
 
 /* Per-phase timing with CUDA events recorded on the call's stream.
