@@ -50,8 +50,16 @@ __device__ __forceinline__ void ffma2(float2& acc, float a0, float a1, float b0,
 // chain; the detector's (Count) is one chain over ascending k.
 // For Swiglu / Count the block holds BN / 2 gate columns and the matching up
 // columns, and a thread's first TN / 2 columns are gates.
-// Bound by instruction issue beside the FMA pipes (44 TFLOP/s of 80 at the largest
-// shape; scalar multiply-adds 41) and, for few rows, by the latency of the k-steps.
+// Lanes: neighbours (lane ^ 1) differ in their row, lanes two apart in their column.
+// A 16-byte shared-memory read takes four passes, or two where every lane shares its
+// address with lane ^ 1 or with lane ^ 2; so both operands' reads take two.  With 16
+// consecutive lanes along a row the columns' reads took four: 208 x 768 x 256 8.7 us
+// (now 7.1 at the 16 x 32 tile), 208 x 512 x 1536 29.3 (24.8), 2624 x 512 x 1536 at the
+// 32 x 64 tile 142.6 (136.2), 64 x 64 tiles -1%.
+// Bound by the packed multiply-adds' register reads (44 TFLOP/s of 80 at the largest
+// shape; a loop of them over an 8 x 4 tile in registers alone 46, scalar ones 66, but
+// twice the instructions: scalar 42 here) and, for few rows, by the latency of the
+// k-steps.
 template <int MODE, int BM, int BN, int TM, int TN, int TK, int STAGES, int MIN_BLOCKS, int VEC>
 __global__ void __launch_bounds__((BM / TM) * (BN / TN), MIN_BLOCKS)
     simt_gemm_kernel(const float* __restrict__ A, const float* __restrict__ B0, const float* __restrict__ B1,
@@ -96,7 +104,8 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN), MIN_BLOCKS)
     rows_here = min(BM, M - row_base);
   }
   const int col_base = nt * COLS;
-  const int tx = threadIdx.x % TX, ty = threadIdx.x / TX;
+  const int lane = threadIdx.x & 31;
+  const int tx = (lane >> 1) % TX, ty = (threadIdx.x >> 5) * (32 / TX) + (lane & 1) + 2 * ((lane >> 1) / TX);
 
   // stage k0 .. k0 + TK - 1 of both operands (zeros past the rows, columns and K)
   auto load = [&](int stage, int k0) {
@@ -188,9 +197,9 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN), MIN_BLOCKS)
       }
     }
     if (TWO && p.counts != nullptr) {
-      // a row's TX threads are consecutive lanes: one atomic per row and block
+      // a row's TX threads are every other lane: one atomic per row and block
 #pragma unroll
-      for (int off = TX / 2; off > 0; off >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, off);
+      for (int off = TX; off > 1; off >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, off);
       if (in && tx == 0 && cnt > 0) {
         int idx = -1;
         if (MODE == kGemmCount) {
@@ -214,13 +223,14 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN), MIN_BLOCKS)
 // keys in tiles of 64 with an online softmax (fp32, expf).
 // Scores: a thread holds BQ / TY rows (ty + TY i) x 4 keys (tx + 16 j), Q and K
 // row-major in shared memory and read four dims at a time; a row's 16 threads are
-// consecutive lanes, so its max and sum are shuffles; the probabilities go
+// every other lane of a warp, so its max and sum are shuffles; the probabilities go
 // through shared memory and a thread accumulates its rows x the output columns
 // 4 tx .. 4 tx + 3 (and + 64).  The next K tile is copied by cp.async while the
 // current tile's softmax and PV run, the next V tile while the next scores do.
-// Bound by instruction issue beside the FMA pipes and shared-memory reads.  A warp
-// per (row, head) that reads every key itself took 1209 us for the 8-segment
-// batch of 58 .. 794 rows, 8 heads of 64; this kernel 146.
+// Bound by shared-memory reads (two passes each, see the GEMM's lanes) beside as many
+// FMA cycles.  A warp per (row, head) that reads every key itself took 1209 us for the
+// 8-segment batch of 58 .. 794 rows, 8 heads of 64; this kernel 140 (146 with 16
+// consecutive lanes along a row, four passes for K and V).
 constexpr int AKV = 64;                      // keys per tile
 constexpr int APS = AKV + 16;                // floats per row of probabilities (two rows meet no bank twice)
 
@@ -261,7 +271,7 @@ __global__ void __launch_bounds__(16 * TY) simt_attn_kernel(const float* __restr
   float* Ks = Qs + BQ * ld;                           // [AKV][ld]
   float* Vs = Ks + AKV * ld;                          // [AKV][ld]
   float* Ps = Vs + AKV * ld;                          // [BQ][APS]
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  const int tx = (threadIdx.x & 31) >> 1, ty = (threadIdx.x >> 5) * 2 + (threadIdx.x & 1);   // lanes as in the GEMM
   const int per_row = dh / VEC;
 
   for (int i = threadIdx.x; i < BQ * per_row; i += 16 * TY) {
@@ -327,7 +337,7 @@ __global__ void __launch_bounds__(16 * TY) simt_attn_kernel(const float* __restr
         mx = fmaxf(mx, sc[i][j]);
       }
 #pragma unroll
-      for (int off = 8; off > 0; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
+      for (int off = 16; off > 1; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
       const float alpha = expf(m[i] - mx);
       m[i] = mx;
       float sum = 0.f;
@@ -383,7 +393,7 @@ __global__ void __launch_bounds__(16 * TY) simt_attn_kernel(const float* __restr
   for (int i = 0; i < TM; ++i) {
     float sum = l[i];
 #pragma unroll
-    for (int off = 8; off > 0; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
+    for (int off = 16; off > 1; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
     const int r = ty + TY * i;
     if (r >= rows) continue;
     float* out = reinterpret_cast<float*>(p.out) + static_cast<size_t>(seq0 + q0 + r) * p.ldo + h * dh;
@@ -426,10 +436,10 @@ cudaError_t launch_tile(const float* A, const float* B0, const float* B1, const 
 
 // The largest tile that leaves every SM several blocks (us at 64 x 64 / 32 x 64 /
 // 32 x 32 / 16 x 32 tiles; the transposing 64 x 64 kernel before): 2624 x 1536 x 512
-// 108 / 112 / 134 / 189 (147); 2624 x 512 x 1536 150 / 142 / 143 / 199 (191); 600 x
-// 1536 x 512 49 / 29 / 35 / 50; 600 x 512 x 1536 75 / 50 / 39 / 57; 208 x 768 x 256
-// 13 / 11 / 9.1 / 8.7 (16); 208 x 256 x 768 41 / 27 / 17 / 14 (44); 8192 x 4096 x 1024
-// 44 TFLOP/s at 64 x 64.
+// 108 / 111 / 125 / 168 (147); 2624 x 512 x 1536 148 / 136 / 134 / 171 (191); 800 x
+// 1536 x 512 49 / 37 / 41 / 54; 800 x 512 x 1536 73 / 65 / 62 / 60; 208 x 768 x 256
+// 13 / 8.9 / 8.7 / 7.1 (16); 208 x 256 x 768 40 / 25 / 16 / 11.4 (44); 8192 x 4096 x
+// 1024 44 TFLOP/s at 64 x 64.
 template <int MODE>
 cudaError_t launch_mode(const float* A, const float* B0, const float* B1, const GemmParams& p, int num_sms,
                         cudaStream_t st) {
