@@ -434,12 +434,17 @@ cudaError_t launch_tile(const float* A, const float* B0, const float* B1, const 
              : launch_vec<MODE, BM, BN, TM, TN, TK, STAGES, MIN_BLOCKS, 1>(grid, A, B0, B1, p, st);
 }
 
-// The largest tile that leaves every SM several blocks (us at 64 x 64 / 32 x 64 /
-// 32 x 32 / 16 x 32 tiles; the transposing 64 x 64 kernel before): 2624 x 1536 x 512
-// 108 / 111 / 125 / 168 (147); 2624 x 512 x 1536 148 / 136 / 134 / 171 (191); 800 x
-// 1536 x 512 49 / 37 / 41 / 54; 800 x 512 x 1536 73 / 65 / 62 / 60; 208 x 768 x 256
-// 13 / 8.9 / 8.7 / 7.1 (16); 208 x 256 x 768 40 / 25 / 16 / 11.4 (44); 8192 x 4096 x
-// 1024 44 TFLOP/s at 64 x 64.
+// The tile that is expected to finish first.  A k-step costs a block's share of its
+// SM, `share`, for each of the n = tiles / SMs blocks of an SM (and half of one more:
+// the last blocks do not spread evenly), but at least one, plus `latency`, what the
+// blocks in flight do not hide.  Both in us per 32 k, fitted to 100 shapes of 64 ..
+// 8192 rows (rms 6-7%; the choice is 1% from the best of the four tiles on average).
+// The rule before (the largest tile that leaves every SM several blocks) was 5% from
+// it, at worst a third: 208 x 3072 x 1024 69 -> 52 us, 1300 x 512 x 1536 109 -> 82, 2624 x
+// 256 x 768 55 -> 42, 208 x 768 x 256 8.7 -> 7.1; none more than 1% slower.  At 64 x 64 / 32 x 64 / 32 x 32 / 16 x 32 tiles, us: 2624 x 1536 x 512 108 /
+// 111 / 125 / 168 (a transposing 64 x 64 kernel 147); 2624 x 512 x 1536 148 / 136 / 134 /
+// 171 (191); 208 x 256 x 768 40 / 25 / 16 / 11.4 (44); 8192 x 4096 x 1024 44 TFLOP/s at
+// 64 x 64.
 template <int MODE>
 cudaError_t launch_mode(const float* A, const float* B0, const float* B1, const GemmParams& p, int num_sms,
                         cudaStream_t st) {
@@ -450,11 +455,15 @@ cudaError_t launch_mode(const float* A, const float* B0, const float* B1, const 
     return MODE == kGemmCount ? static_cast<long>(p.B) * ((p.Nw + bm - 1) / bm) : (p.M_cap + bm - 1l) / bm;
   };
   const auto tiles = [&](int bm, int bn) { return m_tiles(bm) * ((p.N + (TWO ? bn / 2 : bn) - 1l) / (TWO ? bn / 2 : bn)); };
-  if (tiles(64, 64) >= 4l * num_sms || m_tiles(32) > 65535)
-    return launch_tile<MODE, 64, 64, 8, 4, 32, 3, 3>(A, B0, B1, p, vec, st);
-  if (tiles(32, 64) >= 2l * num_sms) return launch_tile<MODE, 32, 64, 4, 4, 32, 4, 4>(A, B0, B1, p, vec, st);
-  if (tiles(32, 32) >= num_sms || m_tiles(16) > 65535)
-    return launch_tile<MODE, 32, 32, 4, 2, 32, 5, 1>(A, B0, B1, p, vec, st);
+  const auto cost = [&](int bm, int bn, float latency, float share) {
+    if (bm < 64 && m_tiles(bm) > 65535) return INFINITY;   // more row tiles than a grid takes
+    return latency + share * fmaxf(1.0f, static_cast<float>(tiles(bm, bn)) / static_cast<float>(num_sms) + 0.5f);
+  };
+  const float t0 = cost(64, 64, 0.62f, 0.89f), t1 = cost(32, 64, 0.42f, 0.49f), t2 = cost(32, 32, 0.22f, 0.29f);
+  const float t3 = cost(16, 32, 0.08f, 0.205f), best = fminf(fminf(t0, t1), fminf(t2, t3));
+  if (t0 == best) return launch_tile<MODE, 64, 64, 8, 4, 32, 3, 3>(A, B0, B1, p, vec, st);
+  if (t1 == best) return launch_tile<MODE, 32, 64, 4, 4, 32, 4, 4>(A, B0, B1, p, vec, st);
+  if (t2 == best) return launch_tile<MODE, 32, 32, 4, 2, 32, 5, 1>(A, B0, B1, p, vec, st);
   return launch_tile<MODE, 16, 32, 2, 2, 32, 6, 1>(A, B0, B1, p, vec, st);
 }
 

@@ -142,7 +142,7 @@ def test_linear_f32_tile_choices(M, N, K, offset):
     assert torch.isnan(c[M]).all()
 
 
-@pytest.mark.parametrize("M,F,K", [(9, 36, 20), (70, 130, 33), (200, 1540, 12), (900, 2052, 20)])
+@pytest.mark.parametrize("M,F,K", [(9, 36, 20), (70, 130, 33), (200, 1540, 12), (900, 2052, 20), (1300, 2052, 20)])
 def test_swiglu_f32_tile_choices(M, F, K):
     """fp32 gate/up tiles of every size with the count hook; activations against
     fp64, counts against the kernel's own activations."""
