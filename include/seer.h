@@ -292,7 +292,9 @@ seer_status seer_convert(const void* src, seer_dtype src_dt, void* dst, seer_dty
  * not overlap on the GPU).  Where a call has few units (segment, head, 256
  * query rows) and many keys, each unit's keys are shared by a cluster of CTAs
  * and the shares merged in fp32: such a call's results differ from those of a
- * call that keeps them together by fp32 rounding before the 16-bit store. */
+ * call that keeps them together by fp32 rounding before the 16-bit store.  A
+ * layer with the count hook always keeps them together, so its counts do not
+ * depend on the batch it runs in. */
 seer_status seer_attention(const void* qkv, void* o, seer_dtype dt, const int32_t* cu_seqlens,
                            const int32_t* kv_len, int B, int T_capacity, int n_heads, int head_dim,
                            void* ws, size_t ws_bytes, void* stream);

@@ -422,7 +422,7 @@ ScheduleArgs schedule_args(const int32_t* cu, const int32_t* cu_kv, const int32_
 // scheduled: the schedule of this call is already in the workspace.
 seer_status do_attention(const void* qkv, void* o, seer_dtype dt, const int32_t* cu, const int32_t* kv_len, int B,
                          int T_cap, int H, int dh, void* sched, size_t sched_bytes, cudaStream_t st,
-                         const KvSource& kvs = KvSource(), bool scheduled = false) {
+                         const KvSource& kvs = KvSource(), bool scheduled = false, bool keys_together = false) {
   if (!qkv || !o || !cu) return fail(SEER_ERR_INVALID_ARG, "attention: null pointer");
   if (kvs.kv && (!kvs.cu_kv || kvs.T_kv_cap < 0 || kvs.ld < 2 * H * dh))
     return fail(SEER_ERR_INVALID_ARG, "attention: a separate K/V source needs cu_kv, a capacity and rows of >= 2*H*dh");
@@ -445,7 +445,7 @@ seer_status do_attention(const void* qkv, void* o, seer_dtype dt, const int32_t*
   p.ld_kv = kvs.kv ? kvs.ld : 3 * H * dh;
   p.xk0 = kvs.kv ? kvs.xk0 : H * dh;
   p.xv0 = kvs.kv ? kvs.xv0 : 2 * H * dh;
-  p.kv_rows = kvs.kv ? kvs.T_kv_cap : T_cap;
+  p.kv_rows = keys_together ? 0 : (kvs.kv ? kvs.T_kv_cap : T_cap);
   if (is16(dt)) {
     if (dh != 128) return fail(SEER_ERR_UNSUPPORTED, "16-bit attention needs head_dim == 128");
     if (kvs.kv && (!aligned16(kvs.kv) || (static_cast<long>(kvs.ld) * 2) % 16 != 0 || kvs.xk0 % 64 != 0 || kvs.xv0 % 64 != 0))
@@ -783,8 +783,10 @@ seer_status seer_layer_forward(const seer_layer_weights* w, const seer_dims* dim
   if (!early && rope.tab) SEER_CUDA(launch_rope_table(pre.rope, di->err, di->num_sms, st), "rope table");
   SEER_TRY(do_rmsnorm(x, dt, w->g_attn, xn, it, T_capacity, M_dev, d, eps, st, PH_NORM1, RowMap{}, early ? &pre : nullptr));
   SEER_TRY(do_linear(xn, w->w_qkv, it, nullptr, it, qkv, it, T_capacity, M_dev, 3 * d, d, st, PH_QKV, rope));
+  // A layer that counts keeps each unit's keys on one CTA: shares merged in another
+  // order move activations by a rounding, and a count with one on the threshold.
   SEER_TRY(do_attention(qkv, xn, it, cu_seqlens, kv_len, B, T_capacity, H, dh, sched, L.total - L.off_sched, st, KvSource(),
-                        early));
+                        early, count_resp_start != nullptr));
   SEER_TRY(do_linear(xn, w->w_o, it, x, dt, h, it, T_capacity, M_dev, d, d, st, PH_OPROJ));
   SEER_TRY(do_rmsnorm(h, it, w->g_mlp, xn, it, T_capacity, M_dev, d, eps, st, PH_NORM2));
   SEER_TRY(do_swiglu(xn, w->w_gate, w->w_up, it, act, it, T_capacity, M_dev, F, d, cu_seqlens, B, count_resp_start, N,

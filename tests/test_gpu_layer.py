@@ -248,6 +248,32 @@ def test_rotary_layer_at_long_positions():
         check_close(yh[cu_full[b] + np.asarray(rows)], ref, "bf16", f"rotary layer segment {b}")
 
 
+def test_count_hook_layer_does_not_depend_on_its_batch():
+    # few query tiles over many keys: without the hook the keys of a unit are shared by several CTAs; with
+    # it one long segment gives the bits (outputs and counts) it has among eight of the same, which never share
+    wl = synth.tiny_workload(dtype="bf16", seed=370, d=256, n_heads=2, head_dim=128, d_ff=896, batch=1, window=64)
+    w = synth.layer_weights(wl, 0)
+    d, n, N = wl.d, 2470, 51
+    dims = S.make_dims(d, wl.n_heads, wl.head_dim, wl.d_ff)
+    _, WL = layer_weight_tensors(wl, w)
+    x = synth.round_storage(np.random.default_rng(37).standard_normal((n, d)), "bf16")
+
+    def run(B):
+        T = B * n
+        xd = to_dev(np.tile(x, (B, 1)), "bf16")
+        y = torch.empty_like(xd)
+        counts = torch.empty(B * N, dtype=torch.int32, device=cuda())
+        size = S.seer_layer_workspace_size(dims, "bf16", T, B)
+        ws = torch.empty(size, dtype=torch.uint8, device=cuda())
+        S.seer_layer_forward(weights_struct(WL), dims, "bf16", xd, y, i32([n * b for b in range(B + 1)]),
+                             i32([n - 21] * B), B, T, i32([n * b + n - N for b in range(B)]), N, 3e-4, counts, ws, size)
+        torch.cuda.synchronize()
+        return y[:n], counts[:N]
+
+    for one, eight in zip(run(1), run(8)):
+        assert torch.equal(one, eight)
+
+
 def test_run_from_host_pipelined_matches_device_step():
     # the end-to-end call (pinned host input, double-buffered copies overlapping compute)
     # returns exactly what a device-resident step computes
