@@ -497,15 +497,19 @@ cudaError_t launch_simt_attn(const float* qkv, const AttnParams& p, int num_sms,
   const auto aligned = [](const void* q) { return (reinterpret_cast<uintptr_t>(q) & 15u) == 0; };
   // rows of the separate K/V source start 16-byte aligned when its width and columns do
   const bool vec = aligned(qkv) && (p.kv == nullptr || (aligned(p.kv) && p.ld_kv % 4 == 0)) && p.xk0 % 4 == 0 && p.xv0 % 4 == 0;
-  // 32-row tiles once their blocks fill the SMs twice (unless most segments are far
-  // shorter), then 16-row tiles, with twice the threads where even those leave SMs
-  // idle.  Measured at 32 rows / 16 rows / 16 rows with 256 threads, us: segments of
-  // 114 .. 794 rows, 8 heads of 64 146 / 166 / 214; one of 700 rows 92 / 83 / 97; one of
-  // 121 rows, 4 heads 16 / 14 / 10; 64-row tiles 154 / 123 / 20.
+  // 32-row tiles once their blocks fill the SMs three times (unless most segments are
+  // far shorter); else 16-row tiles, with twice the threads unless heads of at most 64
+  // let four blocks share an SM and the blocks fill the SMs four times.  Measured at 32
+  // rows / 16 rows / 16 rows with 256 threads, us: segments of 58 .. 794 rows, 8 heads of
+  // 64 (4.7 times) 141 / 159 / 163; four of 500 (3.5) 96 / 120 / 123; four of 800, 4 heads
+  // of 128 (2.7) 295 / 345 / 267; one of 1500, 8 heads of 64 (2.5; 16 rows 5.0) 274 / 230 /
+  // 260; one of 700 (1.2; 2.4) 100 / 78 / 75; sixteen of 60, 8 heads of 32 (2.4; 4.0) 14.5 /
+  // 13.7 / 11.5; one of 121, 4 heads 15.8 / 12.7 / 8.2; 64-row tiles 194 at the first.
   const auto blocks = [&](long bq) { return (p.T_cap / bq + p.B) * p.n_heads; };
-  if (blocks(32) >= 2l * num_sms && p.T_cap / p.B >= 16)
+  if (blocks(32) >= 3l * num_sms && p.T_cap / p.B >= 16)
     return vec ? launch_attn<32, 8, 4>(qkv, p, st) : launch_attn<32, 8, 1>(qkv, p, st);
-  if (blocks(16) >= num_sms) return vec ? launch_attn<16, 8, 4>(qkv, p, st) : launch_attn<16, 8, 1>(qkv, p, st);
+  if (p.head_dim <= 64 && blocks(16) > 4l * num_sms)
+    return vec ? launch_attn<16, 8, 4>(qkv, p, st) : launch_attn<16, 8, 1>(qkv, p, st);
   return vec ? launch_attn<16, 16, 4>(qkv, p, st) : launch_attn<16, 16, 1>(qkv, p, st);
 }
 

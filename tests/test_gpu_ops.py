@@ -162,7 +162,8 @@ def test_swiglu_f32_tile_choices(M, F, K):
 @pytest.mark.parametrize("H,dh,lens,kv", [
     (2, 64, [1, 15, 16, 17], [1, 15, 9, 17]),                       # 16-row tiles, 256 threads
     (3, 4, [5, 64, 65], [5, 64, 1]), (2, 28, [70, 3, 129], [70, 2, 128]), (1, 100, [200], [130]), (2, 128, [131], [131]),
-    (16, 64, [150, 31], [97, 31]), (12, 128, [200], [129]),         # 16-row tiles
+    (16, 64, [150, 31], [97, 31]), (12, 128, [200], [129]),
+    (24, 20, [400], [390]),                                         # 16-row tiles, 128 threads
     (32, 32, [400, 63, 257], [399, 63, 64]),                        # 32-row tiles
     (40, 128, [300, 129, 64], [300, 65, 64]), (40, 12, [500, 33], [461, 33])])
 @pytest.mark.parametrize("offset", [0, 1])
