@@ -78,7 +78,8 @@ struct AttnParams {
   const int4* work;       // schedule: (b, h, first q-tile, q-tiles), or null: made in the kernel
   const int* work_count;  // units in `work`
   int* work_next;         // next unit to hand out (zeroed by the schedule kernel)
-  int kv_rows;            // rows of the K/V source (capacity); 0: a unit's keys are not shared among CTAs
+  int kv_rows;            // rows of the K/V source (capacity)
+  bool keys_together;     // a unit's keys are not shared among CTAs
   int parts;              // CTAs sharing a unit's keys (set by launch_tc_attn)
   int* err;
 };

@@ -445,7 +445,8 @@ seer_status do_attention(const void* qkv, void* o, seer_dtype dt, const int32_t*
   p.ld_kv = kvs.kv ? kvs.ld : 3 * H * dh;
   p.xk0 = kvs.kv ? kvs.xk0 : H * dh;
   p.xv0 = kvs.kv ? kvs.xv0 : 2 * H * dh;
-  p.kv_rows = keys_together ? 0 : (kvs.kv ? kvs.T_kv_cap : T_cap);
+  p.kv_rows = kvs.kv ? kvs.T_kv_cap : T_cap;
+  p.keys_together = keys_together;
   if (is16(dt)) {
     if (dh != 128) return fail(SEER_ERR_UNSUPPORTED, "16-bit attention needs head_dim == 128");
     if (kvs.kv && (!aligned16(kvs.kv) || (static_cast<long>(kvs.ld) * 2) % 16 != 0 || kvs.xk0 % 64 != 0 || kvs.xv0 % 64 != 0))

@@ -246,6 +246,11 @@ __global__ void __launch_bounds__(16 * TY) simt_attn_kernel(const float* __restr
     if (blockIdx.x == 0 && threadIdx.x == 0) record_error(p.err, kErrRows);
     return;
   }
+  // segments that no block's slot leads to are checked by the last block, whose own
+  // slot is past every segment's tiles unless all of them end in a partial tile
+  if (blockIdx.x == gridDim.x - 1)
+    for (int b = threadIdx.x; b < p.B; b += blockDim.x)
+      if (p.cu[b] < 0 || p.cu[b + 1] < p.cu[b] || p.cu[b + 1] > p.T_cap) record_error(p.err, kErrLayout);
   // slot -> (segment, query tile): the slots of segment b start at cu[b] / BQ + b,
   // at least as far apart as its tiles
   const int slot = blockIdx.x / H, h = blockIdx.x % H;
@@ -260,7 +265,9 @@ __global__ void __launch_bounds__(16 * TY) simt_attn_kernel(const float* __restr
   const int kv0 = p.cu_kv ? p.cu_kv[lo] : seq0;
   const int Lkv = p.cu_kv ? p.cu_kv[lo + 1] - kv0 : L;
   const int kvL = p.kv_len ? p.kv_len[lo] : Lkv;
-  if (kvL <= 0 || kvL > Lkv) {
+  // rows outside either buffer are neither read nor written: the offsets come from the
+  // device, and a segment's tiles reach all of cu[lo] .. cu[lo + 1] - 1
+  if (seq0 < 0 || L > p.T_cap - seq0 || kvL <= 0 || kvL > Lkv || kv0 < 0 || kvL > p.kv_rows - kv0) {
     if (threadIdx.x == 0) record_error(p.err, kErrLayout);
     return;
   }

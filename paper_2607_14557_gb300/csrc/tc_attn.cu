@@ -881,7 +881,7 @@ cudaError_t launch_split(const CUtensorMap& mQ, const CUtensorMap& mKV, const At
 cudaError_t launch_tc_attn(const CUtensorMap& mQ, const CUtensorMap& mKV, AttnParams p, bool f16, int num_sms,
                            cudaStream_t st) {
   const long max_units = static_cast<long>(p.n_heads) * (p.T_cap / (NT * BQ) + p.B);
-  p.parts = attn_parts(max_units, p.kv_rows, p.B);
+  p.parts = p.keys_together ? 1 : attn_parts(max_units, p.kv_rows, p.B);
   if (p.parts > 1) return launch_split<true>(mQ, mKV, p, f16, static_cast<int>(max_units) * p.parts, st);
   // persistent: one CTA per SM (at most one per unit)
   return launch_split<false>(mQ, mKV, p, f16, static_cast<int>(max_units < num_sms ? max_units : num_sms), st);

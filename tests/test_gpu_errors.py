@@ -116,6 +116,31 @@ def test_attention_segment_past_capacity_is_recorded_and_skipped():
     assert (host(o)[120:] == SENTINEL).all()                            # the bad one is skipped
 
 
+@pytest.mark.parametrize("cu,valid", [([0, 500, 300], []), ([-40, 100, 300], [1]), ([0, 130, 500, 300], [0]),
+                                      ([0, 120, 90, 300], None)])
+@pytest.mark.parametrize("H,dh", [(1, 32), (32, 8), (48, 8)])      # 16-row query tiles, 32-row ones
+def test_f32_attention_segments_outside_the_capacity_are_recorded_and_skipped(H, dh, cu, valid):
+    # segments that run past T_cap, start before row 0 or end before they start, with the
+    # last offset inside the capacity: nothing outside the rows is written, and the valid
+    # segments beside a bad one still run (overlapping segments: which of them does is open)
+    D, T_cap, pad = H * dh, 300, 256
+    g = torch.Generator(device="cuda").manual_seed(H)
+    buf = torch.randn((T_cap + 2 * pad, 3 * D), generator=g, device="cuda")
+    out = torch.full((T_cap + 2 * pad, D), SENTINEL, device="cuda")
+    qkv, o = buf[pad:], out[pad:]
+    S.seer_attention(qkv, o, "f32", i32(cu), None, len(cu) - 1, T_cap, H, dh, None, 0)
+    torch.cuda.synchronize()
+    assert S.seer_check_device() == ERR_LAYOUT
+    assert (out[:pad] == SENTINEL).all() and (o[T_cap:] == SENTINEL).all()
+    if valid is not None:
+        x, got = host(qkv), host(o)[:T_cap]
+        want = np.full((T_cap, D), SENTINEL)
+        for b in valid:
+            q = x[cu[b]:cu[b + 1]]
+            want[cu[b]:cu[b + 1]] = oracle.attention(q[:, :D], q[:, D:2 * D], q[:, 2 * D:], H)
+        np.testing.assert_allclose(got, want, rtol=1e-4, atol=1e-4)
+
+
 # ---------------------------------------------------------------- f16 range guard
 ERR_RANGE = 6
 
