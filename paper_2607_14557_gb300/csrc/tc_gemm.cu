@@ -283,9 +283,12 @@ __global__ void __launch_bounds__(THREADS, 1)
     if (CG == 2 && rank != 0 && leader) pdl_trigger();      // rank 0 triggers after its last MMAs
   } else if (warp == 1) {
     // ------------------------------------------------ MMA issuer
-    // No vote and no warp barrier per stage: the lanes stay together through the
-    // waits, and a lane that gives up (only after a 2 s limit) leaves the loop alone
-    // (narrow tiles 10% faster; 127 rows, down: 42.6 -> 38.4 us).
+    // Every lane waits for a stage and the lanes vote once per stage, between the elected
+    // one's MMAs and its commit: the commit lets the stage be filled again, and a lane
+    // still waiting for the old filling would then find the barrier's parity flipped
+    // back and wait for nothing until the time limit.  The vote there delays no MMA (us
+    // at 127 rows, QKV / O / down: 22.0 / 13.1 / 35.0; before the MMAs 22.1 / 13.6 / 35.3,
+    // the elected lane waiting alone 22.7 / 13.8 / 37.0).
     const bool leader = elect_one();
     const uint32_t idesc = (p.idesc & ~(0x3Fu << 17)) | (static_cast<uint32_t>(BN >> 3) << 17);   // N of the tile
     int s = 0;
@@ -298,9 +301,9 @@ __global__ void __launch_bounds__(THREADS, 1)
       const uint32_t d_tmem = tmem_base + static_cast<uint32_t>(acc * ACC_COLS);
       bool ok = true;
       for (int kb = 0; kb < KB; kb += DEPTH) {
-        if (!mbar_wait(&full[s], ph, abort_flag, p.err)) { ok = false; break; }
+        const bool here = mbar_wait(&full[s], ph, abort_flag, p.err);
         tc_fence_after();
-        if (leader) {
+        if (leader && here) {
           const uint32_t sa = smem_u32(smem + s * sbytes);
           const uint64_t adesc = make_sdesc_sw128(sa, 16, 1024);
           const uint64_t bdesc = make_sdesc_sw128(sa + A_TILE_BYTES, 16, 1024);
@@ -316,12 +319,14 @@ __global__ void __launch_bounds__(THREADS, 1)
               else tc_mma_f16_pair(d_tmem, adesc + off + 2 * k, bdesc + off + 2 * k, idesc, add);
             }
           }
+        }
+        if (!__all_sync(0xffffffffu, here)) { ok = false; break; }
+        if (leader) {
           if (CG == 1) tc_commit(&empty[s]);
           else tc_commit_pair(&empty[s]);
         }
         if (++s == stages) { s = 0; ph ^= 1u; }
       }
-      ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
       if (leader) {
         if (CG == 1) tc_commit(&acc_full[acc]);
@@ -633,15 +638,15 @@ cudaError_t launch_cg(const GemmPlan& plan, const CUtensorMap& mA, const CUtenso
 // columns (the SMs together read ~15 TB/s from L2) and 0.15 at 32.  So pairs are
 // the rule; one-SM tiles remain where a pair's second SM would idle (an odd,
 // small number of row tiles), and narrower tiles where they fill the last wave.
-// Examples (us, one-SM 256-column tiles -> chosen): 842 rows QKV 73.5 -> 57.7
-// (224 columns, 2.9 waves of pairs instead of 2.2 of SMs), O 30.8 -> 25.0 and
-// down 77.7 -> 60.7 (224: 76 tiles on 76 pairs); 127 rows QKV 30.7 -> 22, O 30.6 ->
-// 12.9, down 75.7 -> 32.3; 2976 rows O 74.6 -> 63.0, down 238 -> 182; 35194 rows
+// Examples (us, one-SM 256-column tiles -> chosen): 848 rows QKV 76.0 -> 59.5
+// (224 columns, 2.9 waves of pairs instead of 2.2 of SMs), O 27.7 -> 25.0 and
+// down 74.6 -> 59.6 (224: 76 tiles on 76 pairs); 127 rows QKV 31.5 -> 22.1, O 27.8 ->
+// 13.2, down 71.7 -> 35.0; 2976 rows O 71.3 -> 59.4, down 215 -> 173; 35194 rows
 // QKV 1990 -> 1927, down 2323 -> 2154.
-// Narrow tiles stage two k-blocks at a time: below ~190 columns the issuer's wait,
-// commit and loop per stage (~100 cycles) exceed what the MMAs hide (127 rows, down:
-// 38.4 us with one, 32.3 with two; 842 rows at 128 columns 75.1 and 71.6, at 224
-// columns 61.0 and 63.2).
+// Narrow tiles stage two k-blocks at a time: the issuer's wait, vote, commit and loop
+// per stage (~100 cycles) exceed what the MMAs of a narrow tile hide (127 rows, one
+// k-block / two: O 15.4 / 13.2, down 37.2 / 35.0; 300 rows, pairs of 128 columns, O 17.4 /
+// 17.8, down 39.7 / 40.3; at 224 columns 842 rows down 61.0 / 63.2).
 // A row count read on the device may leave fewer row tiles than the call is sized
 // for (a packed batch in buffers for its full windows): single-weight modes then get
 // a second width for four fifths of the tiles, and among choices within 8% of the

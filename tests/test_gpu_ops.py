@@ -96,6 +96,19 @@ def test_linear_tile_choices(M, N, K, res):
     assert torch.isnan(c[M]).all()                                  # nothing past the last row
 
 
+@pytest.mark.parametrize("M,N,K", [(127, 1024, 12288), (300, 4096, 12288)])
+def test_linear_repeats_bit_for_bit_over_a_long_k_loop(M, N, K):
+    """Each tile runs the operand ring around dozens of times; called back to back on
+    narrow tiles (two k-blocks a stage) and wide ones, every call stores the same bits."""
+    rng = _rng(M + N)
+    a, w = (to_dev(rng.integers(-2, 3, s).astype(np.float32), "f16") for s in ((M, K), (N, K)))
+    ref = (a.double() @ w.double().T).to(torch.bfloat16)              # |sums| <= 4 K < 2^24: exact in fp32
+    out = torch.full((100, M, N), float("nan"), dtype=torch.bfloat16, device=cuda())
+    for c in out:
+        S.seer_linear(a, w, "f16", None, "f16", c, "bf16", M, None, N, K)
+    assert (out == ref).all()
+
+
 @pytest.mark.parametrize("M_cap,N,K", [(640, 12288, 128), (640, 4096, 192), (900, 4096, 64), (1049, 4096, 128),
                                        (1500, 4096, 64), (1500, 12288, 64)])
 @pytest.mark.parametrize("fill", [0.0, 0.01, 0.5, 0.78, 0.8, 0.82, 1.0])
