@@ -271,14 +271,16 @@ __device__ __forceinline__ float4 ld_cluster_f32x4(uint32_t addr) {
   return v;
 }
 
-// Unit index of this CTA's i-th unit, read from the shared ring (-1: no more
-// units or an abort); `arrive` releases the slot for this reader.
+// Unit index of this CTA's i-th unit, read from the shared ring by a whole warp (-1: no
+// more units or an abort).  Lane 0 releases the slot for this reader after the shuffle,
+// when every lane has seen it full (a lane still waiting when the slot is filled again
+// would find the barrier's parity flipped back).
 __device__ __forceinline__ int read_unit(uint64_t* u_full, uint64_t* u_empty, const int* unit_slot, int i,
-                                         volatile int* abort, int* err, bool arrive) {
+                                         volatile int* abort, int* err, int lane) {
   const int s = i % U_SLOTS;
-  if (!mbar_wait(&u_full[s], (i / U_SLOTS) & 1, abort, err)) return -1;
-  const int u = unit_slot[s];
-  if (arrive) mbar_arrive(&u_empty[s]);
+  const bool ok = mbar_wait(&u_full[s], (i / U_SLOTS) & 1, abort, err);
+  const int u = __shfl_sync(0xffffffffu, ok ? unit_slot[s] : -1, 0);
+  if (lane == 0 && ok) mbar_arrive(&u_empty[s]);
   return u;
 }
 
@@ -501,7 +503,7 @@ __global__ void __launch_bounds__(THREADS, 1)
       __syncwarp();
     };
     for (int i = 0; ok; ++i) {
-      const int u = __shfl_sync(0xffffffffu, read_unit(u_full, u_empty, unit_slot, i, abort_flag, p.err, lane == 0), 0);
+      const int u = read_unit(u_full, u_empty, unit_slot, i, abort_flag, p.err, lane);
       if (u < 0) break;
       const Unit d = unit_at(u);
       if (!warp_wait(q_full, i & 1, abort_flag, p.err)) break;
@@ -595,7 +597,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     uint32_t nonfinite = 0;                       // range guard over this thread's output stores
     bool ok = true;
     for (int i = 0; ok; ++i) {
-      const int u = __shfl_sync(0xffffffffu, read_unit(u_full, u_empty, unit_slot, i, abort_flag, p.err, lane == 0), 0);
+      const int u = read_unit(u_full, u_empty, unit_slot, i, abort_flag, p.err, lane);
       if (u < 0) break;
       const Unit d = unit_at(u);
       if (t >= d.nt) {
