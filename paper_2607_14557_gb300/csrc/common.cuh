@@ -382,12 +382,13 @@ __device__ __forceinline__ void bulk_wait_read_1() { asm volatile("cp.async.bulk
 // Until every committed bulk group has completed.
 __device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 
-// 32-byte global store (one full sector); p must be 32-byte aligned.
-__device__ __forceinline__ void st_global_v8(void* p, uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t a4,
+// 32 bytes to global memory as two 16-byte stores; p must be 16-byte aligned, which is
+// what the entry points ask of a caller's buffers.
+__device__ __forceinline__ void st_global_32(void* p, uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t a4,
                                              uint32_t a5, uint32_t a6, uint32_t a7) {
-  asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(p), "r"(a0), "r"(a1), "r"(a2), "r"(a3),
-               "r"(a4), "r"(a5), "r"(a6), "r"(a7)
-               : "memory");
+  uint4* q = static_cast<uint4*>(p);
+  q[0] = make_uint4(a0, a1, a2, a3);
+  q[1] = make_uint4(a4, a5, a6, a7);
 }
 
 // Element storage types understood by the element-wise kernels.

@@ -443,9 +443,9 @@ __global__ void __launch_bounds__(THREADS, 1)
               } else {
 #pragma unroll
                 for (int i = 0; i < 2; ++i) {
-                  st_global_v8(crow + c0 + 16 * i, q0[8 * i], q0[8 * i + 1], q0[8 * i + 2], q0[8 * i + 3], q0[8 * i + 4],
+                  st_global_32(crow + c0 + 16 * i, q0[8 * i], q0[8 * i + 1], q0[8 * i + 2], q0[8 * i + 3], q0[8 * i + 4],
                                q0[8 * i + 5], q0[8 * i + 6], q0[8 * i + 7]);
-                  st_global_v8(crow + c1 + 16 * i, q1[8 * i], q1[8 * i + 1], q1[8 * i + 2], q1[8 * i + 3], q1[8 * i + 4],
+                  st_global_32(crow + c1 + 16 * i, q1[8 * i], q1[8 * i + 1], q1[8 * i + 2], q1[8 * i + 3], q1[8 * i + 4],
                                q1[8 * i + 5], q1[8 * i + 6], q1[8 * i + 7]);
                 }
               }
@@ -489,11 +489,11 @@ __global__ void __launch_bounds__(THREADS, 1)
               if (slab) {
                 store_chunk(second ? mC2 : mC, w, second ? col - p.split : col, second ? row2_0 : mt * BM + q * 32);
               } else {
-                // a lane owns one row: 64 contiguous bytes as two full 32-byte sectors
+                // a lane owns one row: 64 contiguous bytes
                 uint16_t* crow = second ? reinterpret_cast<uint16_t*>(p.C2) + static_cast<size_t>(row2) * p.ldc2 + col - p.split
                                         : reinterpret_cast<uint16_t*>(p.C) + static_cast<size_t>(row) * p.ldc + col;
-                st_global_v8(crow, w[0], w[1], w[2], w[3], w[4], w[5], w[6], w[7]);
-                st_global_v8(crow + 16, w[8], w[9], w[10], w[11], w[12], w[13], w[14], w[15]);
+                st_global_32(crow, w[0], w[1], w[2], w[3], w[4], w[5], w[6], w[7]);
+                st_global_32(crow + 16, w[8], w[9], w[10], w[11], w[12], w[13], w[14], w[15]);
               }
             }
           }
@@ -544,8 +544,8 @@ __global__ void __launch_bounds__(THREADS, 1)
               if (slab_full) {
                 store_chunk(mC, w, n * tile_n + c * 32, mt * BM + q * 32);
               } else {
-                st_global_v8(arow + c * 32, w[0], w[1], w[2], w[3], w[4], w[5], w[6], w[7]);
-                st_global_v8(arow + c * 32 + 16, w[8], w[9], w[10], w[11], w[12], w[13], w[14], w[15]);
+                st_global_32(arow + c * 32, w[0], w[1], w[2], w[3], w[4], w[5], w[6], w[7]);
+                st_global_32(arow + c * 32 + 16, w[8], w[9], w[10], w[11], w[12], w[13], w[14], w[15]);
               }
             }
           }

@@ -29,6 +29,16 @@ def i32(a):
     return torch.as_tensor(np.asarray(a, dtype=np.int32)).to(cuda())
 
 
+def at_16(t):
+    """A copy of t that starts on a 16-byte boundary, not on a 32-byte one."""
+    n = 16 // t.element_size()
+    buf = torch.empty(t.numel() + n, dtype=t.dtype, device=t.device)
+    out = buf[n:].view(t.shape)
+    out.copy_(t)
+    assert out.data_ptr() % 32 == 16
+    return out
+
+
 def host(t):
     return t.detach().float().cpu().numpy().astype(np.float64)
 

@@ -8,7 +8,7 @@ import torch
 
 import oracle
 import synth
-from tests.helpers import check_close, cuda, host, i32, to_dev
+from tests.helpers import at_16, check_close, cuda, host, i32, to_dev
 
 pytestmark = pytest.mark.gpu
 
@@ -137,6 +137,40 @@ def test_cached_layer_long_prefixes_few_rows(ctx, resp):
         pre = k[cu[b]:cu[b] + c]
         ref = oracle.layer_forward_cached(x[cr[b]:cr[b + 1]], pre[:, :d], pre[:, d:], w, H)
         check_close(got[cr[b]:cr[b + 1]], ref, "bf16", f"cached block segment {b}")
+
+
+@pytest.mark.parametrize("rope", [0.0, 1e4])
+def test_layer_and_cache_buffers_on_16_byte_boundaries(rope):
+    """A layer, a prefill and a cached layer whose activations, cache and workspace start
+    on 16-byte boundaries, not 32-byte ones: segments of odd lengths, so rows reach the
+    cache one by one; the same bits as from buffers on larger boundaries."""
+    wl = _workload("bf16")
+    from paper_2607_14557_gb300 import driver as D
+    W = D.LayerWeights.from_host(synth.layer_weights(wl, 0), "bf16")
+    d, ctx, resp = wl.d, [33, 7, 64], [21, 40, 5]
+    B, cu, cr = len(ctx), np.concatenate([[0], np.cumsum(np.add(ctx, resp))]), np.concatenate([[0], np.cumsum(resp)])
+    T, R = int(cu[-1]), int(cr[-1])
+    dims = S.make_dims(d, wl.n_heads, wl.head_dim, wl.d_ff, rope_theta=rope)
+    n = S.seer_layer_workspace_size(dims, "bf16", T, B)
+    g = torch.Generator(device="cuda").manual_seed(5)
+    x = torch.randn((T, d), generator=g, device="cuda").bfloat16()
+    xr = torch.cat([x[int(a) + c:int(b)] for a, b, c in zip(cu[:-1], cu[1:], ctx)])
+    out = []
+    for place in (lambda t: t, at_16):
+        ws = place(torch.zeros(n, dtype=torch.uint8, device="cuda"))
+        y = place(torch.zeros((T, d), dtype=torch.bfloat16, device="cuda"))
+        S.seer_layer_forward(W.struct(), dims, "bf16", place(x), y, i32(cu), None, B, T, None, 0, 0.0, None, ws, n)
+        got = [y]
+        if not rope:                                                   # the cache path has no rotary embedding
+            cache = place(torch.zeros((T, 2 * d), dtype=torch.float16, device="cuda"))
+            yr = place(torch.zeros((R, d), dtype=torch.bfloat16, device="cuda"))
+            S.seer_kv_prefill(W.struct(), dims, "bf16", place(x), i32(cu), i32(ctx), B, T, cache, i32(cu), T, ws, n)
+            S.seer_layer_forward_cached(W.struct(), dims, "bf16", place(xr), yr, i32(cr), i32(ctx), B, R, cache, i32(cu),
+                                        None, T, ws, n)
+            got += [cache, yr]
+        out.append(got)
+    assert all(torch.equal(p, q) for p, q in zip(*out))
+    assert all(t.any() for t in out[0])
 
 
 def test_cache_entry_points_reject_bad_arguments():

@@ -13,7 +13,7 @@ import torch
 
 import oracle
 import synth
-from tests.helpers import check_close, cuda, host, i32, tdtype, to_dev
+from tests.helpers import at_16, check_close, cuda, host, i32, tdtype, to_dev
 
 pytestmark = pytest.mark.gpu
 
@@ -94,6 +94,25 @@ def test_linear_tile_choices(M, N, K, res):
     ref = ad.double() @ wd.double().T + (rd.double() if res else 0.0)
     assert torch.equal(c[:M], ref.to(torch.bfloat16))
     assert torch.isnan(c[M]).all()                                  # nothing past the last row
+
+
+@pytest.mark.parametrize("M", [1, 45, 300])                          # rows stored lane by lane, alone and after full slabs
+def test_gemm_outputs_on_16_byte_boundaries(M):
+    """Operands, residual and outputs need 16-byte alignment, not 32: the same bits as
+    from buffers on larger boundaries."""
+    N, K = 256, 128
+    g = torch.Generator(device="cuda").manual_seed(M)
+    r = lambda *s: torch.randn(s, generator=g, device="cuda").half()
+    a, w, w2, res = r(M, K), 0.1 * r(N, K), 0.1 * r(N, K), r(M, N)
+    out = []
+    for place in (lambda t: t, at_16):
+        c = [place(torch.zeros((M, N), dtype=torch.float16, device="cuda")) for _ in range(3)]
+        a_, w_, w2_, res_ = place(a), place(w), place(w2), place(res)
+        S.seer_linear(a_, w_, "f16", None, "f16", c[0], "f16", M, None, N, K)
+        S.seer_linear(a_, w_, "f16", res_, "f16", c[1], "f16", M, None, N, K)
+        S.seer_swiglu(a_, w_, w2_, "f16", c[2], "f16", M, None, N, K)
+        out.append(c)
+    assert all(torch.equal(p, q) for p, q in zip(*out))
 
 
 @pytest.mark.parametrize("M,N,K", [(127, 1024, 12288), (300, 4096, 12288)])
