@@ -788,6 +788,11 @@ cudaError_t launch_snr_scan(const int* counts, int B, int N, int F, double tau_j
                             int* L_star, int* i_star, cudaStream_t st) {
   if (B <= 0) return cudaSuccess;
   const size_t sm = N <= kScanSmemInts ? static_cast<size_t>(N) * sizeof(int) : 0;
+  if (sm + sizeof(int) * (kScanThreads / 32) > 48 * 1024) {     // with the kernel's own array past the default limit
+    static bool attr_set[64] = {};
+    cudaError_t e = set_smem_limit_once(snr_scan_kernel, kScanSmemInts * static_cast<int>(sizeof(int)), attr_set);
+    if (e != cudaSuccess) return e;
+  }
   return launch_kernel(snr_scan_kernel, dim3(B), dim3(kScanThreads), sm, st, counts, N, F, tau_jump, gamma, window, L_star, i_star);
 }
 

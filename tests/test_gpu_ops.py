@@ -643,7 +643,7 @@ def test_pack_route_bucket_set_variants(bucket_min):
     _pack_case("bf16", ctx, L, 1024, 256, seed=30 + bucket_min, bucket_min=bucket_min)
 
 
-@pytest.mark.parametrize("N,w", [(2, 1), (4, 3), (129, 3), (130, 1), (257, 10), (12289, 3)])
+@pytest.mark.parametrize("N,w", [(2, 1), (4, 3), (129, 3), (130, 1), (257, 10), (12284, 3), (12285, 3), (12288, 3), (12289, 3)])
 @pytest.mark.parametrize("F,tau,gamma", [(12288, 0.03, 0.6), (100, 0.07, 0.5), (3 * 12288, 0.0, 0.0), (7, 3 / 7, 1.0)])
 def test_snr_scan_at_the_thresholds(N, w, F, tau, gamma):
     """Counts whose jump and noise land on, just under and just over tau F and gamma
