@@ -483,8 +483,11 @@ __device__ __forceinline__ int graph_capacity(int total) {
 // publishes it, then all blocks copy rows.  Segments, buckets and control words are
 // each handled side by side by the block's threads: with one thread walking them (its
 // loads, fp64 quotients and the 135 words it stored to host memory) a batch of one
-// took 13 us, now 8.7; 32 segments, 77k rows of 8 KB 205.6 -> 201.5 us.  Dynamic smem: seg/cu/bucket-index arrays of
-// B+1 ints each.
+// took 13 us, now 8.7; 32 segments, 77k rows of 8 KB 205.6 -> 201.5 us.  Dynamic smem
+// (route_smem_bytes): the segments' lengths and offsets as ints, their buckets as bytes.
+__host__ __device__ constexpr size_t route_smem_bytes(int B) {
+  return (2 * static_cast<size_t>(B) + 1) * sizeof(int) + static_cast<size_t>(B);
+}
 __global__ void __launch_bounds__(256, 4) pack_route_kernel(const uint8_t* __restrict__ x_full, int row_bytes,
                                                          const int* __restrict__ cu_full,
                                                          const int* __restrict__ ctx_len,
@@ -496,7 +499,7 @@ __global__ void __launch_bounds__(256, 4) pack_route_kernel(const uint8_t* __res
   extern __shared__ int dyn[];
   int* seg = dyn;              // [B]
   int* cus = dyn + B;          // [B+1]
-  int* bidx = dyn + 2 * B + 1; // [B]
+  uint8_t* bidx = reinterpret_cast<uint8_t*>(dyn + 2 * B + 1);   // [B], below kCtrlMaxGroups
   __shared__ RouteSmem rs;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
@@ -530,7 +533,7 @@ __global__ void __launch_bounds__(256, 4) pack_route_kernel(const uint8_t* __res
     }
     int k = 0;
     while (k < rs.n_buckets - 1 && Ls > rs.bucket[k]) ++k;
-    bidx[i] = k;
+    bidx[i] = static_cast<uint8_t>(k);
     atomicAdd(&rs.count[k], 1);
     atomicAdd(reinterpret_cast<unsigned long long*>(&rs.sum[k]), static_cast<unsigned long long>(Ls));
   }
@@ -800,8 +803,8 @@ cudaError_t launch_pack_route(const void* x_full, int elem_bytes, const int* cu_
                               const int* L_star, int B, int d, int N, int T_cap, double tau_pad,
                               int eager_max_bucket, int bucket_min, void* x_packed, int* cu_out, int* kv_out,
                               int* meta_out, int* host_ctrl_dev, int epoch, int* err, int num_sms, cudaStream_t st) {
-  const size_t sm = static_cast<size_t>(3 * B + 1) * sizeof(int);
-  if (sm > 48 * 1024) {
+  const size_t sm = route_smem_bytes(B);
+  if (sm + sizeof(RouteSmem) > 48 * 1024) {
     cudaError_t e = cudaFuncSetAttribute(pack_route_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          static_cast<int>(sm));
     if (e != cudaSuccess) return e;

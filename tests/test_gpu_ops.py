@@ -669,9 +669,11 @@ def test_snr_scan_at_the_thresholds(N, w, F, tau, gamma):
     np.testing.assert_array_equal(L.cpu().numpy(), L_ref)
 
 
-@pytest.mark.parametrize("B,N,bucket_min", [(1, 1, 1), (33, 1000, 8), (64, 64, 1), (300, 4096, 3), (1000, 17, 8)])
+@pytest.mark.parametrize("B,N,bucket_min", [(1, 1, 1), (33, 1000, 8), (64, 64, 1), (300, 4096, 3), (1000, 17, 8),
+                                            (4000, 17, 8), (5327, 17, 8), (5328, 17, 8), (19303, 17, 8)])
 def test_pack_route_many_segments(B, N, bucket_min):
-    """More segments than a warp, every bucket count, rows of 48 bytes .. 8 KB."""
+    """More segments than a warp, every bucket count, rows of 48 bytes .. 8 KB; segments
+    whose lengths, offsets and buckets need more than the default shared memory."""
     rng = _rng(B + N)
     ctx, L = rng.integers(0, 20, B), rng.integers(1, N + 1, B)
     _pack_case("bf16", ctx, L, N, 24 if B > 100 else 4096, seed=B, bucket_min=bucket_min)
