@@ -4,6 +4,7 @@
 //   snr_scan         Seer Sec. 3.3 boundary criterion, one warp per sequence
 //   pack_route       Seer Sec. 3.4-3.5: micro-bucket routing (Eq. 4) fused
 //                    with device-resident compaction and the pinned control word
+#include <float.h>
 #include <math.h>
 
 #include "attn_schedule.cuh"
@@ -416,7 +417,10 @@ __global__ void __launch_bounds__(kScanThreads) snr_scan_kernel(const int* __res
     c = staged;
   }
   const double Fd = static_cast<double>(F);
-  const float need = static_cast<float>(tau_jump * Fd), g = static_cast<float>(gamma);
+  // gamma beyond the fp32 range is held at its ends: infinity times a jump of 0 would
+  // reject a candidate that the exact test takes (a NaN passes on to it, and fails there)
+  const float need = static_cast<float>(tau_jump * Fd);
+  const float g = fminf(fmaxf(static_cast<float>(gamma), -FLT_MAX), FLT_MAX);
   int found = -1;
   const int last = N - window;   // inclusive
   for (int base = 1; base <= last; base += kScanThreads) {

@@ -669,6 +669,19 @@ def test_snr_scan_at_the_thresholds(N, w, F, tau, gamma):
     np.testing.assert_array_equal(L.cpu().numpy(), L_ref)
 
 
+@pytest.mark.parametrize("tau", [0.0, -1.0, 1e300, -1e300])
+@pytest.mark.parametrize("gamma", [0.6, 1e38, 1e300, -1e300, float("inf")])
+def test_snr_scan_parameters_beyond_the_fp32_range(tau, gamma):
+    """Thresholds that the fp32 filter cannot hold: flat, rising, falling and noisy counts."""
+    c = np.array([[5] * 20, [5] * 8 + [9] * 12, [9] * 8 + [5] * 12, [3, 7] * 10, list(range(20))], dtype=np.int32)
+    B, N = c.shape
+    L, I = torch.empty(B, dtype=torch.int32, device=cuda()), torch.empty(B, dtype=torch.int32, device=cuda())
+    S.seer_snr_scan(torch.from_numpy(c).to(cuda()), B, N, 768, S.make_params(0.0, tau_jump=tau, gamma=gamma, window=3), L, I)
+    i_ref, L_ref = oracle.snr_boundaries(c, 768, tau, gamma, 3)
+    np.testing.assert_array_equal(I.cpu().numpy(), i_ref)
+    np.testing.assert_array_equal(L.cpu().numpy(), L_ref)
+
+
 @pytest.mark.parametrize("B,N,bucket_min", [(1, 1, 1), (33, 1000, 8), (64, 64, 1), (300, 4096, 3), (1000, 17, 8),
                                             (4000, 17, 8), (5327, 17, 8), (5328, 17, 8), (19303, 17, 8)])
 def test_pack_route_many_segments(B, N, bucket_min):
