@@ -188,7 +188,8 @@ __global__ void __launch_bounds__(THREADS, 1)
   constexpr bool halfN = (MODE == kGemmSwiglu || MODE == kGemmCount);
   // the tile choice for the rows there are: a call sized for more may be better off
   // with other tiles (tc_gemm_plan)
-  const bool few = !halfN && MODE != kGemmRope && (num_mt + CG - 1) / CG <= p.few_m;
+  // (no second choice: few_m = 0, which a row count of 0 would meet)
+  const bool few = !halfN && MODE != kGemmRope && p.few_m > 0 && (num_mt + CG - 1) / CG <= p.few_m;
   const int BN = few ? p.few_bn : p.bn;
   const int stages = few ? p.few_stages : p.stages;         // of DEPTH k-blocks
   const int bbytes = stage_bytes(CG, BN);                   // operand bytes of a k-block
