@@ -228,16 +228,21 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN), MIN_BLOCKS)
 // 4 tx .. 4 tx + 3 (and + 64).  The next K tile is copied by cp.async while the
 // current tile's softmax and PV run, the next V tile while the next scores do.
 // Bound by shared-memory reads (two passes each, see the GEMM's lanes) beside as many
-// FMA cycles.  A warp per (row, head) that reads every key itself took 1209 us for the
-// 8-segment batch of 58 .. 794 rows, 8 heads of 64; this kernel 140 (146 with 16
-// consecutive lanes along a row, four passes for K and V).
+// FMA cycles.  A warp per (row, head) that reads every key itself took 1190 us for an
+// 8-segment batch of 58 .. 790 rows, 8 heads of 64; this kernel 132.
+// Blocks per SM are what its shared memory allows, so the registers are bounded to it:
+// five blocks at 16 rows and 128 threads (without the bound 114 registers let four in,
+// one segment of 1500 rows 216 -> 308 us); heads wider than 64 (HALVES = 2: a second
+// float4 of output columns per thread) fit two blocks, and bounded as the others they
+// spilled (four of 1000 rows, 4 heads of 128: 395 -> 441).
 constexpr int AKV = 64;                      // keys per tile
 constexpr int APS = AKV + 16;                // floats per row of probabilities (two rows meet no bank twice)
 
 __host__ __device__ constexpr int attn_ld(int dh) { return 4 * ((dh / 4) | 1); }   // an odd number of 16-byte words
 
-template <int BQ, int TY, int VEC>
-__global__ void __launch_bounds__(16 * TY) simt_attn_kernel(const float* __restrict__ qkv, const AttnParams p) {
+template <int BQ, int TY, int VEC, int HALVES>
+__global__ void __launch_bounds__(16 * TY, HALVES == 2 ? 2 : (BQ == 32 ? 4 : (TY == 8 ? 5 : 3)))
+    simt_attn_kernel(const float* __restrict__ qkv, const AttnParams p) {
   pdl_enter();
   constexpr int TM = BQ / TY;
   const int H = p.n_heads, dh = p.head_dim, D = H * dh;
@@ -300,37 +305,55 @@ __global__ void __launch_bounds__(16 * TY) simt_attn_kernel(const float* __restr
   load_keys(Vs, p.xv0, 0);
 
   const float scale = 1.0f / sqrtf(static_cast<float>(dh));
-  float m[TM], l[TM], o[TM][8];
+  float m[TM], l[TM], o[TM][4 * HALVES];
 #pragma unroll
   for (int i = 0; i < TM; ++i) {
     m[i] = -INFINITY;
     l[i] = 0.f;
 #pragma unroll
-    for (int c = 0; c < 8; ++c) o[i][c] = 0.f;
+    for (int c = 0; c < 4 * HALVES; ++c) o[i][c] = 0.f;
   }
-  const int c0 = 4 * tx, c1 = 64 + 4 * tx;            // output columns of this thread
-  const bool has0 = c0 < dh, has1 = c1 < dh;
+  const int c0 = 4 * tx;                              // output columns of this thread: c0 .. c0 + 3 (and + 64)
   const int tiles = (kvL + AKV - 1) / AKV;
   for (int t = 0; t < tiles; ++t) {
     cp_async_wait<1>();                               // K of tile t (its V is the group after)
     __syncthreads();
-    float sc[TM][4] = {};
-    for (int k = 0; k < dh; k += 4) {
-      float4 kk[4];
+    // A score is summed in blocks of 16 dims, each two packed chains of 8, and the blocks
+    // in two chains: about the roundings of a tree over a warp's lanes.  One chain over the
+    // head's dims was up to 2.5 times further from 64 bits (q and k of size 3, 2 heads of
+    // 128, 1000 rows: 1.76e-6; so 5.7e-7, a warp per row 7.0e-7; of size 1 7.0e-7, 5.9e-7
+    // and 7.5e-7) and no faster at heads of 64 (132 and 136 us above; of 128 2-4% faster).
+    float sc[TM][4] = {}, odd[TM][4] = {};
+    for (int k0 = 0; k0 < dh; k0 += 16) {
+      float2 part[TM][4] = {};
+#pragma unroll 1
+      for (int k = k0; k < min(k0 + 16, dh); k += 4) {
+        float4 kk[4];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) kk[j] = *reinterpret_cast<const float4*>(Ks + (tx + 16 * j) * ld + k);
+        for (int j = 0; j < 4; ++j) kk[j] = *reinterpret_cast<const float4*>(Ks + (tx + 16 * j) * ld + k);
 #pragma unroll
-      for (int i = 0; i < TM; ++i) {
-        const float4 q = *reinterpret_cast<const float4*>(Qs + (ty + TY * i) * ld + k);
+        for (int i = 0; i < TM; ++i) {
+          const float4 q = *reinterpret_cast<const float4*>(Qs + (ty + TY * i) * ld + k);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          sc[i][j] = fmaf(q.x, kk[j].x, sc[i][j]);
-          sc[i][j] = fmaf(q.y, kk[j].y, sc[i][j]);
-          sc[i][j] = fmaf(q.z, kk[j].z, sc[i][j]);
-          sc[i][j] = fmaf(q.w, kk[j].w, sc[i][j]);
+          for (int j = 0; j < 4; ++j) {
+            ffma2(part[i][j], q.x, q.y, kk[j].x, kk[j].y);
+            ffma2(part[i][j], q.z, q.w, kk[j].z, kk[j].w);
+          }
         }
       }
+#pragma unroll
+      for (int i = 0; i < TM; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const float v = part[i][j].x + part[i][j].y;
+          if (k0 & 16) odd[i][j] += v;
+          else sc[i][j] += v;
+        }
     }
+#pragma unroll
+    for (int i = 0; i < TM; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) sc[i][j] += odd[i][j];
     __syncthreads();                                  // every warp is done with K
     if (t + 1 < tiles) load_keys(Ks, p.xk0, (t + 1) * AKV);
     else cp_async_commit();
@@ -356,7 +379,7 @@ __global__ void __launch_bounds__(16 * TY) simt_attn_kernel(const float* __restr
       }
       l[i] = l[i] * alpha + sum;                      // this thread's share; summed over the row at the end
 #pragma unroll
-      for (int c = 0; c < 8; ++c) o[i][c] *= alpha;
+      for (int c = 0; c < 4 * HALVES; ++c) o[i][c] *= alpha;
     }
     cp_async_wait<1>();                               // V of tile t
     __syncthreads();
@@ -368,26 +391,17 @@ __global__ void __launch_bounds__(16 * TY) simt_attn_kernel(const float* __restr
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
         const float* vrow = Vs + (k + e) * ld;
-        if (has0) {
-          const float4 v = *reinterpret_cast<const float4*>(vrow + c0);
+#pragma unroll
+        for (int h2 = 0; h2 < HALVES; ++h2) {
+          if (c0 + 64 * h2 >= dh) continue;
+          const float4 v = *reinterpret_cast<const float4*>(vrow + c0 + 64 * h2);
 #pragma unroll
           for (int i = 0; i < TM; ++i) {
             const float w = e == 0 ? pr[i].x : (e == 1 ? pr[i].y : (e == 2 ? pr[i].z : pr[i].w));
-            o[i][0] = fmaf(w, v.x, o[i][0]);
-            o[i][1] = fmaf(w, v.y, o[i][1]);
-            o[i][2] = fmaf(w, v.z, o[i][2]);
-            o[i][3] = fmaf(w, v.w, o[i][3]);
-          }
-        }
-        if (has1) {
-          const float4 v = *reinterpret_cast<const float4*>(vrow + c1);
-#pragma unroll
-          for (int i = 0; i < TM; ++i) {
-            const float w = e == 0 ? pr[i].x : (e == 1 ? pr[i].y : (e == 2 ? pr[i].z : pr[i].w));
-            o[i][4] = fmaf(w, v.x, o[i][4]);
-            o[i][5] = fmaf(w, v.y, o[i][5]);
-            o[i][6] = fmaf(w, v.z, o[i][6]);
-            o[i][7] = fmaf(w, v.w, o[i][7]);
+            o[i][4 * h2 + 0] = fmaf(w, v.x, o[i][4 * h2 + 0]);
+            o[i][4 * h2 + 1] = fmaf(w, v.y, o[i][4 * h2 + 1]);
+            o[i][4 * h2 + 2] = fmaf(w, v.z, o[i][4 * h2 + 2]);
+            o[i][4 * h2 + 3] = fmaf(w, v.w, o[i][4 * h2 + 3]);
           }
         }
       }
@@ -405,9 +419,10 @@ __global__ void __launch_bounds__(16 * TY) simt_attn_kernel(const float* __restr
     if (r >= rows) continue;
     float* out = reinterpret_cast<float*>(p.out) + static_cast<size_t>(seq0 + q0 + r) * p.ldo + h * dh;
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      if (has0) out[c0 + c] = o[i][c] / sum;
-      if (has1) out[c1 + c] = o[i][4 + c] / sum;
+    for (int h2 = 0; h2 < HALVES; ++h2) {
+      if (c0 + 64 * h2 >= dh) continue;
+#pragma unroll
+      for (int c = 0; c < 4; ++c) out[c0 + 64 * h2 + c] = o[i][4 * h2 + c] / sum;
     }
   }
 }
@@ -474,16 +489,21 @@ cudaError_t launch_mode(const float* A, const float* B0, const float* B1, const 
   return launch_tile<MODE, 16, 32, 2, 2, 32, 6, 1>(A, B0, B1, p, vec, st);
 }
 
-template <int BQ, int TY, int VEC>
-cudaError_t launch_attn(const float* qkv, const AttnParams& p, cudaStream_t st) {
+template <int BQ, int TY, int VEC, int HALVES>
+cudaError_t launch_attn_halves(const float* qkv, const AttnParams& p, cudaStream_t st) {
   const long blocks = ((static_cast<long>(p.T_cap) + BQ - 1) / BQ + p.B) * p.n_heads;
   if (blocks > 0x7fffffffL) return cudaErrorInvalidValue;
   constexpr auto bytes = [](int dh) { return static_cast<int>(sizeof(float)) * ((BQ + 2 * AKV) * attn_ld(dh) + BQ * APS); };
   static bool attr_set[64] = {};
-  cudaError_t e = set_smem_limit_once(simt_attn_kernel<BQ, TY, VEC>, bytes(128), attr_set);
+  cudaError_t e = set_smem_limit_once(simt_attn_kernel<BQ, TY, VEC, HALVES>, bytes(64 * HALVES), attr_set);
   if (e != cudaSuccess) return e;
-  return launch_kernel(simt_attn_kernel<BQ, TY, VEC>, dim3(static_cast<unsigned>(blocks)), dim3(16 * TY), bytes(p.head_dim), st,
-                       qkv, p);
+  return launch_kernel(simt_attn_kernel<BQ, TY, VEC, HALVES>, dim3(static_cast<unsigned>(blocks)), dim3(16 * TY),
+                       bytes(p.head_dim), st, qkv, p);
+}
+
+template <int BQ, int TY, int VEC>
+cudaError_t launch_attn(const float* qkv, const AttnParams& p, cudaStream_t st) {
+  return p.head_dim <= 64 ? launch_attn_halves<BQ, TY, VEC, 1>(qkv, p, st) : launch_attn_halves<BQ, TY, VEC, 2>(qkv, p, st);
 }
 
 }  // namespace
@@ -506,12 +526,14 @@ cudaError_t launch_simt_attn(const float* qkv, const AttnParams& p, int num_sms,
   const bool vec = aligned(qkv) && (p.kv == nullptr || (aligned(p.kv) && p.ld_kv % 4 == 0)) && p.xk0 % 4 == 0 && p.xv0 % 4 == 0;
   // 32-row tiles once their blocks fill the SMs three times (unless most segments are
   // far shorter); else 16-row tiles, with twice the threads unless heads of at most 64
-  // let four blocks share an SM and the blocks fill the SMs four times.  Measured at 32
-  // rows / 16 rows / 16 rows with 256 threads, us: segments of 58 .. 794 rows, 8 heads of
-  // 64 (4.7 times) 141 / 159 / 163; four of 500 (3.5) 96 / 120 / 123; four of 800, 4 heads
-  // of 128 (2.7) 295 / 345 / 267; one of 1500, 8 heads of 64 (2.5; 16 rows 5.0) 274 / 230 /
-  // 260; one of 700 (1.2; 2.4) 100 / 78 / 75; sixteen of 60, 8 heads of 32 (2.4; 4.0) 14.5 /
-  // 13.7 / 11.5; one of 121, 4 heads 15.8 / 12.7 / 8.2; 64-row tiles 194 at the first.
+  // let five blocks share an SM and the blocks fill the SMs four times.  Measured at 32
+  // rows / 16 rows / 16 rows with 256 threads, us: segments of 58 .. 790 rows, 8 heads of
+  // 64 (4.7 times) 132 / 148 / 151; four of 500 (3.5) 92 / 109 / 115; four of 800, 4 heads
+  // of 128 (2.7) 281 / 348 / 273; one of 1500, 8 heads of 64 (2.5; 16 rows 4.9) 262 / 216 /
+  // 241; one of 700 (1.2; 2.3) 85 / 90 / 69; sixteen of 60, 8 heads of 32 (2.4; 4.0) 13.0 /
+  // 10.8 / 10.8; one of 121, 4 heads 15.4 / 11.5 / 8.1.  Of 28 shapes it misses the best by
+  // more than 5% at four: six of 300, 8 heads of 128 126 / 138 / 109; one of 1000 199 / 287 /
+  // 225; eight of 300, 8 heads of 32 71 / 64 / 64; eight of 40, 8 heads of 64 9.7 / 7.8 / 8.5.
   const auto blocks = [&](long bq) { return (p.T_cap / bq + p.B) * p.n_heads; };
   if (blocks(32) >= 3l * num_sms && p.T_cap / p.B >= 16)
     return vec ? launch_attn<32, 8, 4>(qkv, p, st) : launch_attn<32, 8, 1>(qkv, p, st);

@@ -219,6 +219,23 @@ def test_attention_f32_tile_choices(H, dh, lens, kv, offset):
     assert torch.isnan(o[T]).all()
 
 
+@pytest.mark.parametrize("H,dh,T", [(2, 128, 1000), (8, 64, 353), (40, 64, 400), (4, 32, 121)])
+def test_attention_f32_error_at_large_scores(H, dh, T):
+    """Scores of magnitude ~9 (up to ~45): a score summed in blocks is off by about sqrt(7)
+    roundings of 2^-24 / sqrt(3) of it, 9e-8 x 9 = 8e-7 in the exponent and less in a row's
+    result, where its keys' errors average out; one chain over the head's dims is off by
+    three times as much at 128 dims (measured 1.8e-6, in blocks 0.6e-6)."""
+    D = H * dh
+    g = torch.Generator(device="cuda").manual_seed(T)
+    qkv = torch.randn((T, 3 * D), generator=g, device="cuda")
+    qkv[:, :2 * D] *= 3.0
+    o = torch.empty((T, D), device="cuda")
+    S.seer_attention(qkv, o, "f32", i32([0, T]), None, 1, T, H, dh)
+    q, k, v = (t.view(T, H, dh).transpose(0, 1) for t in qkv.double().split(D, 1))
+    ref = (torch.softmax(q @ k.transpose(1, 2) / dh ** 0.5, -1) @ v).transpose(0, 1).reshape(T, D)
+    assert ((o.double() - ref).norm() / ref.norm()).item() < 8e-7
+
+
 # ------------------------------------------------------------------ SwiGLU + count hook (S10, S1)
 @pytest.mark.parametrize("op", ["bf16", "f16"])
 def test_swiglu_counts_at_the_threshold_follow_the_ieee_quotient(op):
