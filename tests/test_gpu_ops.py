@@ -264,6 +264,31 @@ def test_swiglu_counts_at_the_threshold_follow_the_ieee_quotient(op):
         np.testing.assert_array_equal(counts(op, float(eps))[1], counts("f32", float(eps))[1], err_msg=f"eps={eps}")
 
 
+@pytest.mark.parametrize("op,act,up", [("bf16", "bf16", 3.0), ("f16", "bf16", 3.0), ("bf16", "f16", 2.0 ** 116),
+                                      ("f16", "f16", 3.0)])
+def test_swiglu_stores_what_the_ieee_quotient_gives_at_very_negative_gates(op, act, up):
+    """Gates of -88 and -87.5, whose approximate quotient is 0: the fp32 path's activation
+    (of about -5e-37 times u) rounded once to the output's type, nonzero where that type
+    or a large u can show it; gates of 1 in the same chunk of columns stay right."""
+    M, F, K = 130, 128, 64
+    a, wg, wu = (np.zeros(s, dtype=np.float32) for s in ((M, K), (F, K), (F, K)))
+    a[:, 0], a[:, 1], a[:, 2] = -88.0, -87.5, 1.0
+    wg[np.arange(F), np.arange(F) % 3] = 1.0
+    wu[:, 2] = up
+    out = {}
+    for dt, ot in (("f32", "f32"), (op, act)):
+        o = torch.empty((M, F), dtype=tdtype(ot), device=cuda())
+        S.seer_swiglu(to_dev(a, dt), to_dev(wg, dt), to_dev(wu, dt), dt, o, ot, M, None, F, K)
+        out[ot] = o
+    if (op, act) == ("bf16", "f16"):                                  # silu(1) * 2^116 is beyond f16, and recorded
+        assert S.seer_check_device() == 6
+    want, low = out["f32"].to(tdtype(act)), np.arange(F) % 3 < 2
+    assert torch.equal(out[act][:, low], want[:, low])
+    assert (out[act][:, low] != 0).all() == (act == "bf16" or op == "bf16")
+    ref, got = out["f32"][:, ~low].double(), out[act][:, ~low].double()
+    assert ((got - ref).abs() <= 1e-2 * ref.abs()).all() or act == "f16" and op == "bf16"
+
+
 @pytest.mark.parametrize("op", ["bf16", "f16", "f32"])
 def test_swiglu_with_count_hook(op):
     rng = _rng(7)
