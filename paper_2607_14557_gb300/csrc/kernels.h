@@ -50,7 +50,8 @@ struct GemmParams {
   int res_type;           // ElemType of R
   int bn;                 // accumulator columns per tile (multiple of 32)
   int stages;             // operand ring: stages
-  int few_m;              // with at most this many row tiles (of cg * 128 rows), instead of bn ...
+  int few_m;              // with at most this many row tiles (of cg * 128 rows), and bit (row tiles - 1) ...
+  uint64_t few_mask;      // ... of this set (counts above 64: always), instead of bn ...
   int few_bn;             // ... this many columns per tile (single-weight modes; mB1 has its boxes) ...
   int few_stages;         // ... and stages
   int group_m;            // raster: row tiles per group (see tc_gemm.cu)
@@ -94,7 +95,8 @@ struct GemmPlan {
   int group_m;   // raster: row tiles per group
   int depth;     // 64-deep k-blocks per stage: 1 or 2
   int few_m;     // tile choice of a call whose device row count leaves at most few_m row
-  int few_bn;    // tiles: few_bn columns (few_m = 0: no second choice)
+  int few_bn;    // tiles: few_bn columns (few_m = 0: no second choice), but for counts of
+  uint64_t few_mask;   // up to 64 row tiles only those whose bit (row tiles - 1) is set
 };
 // m_tiles: 128-row tiles; n_cols: accumulator columns (N; Swiglu / Count: 2 F);
 // K: depth; device_rows: the row count is read on the device (m_tiles is a bound);

@@ -191,14 +191,14 @@ __global__ void __launch_bounds__(THREADS, 1)
   constexpr bool halfN = (MODE == kGemmSwiglu || MODE == kGemmCount);
   // the tile choice for the rows there are: a call sized for more may be better off
   // with other tiles (tc_gemm_plan)
-  // (no second choice: few_m = 0, which a row count of 0 would meet)
-  const bool few = !halfN && MODE != kGemmRope && p.few_m > 0 && (num_mt + CG - 1) / CG <= p.few_m;
+  const int num_m = (num_mt + CG - 1) / CG;
+  const bool few = !halfN && MODE != kGemmRope && num_m > 0 && num_m <= p.few_m &&
+                   (num_m > 64 || ((p.few_mask >> (num_m - 1)) & 1) != 0);
   const int BN = few ? p.few_bn : p.bn;
   const int stages = few ? p.few_stages : p.stages;         // of DEPTH k-blocks
   const int bbytes = stage_bytes(CG, BN);                   // operand bytes of a k-block
   const int sbytes = DEPTH * bbytes;
   const int tile_n = halfN ? BN / 2 : BN;                   // columns of p.N covered by a tile
-  const int num_m = (num_mt + CG - 1) / CG;
   const int num_n = (p.N + tile_n - 1) / tile_n;
   const int num_tiles = num_m * num_n;
   const int KB = p.K / BK;
@@ -617,6 +617,7 @@ cudaError_t launch_mode(const GemmPlan& plan, const CUtensorMap& mA, const CUten
   }
   p.bn = plan.bn;
   p.few_m = plan.few_m;
+  p.few_mask = plan.few_mask;
   p.few_bn = plan.few_bn;
   p.few_stages = plan.few_m > 0 ? plan_stages(CG, plan.few_bn, DEPTH) : 0;
   p.stages = plan.stages;
@@ -663,9 +664,13 @@ cudaError_t launch_cg(const GemmPlan& plan, const CUtensorMap& mA, const CUtenso
 // 17.8, down 39.7 / 40.3; at 224 columns 842 rows down 61.0 / 63.2).
 // A row count read on the device may leave fewer row tiles than the call is sized
 // for (a packed batch in buffers for its full windows): single-weight modes then get
-// a second width for four fifths of the tiles, and among choices within 8% of the
-// best at full size the one that is best over both is taken (the path at batch 1, 842
-// rows in buffers for 1049: 377 -> 371 us).
+// a second width for four fifths of the tiles, used at the counts of up to that many
+// where the model has it ahead; and among choices within 8% of the best at full size the
+// one that is best over both is taken.  With / without the second width, us at fills of
+// 0.4, 0.8 and 1 of the rows a call is sized for: 640 rows QKV 26.2 / 28.4, 39 / 45, 46 / 46;
+// 1049 rows O 19.9 / 28.5, 26 / 29, 31.6 / 30.2, down 44.8 / 70, 63 / 72, 80 / 75; 1500 rows down
+// 53 / 53, 83 / 93, 97 / 97; 3000 rows O 36 / 40, 54 / 58, 62 / 62.  At every count below four fifths
+// instead, 1500 rows down took 76 at 0.4 and 3000 rows 141 for 120 at 0.6.
 GemmPlan tc_gemm_plan(int mode, long m_tiles, long n_cols, int K, bool device_rows, int num_sms) {
   const bool half_n = mode == kGemmSwiglu || mode == kGemmCount;
   // whole 32-column chunks of the output, and whole heads for Rope
@@ -691,7 +696,7 @@ GemmPlan tc_gemm_plan(int mode, long m_tiles, long n_cols, int K, bool device_ro
   const long few = device_rows && m_tiles > 2 ? (4 * m_tiles + 4) / 5 : m_tiles;
   const bool second = !half_n && mode != kGemmRope;
 
-  GemmPlan g{2, width(2, m_tiles, 0), 0, 1, 1, 0, 0};
+  GemmPlan g{2, width(2, m_tiles, 0), 0, 1, 1, 0, 0, 0};
   int one = width(1, m_tiles, 0);                      // the one-SM choice
   const double pair_full = cost(2, g.bn, m_tiles), one_full = cost(1, one, m_tiles);
   bool use_one = one_full < 0.98 * pair_full;
@@ -704,6 +709,10 @@ GemmPlan tc_gemm_plan(int mode, long m_tiles, long n_cols, int K, bool device_ro
     if (second && other > 0 && other != (use_one ? one : g.bn)) {
       g.few_bn = other;
       g.few_m = static_cast<int>((few + cg - 1) / cg);
+      const int full_bn = use_one ? one : g.bn;
+      for (int m = 1; m <= (g.few_m < 64 ? g.few_m : 64); ++m)
+        if (cost(cg, other, static_cast<long>(m) * cg) < cost(cg, full_bn, static_cast<long>(m) * cg))
+          g.few_mask |= uint64_t{1} << (m - 1);
     }
   }
   if (use_one) {

@@ -129,8 +129,8 @@ def test_linear_repeats_bit_for_bit_over_a_long_k_loop(M, N, K):
 
 
 @pytest.mark.parametrize("M_cap,N,K", [(100, 256, 64), (640, 12288, 128), (640, 4096, 192), (900, 4096, 64), (1049, 4096, 128),
-                                       (1500, 4096, 64), (1500, 12288, 64)])
-@pytest.mark.parametrize("fill", [0.0, 0.01, 0.5, 0.78, 0.8, 0.82, 1.0])
+                                       (1500, 4096, 64), (1500, 12288, 64), (1500, 4096, 1024)])
+@pytest.mark.parametrize("fill", [0.0, 0.01, 0.25, 0.4, 0.5, 0.78, 0.8, 0.82, 1.0])
 def test_linear_second_tile_choice_for_fewer_device_rows(M_cap, N, K, fill):
     """Calls whose device row count is below the size they are planned for use the
     plan's second tile width up to four fifths of the row tiles: exact on integers,
