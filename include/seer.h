@@ -292,9 +292,15 @@ seer_status seer_convert(const void* src, seer_dtype src_dt, void* dst, seer_dty
  * not overlap on the GPU).  Where a call has few units (segment, head, 256
  * query rows) and many keys, each unit's keys are shared by a cluster of CTAs
  * and the shares merged in fp32: such a call's results differ from those of a
- * call that keeps them together by fp32 rounding before the 16-bit store.  A
- * layer with the count hook always keeps them together, so its counts do not
- * depend on the batch it runs in. */
+ * call that keeps them together by fp32 rounding before the 16-bit store.
+ * Which of the two a 16-bit call does follows from n_heads, B and the
+ * capacities it is given, so the same rows may be rounded otherwise in another
+ * batch or in buffers of another capacity.  A layer with the count hook always
+ * keeps them together: for the same input rows its counts are the same in any
+ * batch and at any capacity, and its y may differ from the same call without
+ * the hook by that rounding.  Layers before a hooked one do share keys, so the
+ * counts of a stack may still differ between batches where an activation lies
+ * within a rounding of the threshold. */
 seer_status seer_attention(const void* qkv, void* o, seer_dtype dt, const int32_t* cu_seqlens,
                            const int32_t* kv_len, int B, int T_capacity, int n_heads, int head_dim,
                            void* ws, size_t ws_bytes, void* stream);

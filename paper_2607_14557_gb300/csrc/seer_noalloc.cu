@@ -17,10 +17,11 @@
 // The cached address belongs to the device's current context: resetting the
 // device (cudaDeviceReset) while libseer is loaded is not supported.
 //
-// All calls share the one array and leave their schedule in it.  Nothing in
-// it has to start at zero: the schedule kernel rewrites the entries and the
-// count it uses on every call.  Calls whose kernels overlap on the GPU (for
-// example on two streams at once) race on the array and must not be issued.
+// All calls share the one array.  Nothing in it has to start at zero: a call
+// either has the schedule kernel rewrite the entries and the count it uses, or
+// (with at most one unit per SM) makes its schedule in the attention kernel and
+// leaves the array alone.  Calls whose kernels overlap on the GPU (for example
+// on two streams at once) race on the array and must not be issued.
 #include <cuda_runtime.h>
 
 #include <cstddef>

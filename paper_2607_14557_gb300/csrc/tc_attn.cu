@@ -852,7 +852,8 @@ int tc_attn_smem_bytes() { return SMEM_BYTES; }
 
 // CTAs that share a unit's keys, from what the host knows: the most units the
 // call can have (a segment of L rows has ceil(L / 256) per head) and the average
-// number of key tiles.  Split only where units leave most SMs idle, each share keeps
+// number of key tiles (the lengths are on the device: one long segment among many
+// short ones is not split).  Split only where units leave most SMs idle, each share keeps
 // four key tiles (six of two), and the clusters fit at once (152 SMs hold 76 clusters of 2, 36
 // of 4, 15 of 8).  us, one CTA per unit -> split: the cached 8B layer of one sequence,
 // 50 rows over 3062 keys 154 -> 140 (4 CTAs), 120 over 12120 241 -> 166; 2 heads of

@@ -502,7 +502,7 @@ def test_snr_scan_golden_bit_exact():
 
 @pytest.mark.parametrize("B,N", [(256, 1024), (3, 20000)])
 def test_snr_scan_large_shapes_match_oracle_exactly(B, N):
-    # many sequences (one warp each), and a window longer than the shared-memory
+    # many sequences (one block each), and a window longer than the shared-memory
     # staging of the counts (the scan then reads them from global memory)
     rng = _rng(50 + N)
     F = 12288
