@@ -129,10 +129,13 @@ _DTYPES = {SEER_F32: SEER_F32, SEER_BF16: SEER_BF16, SEER_F16: SEER_F16, "bf16":
 
 
 def _dt(dt) -> int:
-    code = _DTYPES.get(dt)
-    if code is None:
-        raise ValueError(f"unsupported dtype {dt!r}")
-    return code
+    # only types whose equality is exact go through the table (1.0 equals its key 1)
+    code = _DTYPES.get(dt) if isinstance(dt, (int, str, torch.dtype)) else None
+    if code is not None:
+        return code
+    if dt in (SEER_F32, SEER_BF16, SEER_F16):      # other integers; the C call's arguments refuse the rest
+        return dt
+    raise ValueError(f"unsupported dtype {dt!r}")
 
 
 # The current stream's handle without building a torch.cuda.Stream around it (2.8 us

@@ -61,3 +61,16 @@ def test_poll_ctrl_times_out_on_host_flag_never_set(libseer):
     copy = (ctypes.c_int32 * S.CTRL_WORDS)()
     assert S.lib().seer_poll_ctrl(ctypes.addressof(buf), 7, 2000, ctypes.addressof(copy)) == 0
     assert copy[1] == 1234
+
+
+def test_dtype_names_codes_and_refusals(libseer):
+    import numpy as np
+    import torch
+    from paper_2607_14557_gb300 import seer as S
+    for dt in (S.SEER_BF16, "bf16", torch.bfloat16, np.int64(1)):
+        assert S._dt(dt) == S.SEER_BF16
+    for dt in ("int8", torch.int8, 7, [], None):
+        with pytest.raises(ValueError):
+            S._dt(dt)
+    with pytest.raises(ctypes.ArgumentError):          # a float is no code, also where it equals one
+        S.seer_convert(0, 1.0, 0, 2.0, 0, stream=1)
